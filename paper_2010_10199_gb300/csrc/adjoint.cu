@@ -10,11 +10,11 @@
 //      (spread_f32 sorted items, spread3_f32) -- and added to the shared grid
 //      once per cell; without records every node's window is added with
 //      shared-memory atomics.
-//   2. reduce_partials: grid = sum_z partials[z] in a fixed order.
-//   3. adjoint_post: per term, fold the halos back onto the periodic grid, FFT
-//      with sign -, multiply by the deconvolution factors and crop the block
-//      (I_N minus {0})^{|u|}.
-//   4. empty-set terms: sum_j y_j by a two-stage reduction.
+//   2. adjoint_post: per term, sum the partial grids in a fixed order
+//      (reduce_partials before it where there are many), fold the halos back
+//      onto the periodic grid, FFT with sign -, multiply by the deconvolution
+//      factors and crop the block (I_N minus {0})^{|u|}.
+//   3. empty-set terms: sum_j y_j, partial sums first, added by adjoint_post.
 #include <algorithm>
 #include <cstring>
 
@@ -28,13 +28,14 @@ __device__ __forceinline__ void red_add(float *addr, float v) {
     asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(smem_addr(addr)), "f"(v) : "memory");
 }
 
-__device__ __forceinline__ int freq_index_a(int q, int N) { return q < N / 2 ? q - N / 2 : q - N / 2 + 1; }
-
 enum { SK_STAGED = 0, SK_ORDER3 = 1, SK_MMA = 2, SK_MMA3 = 3 };
 // the order-1/2 tensor-core spread: 12 warps per CTA, 2 CTAs per SM (80
 // registers); two grid copies per SM leave each warp room for deep rings
 constexpr int SPREAD_MMA_THREADS = 384;
 constexpr int SPREAD_MMA_CTAS_PER_SM = 2;
+
+constexpr int POST_MAX_CHUNKS = 16;   // chunks per term summed inside adjoint_post_f32
+constexpr int SUM_Y_BLOCKS = 256;     // partial sums of y (at most this many per problem)
 
 constexpr int SP_CH = 512;   // nodes staged per block of a work item (order 1/2: SP_CH or SP_CH / 2)
 
@@ -1131,14 +1132,43 @@ __global__ void reduce_partials_f32(DevPlan single, BatchArgs B) {
     }
 }
 
+// the empty-set coefficients from the partial sums of y (one block)
+__device__ __forceinline__ void sum_y_finish(const DevPlan &P, const double2 *part, int nparts, float2 *fhat_base) {
+    __shared__ double sh[32];
+    if (P.n_empty == 0 || (P.skip && *P.skip)) return;
+    double sx = 0, sy = 0;
+    for (int i = threadIdx.x; i < nparts; i += blockDim.x) {
+        sx += part[i].x;
+        sy += part[i].y;
+    }
+    sx = block_sum_fixed(sx, sh);
+    sy = block_sum_fixed(sy, sh);
+    if (threadIdx.x != 0) return;
+    float2 *fhat = fhat_base + P.vec_coef_off;
+    for (int e = 0; e < P.n_empty; ++e) fhat[P.empty_off[e]] = make_float2((float)sx, (float)sy);
+}
+
+// One block per active term, and behind them one block per problem that adds
+// the empty-set coefficient's partial sums and, in block 0, returns the work
+// counters to zero.  With nparts > 0 the FP32 partial grids are summed (in
+// chunk order) while the halos are folded, which saves the reduction's launch
+// and its pass over the grid; many chunks per term read faster spread over the
+// whole chip (reduce_partials_f32, then nparts = 0).
 template <typename G>
-__global__ void adjoint_post_f32(DevPlan single, BatchArgs B, float2 *__restrict__ fhat_base) {
+__global__ void __launch_bounds__(FFT_THREADS)
+adjoint_post_f32(DevPlan single, BatchArgs B, float2 *__restrict__ fhat_base, int n_blocks, int *counter,
+                 bool fuse_reduce, const double2 *y_part, int n_ypart) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    if (blockIdx.x == 0 && threadIdx.x < 2) counter[threadIdx.x] = 0;
+    if ((int)blockIdx.x >= n_blocks) {
+        const int p = (int)blockIdx.x - n_blocks;
+        sum_y_finish(B.plans ? B.plans[p] : single, y_part + (long long)p * n_ypart, n_ypart, fhat_base);
+        return;
+    }
     const int pb = B.plans ? B.blk_prob[blockIdx.x] : 0;
     const DevPlan &P = B.plans ? B.plans[pb] : single;
     const int sblk = B.plans ? (int)blockIdx.x - B.blk0[pb] : (int)blockIdx.x;
     if (P.skip && *P.skip) return;
-    const G *__restrict__ grids = (const G *)P.grids;
     float2 *__restrict__ fhat = fhat_base + P.vec_coef_off;
     const Term T = P.terms[P.act[sblk]];
     const int n = T.n, s = T.order, N = T.N;
@@ -1146,183 +1176,80 @@ __global__ void adjoint_post_f32(DevPlan single, BatchArgs B, float2 *__restrict
     for (int j = 1; j < s; ++j) fe *= n;
     float2 *a = (float2 *)smem_raw;
     float2 *b = a + fe;
-    const G *g = grids + T.grid_off;
     // fold the stored (halo) grid onto the periodic grid
-    for (int e = threadIdx.x; e < fe; e += blockDim.x) {
-        float2 v = make_float2(0.f, 0.f);
-        if (s <= 2) {
-            int qc = e % n, qr = s == 2 ? e / n : 0;
-            int ecw = n + 2 * T.hc + 1;
-            for (int dr = -1; dr <= 1; ++dr) {
-                int er = s == 2 ? qr + T.hr + dr * n : 0;
-                if (s == 1 && dr != 0) continue;
-                if (er < 0 || er >= T.erows) continue;
-                for (int dc = -1; dc <= 1; ++dc) {
-                    int ec = qc + T.hc + dc * n;
-                    if (ec < 0 || ec >= ecw) continue;
-                    const float2 u = GridEl<G>::load(g[(long long)er * T.stride + ec]);
-                    v.x += u.x;
-                    v.y += u.y;
-                }
+    if (fuse_reduce) {
+        const float4 *g = (const float4 *)(P.partials + T.grid_off);
+        const int K = P.spread_chunks;
+        const long long pstride = P.grid_elems / 2;
+        fold_halo(T, a, b, fe, [&](int i, float2 &v0, float2 &v1) {
+            v0 = v1 = make_float2(0.f, 0.f);
+#pragma unroll 4
+            for (int c = 0; c < K; ++c) {
+                const float4 u = __ldg(g + c * pstride + i);
+                v0.x += u.x;
+                v0.y += u.y;
+                v1.x += u.z;
+                v1.y += u.w;
             }
-        } else {
-            int row = e / n, c = e % n;
-            v = GridEl<G>::load(g[(long long)row * T.stride + c]);
-        }
-        a[e] = v;
+        });
+    } else {
+        const G *g = (const G *)P.grids + T.grid_off;
+        fold_halo(T, a, b, fe, [&](int i, float2 &v0, float2 &v1) {
+            v0 = GridEl<G>::load(g[2 * i]);
+            v1 = GridEl<G>::load(g[2 * i + 1]);
+        });
     }
-    __syncthreads();
     // FFT along every axis, sign -
-    float2 *cur = a, *oth = b;
-    int inner = 1;
-    for (int ax = s - 1; ax >= 0; --ax) {
-        int rad[24];
-        int ns = fft_radices(n, rad);
-        const int nlines = fe / n;
-        float2 *src = cur, *dst = oth;
-        int which = 0, Ns = 1;
-        for (int st = 0; st < ns; ++st) {
-            const int Rr = rad[st];
-            const int nb = n / Rr;
-            for (int w = threadIdx.x; w < nlines * nb; w += blockDim.x) {
-                const int l = w / nb, j = w - l * nb;
-                const int base = (l / inner) * inner * n + (l % inner);
-                const float2 *in = src + base;
-                float2 *out = dst + base;
-                float2 v[5];
-                const int jm = j % Ns;
-                for (int r = 0; r < Rr; ++r) {
-                    float2 x = in[(j + r * nb) * inner];
-                    if (r && jm) {
-                        float sn, cs;
-                        sincospif(-(float)(2 * r * jm) / (float)(Ns * Rr), &sn, &cs);
-                        x = cmul(x, make_float2(cs, sn));
-                    }
-                    v[r] = x;
-                }
-                float2 V[5];
-                if (Rr == 2) {
-                    V[0] = make_float2(v[0].x + v[1].x, v[0].y + v[1].y);
-                    V[1] = make_float2(v[0].x - v[1].x, v[0].y - v[1].y);
-                } else if (Rr == 4) {
-                    float2 s0 = make_float2(v[0].x + v[2].x, v[0].y + v[2].y);
-                    float2 d0 = make_float2(v[0].x - v[2].x, v[0].y - v[2].y);
-                    float2 s1 = make_float2(v[1].x + v[3].x, v[1].y + v[3].y);
-                    float2 d1 = make_float2(v[1].x - v[3].x, v[1].y - v[3].y);
-                    float2 jd1 = make_float2(d1.y, -d1.x);   // -i d1
-                    V[0] = make_float2(s0.x + s1.x, s0.y + s1.y);
-                    V[2] = make_float2(s0.x - s1.x, s0.y - s1.y);
-                    V[1] = make_float2(d0.x + jd1.x, d0.y + jd1.y);
-                    V[3] = make_float2(d0.x - jd1.x, d0.y - jd1.y);
-                } else {
-                    for (int q = 0; q < Rr; ++q) {
-                        float2 acc = v[0];
-                        for (int r = 1; r < Rr; ++r) {
-                            float sn, cs;
-                            sincospif(-(float)(2 * ((r * q) % Rr)) / (float)Rr, &sn, &cs);
-                            float2 t = cmul(v[r], make_float2(cs, sn));
-                            acc.x += t.x;
-                            acc.y += t.y;
-                        }
-                        V[q] = acc;
-                    }
-                }
-                const int idxD = (j / Ns) * Ns * Rr + jm;
-                for (int r = 0; r < Rr; ++r) out[(idxD + r * Ns) * inner] = V[r];
-            }
-            __syncthreads();
-            float2 *t = src;
-            src = dst;
-            dst = t;
-            which ^= 1;
-            Ns *= Rr;
-        }
-        if (which) {
-            float2 *t = cur;
-            cur = oth;
-            oth = t;
-        }
-        inner *= n;
-    }
+    const float2 *cur = grid_fft<float2, float>(a, b, n, s, -1);
     // crop and deconvolve
-    const int Nm = N - 1;
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis == ANOVA_BASIS_COS; q += blockDim.x) {
+    const int len = (int)T.coef_len;
+    if (T.basis == ANOVA_BASIS_COS) {
         // cosine term: 2^{-s/2} times the sum over its 2^s mirrored frequencies
-        int k[3];
-        cos_decode(q, s, N, k);
-        float sx = 0.f, sy = 0.f;
-        for (int sg = 0; sg < (1 << s); ++sg) {
-            float D = (float)cos_amp(s);
-            const float2 v = cur[cos_mirror(k, s, sg, N, n, P.deconv, T.dc_off, T.dr_off, D)];
-            sx = fmaf(v.x, D, sx);
-            sy = fmaf(v.y, D, sy);
+        for (int q = threadIdx.x; q < len; q += blockDim.x) {
+            int k[3];
+            cos_decode(q, s, N, k);
+            float sx = 0.f, sy = 0.f;
+            for (int sg = 0; sg < (1 << s); ++sg) {
+                float D = (float)cos_amp(s);
+                const float2 v = cur[cos_mirror(k, s, sg, N, n, P.deconv, T.dc_off, T.dr_off, D)];
+                sx = fmaf(v.x, D, sx);
+                sy = fmaf(v.y, D, sy);
+            }
+            fhat[T.coef_off + q] = make_float2(sx, sy);
         }
-        fhat[T.coef_off + q] = make_float2(sx, sy);
+        return;
     }
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis != ANOVA_BASIS_COS; q += blockDim.x) {
-        long long rr = q;
-        int pos = 0, mul = 1;
-        float D = 1.f;
-        for (int t = s - 1; t >= 0; --t) {
-            int it = (int)(rr % Nm);
-            rr /= Nm;
-            int kk = freq_index_a(it, N);
-            pos += (kk < 0 ? kk + n : kk) * mul;
-            mul *= n;
-            D *= (t == s - 1) ? P.deconv[T.dc_off + it] : P.deconv[T.dr_off + it];
-        }
-        float2 v = cur[pos];
+    const FastDiv by_Nm(N - 1);
+    for (int q = threadIdx.x; q < len; q += blockDim.x) {
+        float D;
+        const float2 v = cur[exp_position(q, s, N, n, by_Nm, P.deconv, T.dc_off, T.dr_off, D)];
         fhat[T.coef_off + q] = make_float2(v.x * D, v.y * D);
     }
 }
 
-// two-stage sum of y for the empty-set coefficients
-__global__ void sum_y_stage1(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, double2 *part_base) {
+// partial sums of y for the empty-set coefficients, one per block (of the
+// problem blockIdx.y); adjoint_post_f32 adds them
+__global__ void sum_y_partial(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, double2 *part_base) {
+    __shared__ double sh[32];
     const DevPlan &P = B.plans ? B.plans[blockIdx.y] : single;
-    if (P.skip && *P.skip) return;
-    if (P.n_empty == 0) return;
+    if (P.n_empty == 0 || (P.skip && *P.skip)) return;
     const float2 *__restrict__ y = y_base + P.vec_node_off;
-    const long long M = P.M;
-    double2 *part = part_base + (long long)blockIdx.y * gridDim.x;
-    __shared__ double2 red[256];
     double sx = 0, sy = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < M; i += (long long)gridDim.x * blockDim.x) {
-        float2 v = y[i];
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P.M; i += (long long)gridDim.x * blockDim.x) {
+        const float2 v = y[i];
         sx += v.x;
         sy += v.y;
     }
-    red[threadIdx.x] = make_double2(sx, sy);
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            red[threadIdx.x].x += red[threadIdx.x + o].x;
-            red[threadIdx.x].y += red[threadIdx.x + o].y;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-__global__ void sum_y_stage2(DevPlan single, BatchArgs B, const double2 *part_base, int nparts, float2 *fhat_base) {
-    const DevPlan &P = B.plans ? B.plans[blockIdx.x] : single;
-    if (threadIdx.x != 0 || (P.skip && *P.skip) || P.n_empty == 0) return;
-    const double2 *part = part_base + (long long)blockIdx.x * nparts;
-    float2 *fhat = fhat_base + P.vec_coef_off;
-    const long long *eoff = P.empty_off;
-    const int n_empty = P.n_empty;
-    double sx = 0, sy = 0;
-    for (int i = 0; i < nparts; ++i) {
-        sx += part[i].x;
-        sy += part[i].y;
-    }
-    for (int e = 0; e < n_empty; ++e) fhat[eoff[e]] = make_float2((float)sx, (float)sy);
+    sx = block_sum_fixed(sx, sh);
+    sy = block_sum_fixed(sy, sh);
+    if (threadIdx.x == 0) part_base[(long long)blockIdx.y * gridDim.x + blockIdx.x] = make_double2(sx, sy);
 }
 
 template <typename G>
 static void adjoint_attrs() {
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
-        cudaFuncSetAttribute(adjoint_post_f32<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(adjoint_post_f32<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
         cudaFuncSetAttribute(spread_f32<3, G, SP_CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
         cudaFuncSetAttribute(spread_f32<4, G, SP_CH>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
         cudaFuncSetAttribute(spread_f32<3, G, SP_CH / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
@@ -1337,78 +1264,82 @@ static void adjoint_attrs() {
 }
 
 // spread + reduce + post for grids stored as G; sgrid = bytes of the largest
-// grid in FP32 (the spread's shared-memory copy)
+// grid in FP32 (the spread's shared-memory copy).  n_ypart > 0: partial sums of
+// y for the empty set wait in y_part.
 template <typename G>
 static void adjoint_kernels(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P,
                             const float2 *y, float2 *fhat, int n_items, int n_items3, int *counter, int n_blocks,
-                            int mr, long long sgrid, int max_fft_elems, int sm_count, long long max_grid_elems,
-                            bool tc) {
+                            int mr, long long sgrid, int max_fft_elems, int max_n, int max_stage, int sm_count,
+                            long long max_grid_elems, int max_chunks, const double2 *y_part, int n_ypart, bool tc) {
     adjoint_attrs<G>();
     const int sp = spread_block_nodes(sgrid);
     const size_t ssm = spread_smem_bytes(sgrid, false, sp), ssm3 = spread_smem_bytes(sgrid, true, sp);
     const int per_sm = spread_ctas_per_sm(sgrid, false);
-    if (prof) stage_begin(*prof, ST_SPREAD);
-    cudaMemsetAsync(counter, 0, 2 * sizeof(int), st);
-    if (n_items3 > 0 && tc) {
-        const size_t sm3 = spread3_mma_smem_bytes(sgrid);
-        const int per3 = (int)std::max<size_t>(1, std::min<size_t>(2, (size_t)(MAX_SMEM + 1024) / (sm3 + 1024)));
-        const int c3 = std::max(1, std::min(n_items3, per3 * sm_count));
-        auto k = mr <= 3 ? spread3_mma_f32<3, G> : spread3_mma_f32<4, G>;
-        k<<<c3, SPREAD_THREADS, sm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
-    } else if (n_items3 > 0) {
-        const int c3 = std::max(1, std::min(n_items3, std::min(per_sm, 2) * sm_count));
-        if (mr <= 3)
-            spread3_f32<3, G><<<c3, SPREAD_THREADS, ssm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
-        else
-            spread3_f32<4, G><<<c3, SPREAD_THREADS, ssm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
+    if (n_blocks > 0) {
+        if (prof) stage_begin(*prof, ST_SPREAD);
+        if (n_items3 > 0 && tc) {
+            const size_t sm3 = spread3_mma_smem_bytes(sgrid);
+            const int per3 = (int)std::max<size_t>(1, std::min<size_t>(2, (size_t)(MAX_SMEM + 1024) / (sm3 + 1024)));
+            const int c3 = std::max(1, std::min(n_items3, per3 * sm_count));
+            auto k = mr <= 3 ? spread3_mma_f32<3, G> : spread3_mma_f32<4, G>;
+            k<<<c3, SPREAD_THREADS, sm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
+        } else if (n_items3 > 0) {
+            const int c3 = std::max(1, std::min(n_items3, std::min(per_sm, 2) * sm_count));
+            if (mr <= 3)
+                spread3_f32<3, G><<<c3, SPREAD_THREADS, ssm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
+            else
+                spread3_f32<4, G><<<c3, SPREAD_THREADS, ssm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
+        }
+        if (n_items > n_items3 && tc) {
+            const size_t sm = spread_mma_smem_bytes(sgrid);
+            const int per = (int)std::max<size_t>(
+                1, std::min<size_t>(SPREAD_MMA_CTAS_PER_SM, (size_t)(MAX_SMEM + 1024) / (sm + 1024)));
+            const int c = std::max(1, std::min(n_items - n_items3, per * sm_count));
+            auto k = mr <= 3 ? spread_mma_f32<3, G> : spread_mma_f32<4, G>;
+            k<<<c, SPREAD_MMA_THREADS, sm, st>>>(v, B, y, n_items3, n_items, counter + 1, sgrid);
+        } else if (n_items > n_items3) {
+            const int c = std::max(1, std::min(n_items - n_items3, per_sm * sm_count));
+            auto k = mr <= 3 ? (sp == SP_CH ? spread_f32<3, G, SP_CH> : spread_f32<3, G, SP_CH / 2>)
+                             : (sp == SP_CH ? spread_f32<4, G, SP_CH> : spread_f32<4, G, SP_CH / 2>);
+            k<<<c, SPREAD_THREADS, ssm, st>>>(v, B, y, n_items3, n_items, counter + 1, sgrid);
+        }
+        if (prof) stage_end(*prof, ST_SPREAD);
     }
-    if (n_items > n_items3 && tc) {
-        const size_t sm = spread_mma_smem_bytes(sgrid);
-        const int per = (int)std::max<size_t>(
-            1, std::min<size_t>(SPREAD_MMA_CTAS_PER_SM, (size_t)(MAX_SMEM + 1024) / (sm + 1024)));
-        const int c = std::max(1, std::min(n_items - n_items3, per * sm_count));
-        auto k = mr <= 3 ? spread_mma_f32<3, G> : spread_mma_f32<4, G>;
-        k<<<c, SPREAD_MMA_THREADS, sm, st>>>(v, B, y, n_items3, n_items, counter + 1, sgrid);
-    } else if (n_items > n_items3) {
-        const int c = std::max(1, std::min(n_items - n_items3, per_sm * sm_count));
-        auto k = mr <= 3 ? (sp == SP_CH ? spread_f32<3, G, SP_CH> : spread_f32<3, G, SP_CH / 2>)
-                         : (sp == SP_CH ? spread_f32<4, G, SP_CH> : spread_f32<4, G, SP_CH / 2>);
-        k<<<c, SPREAD_THREADS, ssm, st>>>(v, B, y, n_items3, n_items, counter + 1, sgrid);
+    const bool fuse = std::is_same<G, float2>::value && max_chunks <= POST_MAX_CHUNKS;
+    if (n_blocks > 0 && !fuse) {
+        const long long n4 = max_grid_elems / 2;
+        const int rb =
+            (int)std::max<long long>(1, std::min<long long>(sm_count * 8LL / std::max(1, P) + 1, (n4 + 255) / 256));
+        if (prof) stage_begin(*prof, ST_REDUCE);
+        reduce_partials_f32<G><<<dim3(rb, P), 256, 0, st>>>(v, B);
+        if (prof) stage_end(*prof, ST_REDUCE);
     }
-    if (prof) stage_end(*prof, ST_SPREAD);
-    const long long n4 = max_grid_elems / 2;
-    const int rb = (int)std::max<long long>(1, std::min<long long>(sm_count * 8LL / std::max(1, P) + 1, (n4 + 255) / 256));
-    if (prof) stage_begin(*prof, ST_REDUCE);
-    reduce_partials_f32<G><<<dim3(rb, P), 256, 0, st>>>(v, B);
-    if (prof) stage_end(*prof, ST_REDUCE);
-    const size_t post_smem = (size_t)max_fft_elems * 2 * sizeof(float2);
+    const int blocks = n_blocks + (n_ypart > 0 ? P : 0);
+    if (blocks == 0) return;
     if (prof) stage_begin(*prof, ST_POST);
-    adjoint_post_f32<G><<<n_blocks, 256, post_smem, st>>>(v, B, fhat);
+    adjoint_post_f32<G><<<blocks, FFT_THREADS, fft_smem_bytes<float2>(max_fft_elems, max_n, max_stage), st>>>(
+        v, B, fhat, n_blocks, counter, fuse, y_part, n_ypart);
     if (prof) stage_end(*prof, ST_POST);
 }
 
 // The adjoint kernels for one problem (B.plans == null) or a batch of P problems.
 int adjoint_launch(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P, const float2 *y,
                    float2 *fhat, int n_items, int n_items3, int *counter, int n_blocks, int mr,
-                   long long max_grid_bytes, int max_fft_elems, int sm_count, long long max_grid_elems,
-                   bool any_empty, double2 *scratch, int prec, bool tc) {
+                   long long max_grid_bytes, int max_fft_elems, int max_n, int max_stage, int sm_count, long long max_grid_elems,
+                   int max_chunks, bool any_empty, double2 *scratch, int prec, bool tc) {
+    // enough blocks to fill the chip, shared among the problems
+    const int n_ypart = any_empty ? std::max(8, SUM_Y_BLOCKS / P) : 0;
     if (any_empty) {
-        const int nb = 256;
         if (prof) stage_begin(*prof, ST_SUMY);
-        sum_y_stage1<<<dim3(nb, P), 256, 0, st>>>(v, B, y, scratch);
-        sum_y_stage2<<<P, 32, 0, st>>>(v, B, scratch, nb, fhat);
+        sum_y_partial<<<dim3(n_ypart, P), 256, 0, st>>>(v, B, y, scratch);
         if (prof) stage_end(*prof, ST_SUMY);
     }
-    if (n_blocks == 0) return cuda_status(cudaGetLastError());
-    if (prec == ANOVA_PREC_F16)
-        adjoint_kernels<__half2>(prof, st, v, B, P, y, fhat, n_items, n_items3, counter, n_blocks, mr,
-                                 2 * max_grid_bytes, max_fft_elems, sm_count, max_grid_elems, tc);
-    else if (prec == ANOVA_PREC_BF16)
-        adjoint_kernels<__nv_bfloat162>(prof, st, v, B, P, y, fhat, n_items, n_items3, counter, n_blocks, mr,
-                                        2 * max_grid_bytes, max_fft_elems, sm_count, max_grid_elems, tc);
-    else
-        adjoint_kernels<float2>(prof, st, v, B, P, y, fhat, n_items, n_items3, counter, n_blocks, mr,
-                                max_grid_bytes, max_fft_elems, sm_count, max_grid_elems, tc);
+    auto run = prec == ANOVA_PREC_F16    ? adjoint_kernels<__half2>
+               : prec == ANOVA_PREC_BF16 ? adjoint_kernels<__nv_bfloat162>
+                                         : adjoint_kernels<float2>;
+    const long long sgrid = prec == ANOVA_PREC_F32 ? max_grid_bytes : 2 * max_grid_bytes;
+    run(prof, st, v, B, P, y, fhat, n_items, n_items3, counter, n_blocks, mr, sgrid, max_fft_elems, max_n, max_stage,
+        sm_count, max_grid_elems, max_chunks, scratch, n_ypart, tc);
     return cuda_status(cudaGetLastError());
 }
 
@@ -1424,7 +1355,7 @@ int launch_adjoint_f32(Plan &p, const float2 *y, float2 *fhat) {
     int mr = 3;
     for (int s = 0; s < p.n_terms; ++s) mr = p.h_terms[s].mr > 0 ? p.h_terms[s].mr : mr;
     return adjoint_launch(&p, p.stream, v, B, 1, y, fhat, p.n_items, p.n_items3, p.counter, p.n_act, mr,
-                          p.max_grid_bytes, p.max_fft_elems, p.sm_count, p.grid_elems, p.n_empty > 0,
+                          p.max_grid_bytes, p.max_fft_elems, p.max_n, p.max_stage, p.sm_count, p.grid_elems, p.spread_K, p.n_empty > 0,
                           (double2 *)p.scratch, p.precision, p.srec && p.cell_tc);
 }
 

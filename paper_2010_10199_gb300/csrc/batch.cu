@@ -17,13 +17,14 @@
 #include <cstring>
 #include <vector>
 
+#include "device.cuh"
 #include "solvers.cuh"
 
 namespace agft {
 
 int gather_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, const float2 *fhat, float2 *f, int n_tiles,
                   int mr, int pitch, long long max_grid_bytes, int dmax, int sm_count, int prec);
-__global__ void trafo_pre_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base);
+__global__ void trafo_pre_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base, double *part);
 
 constexpr int BRB = 32;   // partial sums per problem segment
 
@@ -39,7 +40,7 @@ struct Batch {
     int *counter = nullptr;
     BatchArgs args;
     int n_tiles = 0, n_items = 0, n_items3 = 0, n_blocks = 0, mr = 3, pitch = 0, dmax = 1, max_fft = 1,
-        sm_count = 152;
+        max_n = 1, max_stage = 0, max_chunks = 1, sm_count = 152;
     long long max_grid_bytes = 16, max_grid_elems = 0;
     bool any_empty = false;
     bool sorted_fwd = true;   // every problem has cell-sorted records for all its terms
@@ -77,26 +78,25 @@ static int upload_views(Batch &b) {
 }
 
 static int batch_trafo(Batch &b, cudaStream_t st, const float2 *fhat, float2 *f) {
-    const size_t pre_smem = (size_t)b.max_fft * 2 * sizeof(float2);
+    const size_t pre_smem = fft_smem_bytes<float2>(b.max_fft, b.max_n);
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
-        cudaFuncSetAttribute(trafo_pre_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(trafo_pre_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
     });
-    trafo_pre_f32<<<b.n_blocks, 256, pre_smem, st>>>(b.views[0], b.args, fhat);
+    trafo_pre_f32<<<b.n_blocks, FFT_THREADS, pre_smem, st>>>(b.views[0], b.args, fhat, (double *)b.scratch);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e);
     if (b.sorted_fwd)
         return gather_sorted_launch(st, b.views[0], b.args, b.P, fhat, f, b.args.items, b.n_items3, b.n_items,
-                                    b.counter, b.max_grid_bytes, b.max_M, b.sm_count, b.mr, (double *)b.scratch,
-                                    b.cell_tc);
+                                    b.counter, b.max_grid_bytes, b.max_M, b.sm_count, b.mr, b.cell_tc);
     return gather_launch(st, b.views[0], b.args, fhat, f, b.n_tiles, b.mr, b.pitch, b.max_grid_bytes, b.dmax,
                          b.sm_count, ANOVA_PREC_F32);
 }
 
 static int batch_adjoint(Batch &b, cudaStream_t st, const float2 *y, float2 *fhat) {
     return adjoint_launch(nullptr, st, b.views[0], b.args, b.P, y, fhat, b.n_items, b.n_items3, b.counter,
-                          b.n_blocks, b.mr, b.max_grid_bytes, b.max_fft, b.sm_count, b.max_grid_elems, b.any_empty,
-                          b.scratch, ANOVA_PREC_F32, b.cell_tc);
+                          b.n_blocks, b.mr, b.max_grid_bytes, b.max_fft, b.max_n, b.max_stage, b.sm_count, b.max_grid_elems,
+                          b.max_chunks, b.any_empty, b.scratch, ANOVA_PREC_F32, b.cell_tc);
 }
 
 // ----------------------------------------------------- segmented kernels --
@@ -287,6 +287,8 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
         }
         b->dmax = std::max(b->dmax, pl.d);
         b->max_fft = std::max(b->max_fft, pl.max_fft_elems);
+        b->max_n = std::max(b->max_n, pl.max_n);
+        b->max_stage = std::max(b->max_stage, pl.max_stage);
         b->max_grid_bytes = std::max(b->max_grid_bytes, pl.max_grid_bytes);
         b->max_grid_elems = std::max(b->max_grid_elems, pl.grid_elems);
         b->any_empty = b->any_empty || pl.n_empty > 0;
@@ -310,6 +312,7 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
         Ks[p] = spread_chunks_for(pl.M, total_act, pl.spread_kmax, b->max_grid_bytes, b->sm_count, b->cell_tc,
                                   order3);
         b->views[p].spread_chunks = Ks[p];
+        b->max_chunks = std::max(b->max_chunks, Ks[p]);
     }
     // third-order items of every problem first, then the others
     for (int sel : {3, 0}) {
@@ -327,7 +330,10 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
     if (e == cudaSuccess) e = cudaMalloc(&b->d_tables, sizeof(int) * nt);
     if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int4) * std::max<size_t>(1, items.size()));
     if (e == cudaSuccess) e = cudaMalloc(&b->counter, 2 * sizeof(int));
-    if (e == cudaSuccess) e = cudaMalloc(&b->scratch, sizeof(double2) * 256 * n_problems);
+    if (e == cudaSuccess) e = cudaMemsetAsync(b->counter, 0, 2 * sizeof(int), b->stream);
+    // partial sums: 256 complex ones per problem, or a double per block of the FFT passes
+    if (e == cudaSuccess)
+        e = cudaMalloc(&b->scratch, std::max(sizeof(double2) * 256 * n_problems, sizeof(double) * b->n_blocks));
     if (e != cudaSuccess) {
         free_batch(b);
         return cuda_status(e);

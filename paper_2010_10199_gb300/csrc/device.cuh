@@ -305,11 +305,20 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, int *e
 
 // ----------------------------------------------------------- shared FFT ---
 
-// Mixed-radix Stockham FFT over a batch of lines held in shared memory.
-// Line l, element i lives at base[l * lstride + i * estride] in both ping-pong
-// buffers.  Computes X[q] = sum_i x[i] exp(sign 2 pi i i q / n) (unnormalised).
-// Radices 4, 2, 3, 5.  All threads of the block must call it; returns the
-// buffer (0 = a, 1 = b) that holds the result.
+// Division of x < 2^16 by a fixed d < 2^16 with one high multiplication:
+// m = ceil(2^32 / d), and the error x (m d - 2^32) / 2^32 < x d / 2^32 < 1 / d
+// never carries the quotient over an integer.
+struct FastDiv {
+    unsigned d, m;
+    __device__ __forceinline__ explicit FastDiv(int d_) : d((unsigned)d_), m(0xffffffffu / (unsigned)d_ + 1u) {}
+    __device__ __forceinline__ int div(int x) const { return d == 1 ? x : (int)__umulhi((unsigned)x, m); }
+    __device__ __forceinline__ int div(int x, int &rem) const {
+        const int q = div(x);
+        rem = x - q * (int)d;
+        return q;
+    }
+};
+
 template <typename C, typename R>
 struct CplxOps;
 
@@ -332,165 +341,241 @@ __device__ __forceinline__ C cmul(C a, C b) {
     return r;
 }
 
-__host__ __device__ inline int fft_radices(int n, int *rad) {
-    int k = 0;
-    while (n % 4 == 0) { rad[k++] = 4; n /= 4; }
-    while (n % 2 == 0) { rad[k++] = 2; n /= 2; }
-    while (n % 3 == 0) { rad[k++] = 3; n /= 3; }
-    while (n % 5 == 0) { rad[k++] = 5; n /= 5; }
-    return n == 1 ? k : -1;
+// Discrete Fourier transform of RADIX values in registers,
+// v[q] <- sum_r v[r] exp(sign 2 pi i r q / RADIX), sign = +-1 in sg.
+template <int RADIX, typename C, typename R>
+__device__ __forceinline__ void dft_regs(C (&v)[RADIX], R sg) {
+    using O = CplxOps<C, R>;
+    auto add = [](C a, C b) { return O::mk(a.x + b.x, a.y + b.y); };
+    auto sub = [](C a, C b) { return O::mk(a.x - b.x, a.y - b.y); };
+    auto imul = [sg](C a) { return O::mk(-sg * a.y, sg * a.x); };   // sign i a
+    if constexpr (RADIX == 2) {
+        const C a = v[0];
+        v[0] = add(a, v[1]);
+        v[1] = sub(a, v[1]);
+    } else if constexpr (RADIX == 3) {
+        const R c = (R)-0.5, s = (R)0.86602540378443864676;   // cos, sin of 2 pi / 3
+        const C t = add(v[1], v[2]), d = sub(v[1], v[2]);
+        const C m = O::mk(fma(c, t.x, v[0].x), fma(c, t.y, v[0].y));
+        const C n = imul(O::mk(s * d.x, s * d.y));
+        v[0] = add(v[0], t);
+        v[1] = add(m, n);
+        v[2] = sub(m, n);
+    } else if constexpr (RADIX == 4) {
+        const C s0 = add(v[0], v[2]), d0 = sub(v[0], v[2]), s1 = add(v[1], v[3]), d1 = imul(sub(v[1], v[3]));
+        v[0] = add(s0, s1);
+        v[1] = add(d0, d1);
+        v[2] = sub(s0, s1);
+        v[3] = sub(d0, d1);
+    } else if constexpr (RADIX == 5) {
+        // cos and sin of 2 pi / 5 and 4 pi / 5
+        const R c1 = (R)0.30901699437494742410, c2 = (R)-0.80901699437494742410;
+        const R s1 = (R)0.95105651629515357212, s2 = (R)0.58778525229247312917;
+        const C t1 = add(v[1], v[4]), t2 = add(v[2], v[3]), t3 = sub(v[1], v[4]), t4 = sub(v[2], v[3]);
+        const C m1 = O::mk(fma(c1, t1.x, fma(c2, t2.x, v[0].x)), fma(c1, t1.y, fma(c2, t2.y, v[0].y)));
+        const C m2 = O::mk(fma(c2, t1.x, fma(c1, t2.x, v[0].x)), fma(c2, t1.y, fma(c1, t2.y, v[0].y)));
+        const C n1 = imul(O::mk(fma(s1, t3.x, s2 * t4.x), fma(s1, t3.y, s2 * t4.y)));
+        const C n2 = imul(O::mk(fma(s2, t3.x, -s1 * t4.x), fma(s2, t3.y, -s1 * t4.y)));
+        v[0] = add(v[0], add(t1, t2));
+        v[1] = add(m1, n1);
+        v[2] = add(m2, n2);
+        v[3] = sub(m2, n2);
+        v[4] = sub(m1, n1);
+    } else {
+        static_assert(RADIX == 8, "radices 2, 3, 4, 5, 8");
+        const R h = (R)0.70710678118654752440;   // exp(sign i pi / 4) = h (1 + sign i)
+        C e[4] = {v[0], v[2], v[4], v[6]}, o[4] = {v[1], v[3], v[5], v[7]};
+        dft_regs<4, C, R>(e, sg);
+        dft_regs<4, C, R>(o, sg);
+        const C o1 = imul(o[1]), o3 = imul(o[3]);
+        const C w1 = O::mk(h * (o[1].x + o1.x), h * (o[1].y + o1.y));
+        const C w2 = imul(o[2]);
+        const C w3 = O::mk(h * (o3.x - o[3].x), h * (o3.y - o[3].y));
+        v[0] = add(e[0], o[0]);
+        v[4] = sub(e[0], o[0]);
+        v[1] = add(e[1], w1);
+        v[5] = sub(e[1], w1);
+        v[2] = add(e[2], w2);
+        v[6] = sub(e[2], w2);
+        v[3] = add(e[3], w3);
+        v[7] = sub(e[3], w3);
+    }
 }
 
-template <typename C, typename R>
-__device__ int smem_fft(C *a, C *b, int n, int nlines, int lstride, int estride, int sign) {
-    using O = CplxOps<C, R>;
-    int rad[24];
-    int ns = fft_radices(n, rad);
-    C *src = a, *dst = b;
-    int which = 0;
-    int Ns = 1;
-    for (int s = 0; s < ns; ++s) {
-        const int Rr = rad[s];
-        const int nb = n / Rr;
-        for (int w = threadIdx.x; w < nlines * nb; w += blockDim.x) {
-            const int l = w / nb, j = w - l * nb;
-            const C *in = src + (size_t)l * lstride;
-            C *out = dst + (size_t)l * lstride;
-            C v[5];
-            const int jm = j % Ns;
-            // twiddles exp(sign 2 pi i r jm / (Ns Rr))
-            for (int r = 0; r < Rr; ++r) {
-                C x = in[(size_t)(j + r * nb) * estride];
-                if (r && jm) {
-                    R sn, cs;
-                    O::sincospi_((R)(2 * sign * r * jm) / (R)(Ns * Rr), &sn, &cs);
-                    x = cmul(x, O::mk(cs, sn));
+// Entries of the twiddle table exp(sign 2 pi i k / n), k < n, kept in shared
+// memory behind the two FFT arrays; longer axes evaluate each factor.
+template <typename C>
+__host__ __device__ constexpr int fft_table_max() {
+    return 16384 / (int)sizeof(C);
+}
+// shared memory of a block that transforms arrays of at most fft_elems values
+// with axes of at most max_n; the adjoint also stages a stored grid of at most
+// stage_elems values behind the first array
+template <typename C>
+inline size_t fft_smem_bytes(int fft_elems, int max_n, int stage_elems = 0) {
+    const int tw = max_n < fft_table_max<C>() ? max_n : fft_table_max<C>();
+    return ((size_t)fft_elems + (fft_elems + tw > stage_elems ? fft_elems + tw : stage_elems)) * sizeof(C);
+}
+constexpr int FFT_THREADS = 512;
+constexpr int FFT_MAX_SMEM = 220 * 1024;   // two 100 KB arrays, the table, and room for static shared memory
+
+// One Stockham stage over every line of one axis: element i of the line at
+// base = (outer, inner position) lies at base + i * inner.  Consecutive
+// threads take neighbouring lines of a strided axis (contiguous addresses) and
+// neighbouring elements of the last axis.
+template <int RADIX, typename C, typename R>
+__device__ __forceinline__ void fft_stage(const C *src, C *dst, int fe, int n, int inner, int Ns, R sg, const C *tw) {
+    const int nb = n / RADIX, step = nb / Ns;
+    const FastDiv by_inner(inner), by_nb(nb), by_Ns(Ns);
+    for (int w = threadIdx.x; w < fe / RADIX; w += blockDim.x) {
+        int li, j, jm;
+        const int rest = by_inner.div(w, li);
+        const int lo = by_nb.div(rest, j);
+        by_Ns.div(j, jm);
+        const int base = lo * inner * n + li;
+        const C *in = src + base + j * inner;
+        C v[RADIX];
+#pragma unroll
+        for (int r = 0; r < RADIX; ++r) v[r] = in[r * nb * inner];
+        if (jm) {
+            const int k = jm * step;   // r k < n
+#pragma unroll
+            for (int r = 1; r < RADIX; ++r) {
+                C t;
+                if (tw) {
+                    t = tw[r * k];
+                } else {
+                    CplxOps<C, R>::sincospi_(sg * (R)(2 * r * k) / (R)n, &t.y, &t.x);
                 }
-                v[r] = x;
+                v[r] = cmul(v[r], t);
             }
-            C V[5];
-            if (Rr == 2) {
-                V[0] = O::mk(v[0].x + v[1].x, v[0].y + v[1].y);
-                V[1] = O::mk(v[0].x - v[1].x, v[0].y - v[1].y);
-            } else if (Rr == 4) {
-                C s0 = O::mk(v[0].x + v[2].x, v[0].y + v[2].y);
-                C d0 = O::mk(v[0].x - v[2].x, v[0].y - v[2].y);
-                C s1 = O::mk(v[1].x + v[3].x, v[1].y + v[3].y);
-                C d1 = O::mk(v[1].x - v[3].x, v[1].y - v[3].y);
-                // multiply d1 by (sign) i
-                C jd1 = sign > 0 ? O::mk(-d1.y, d1.x) : O::mk(d1.y, -d1.x);
-                V[0] = O::mk(s0.x + s1.x, s0.y + s1.y);
-                V[2] = O::mk(s0.x - s1.x, s0.y - s1.y);
-                V[1] = O::mk(d0.x + jd1.x, d0.y + jd1.y);
-                V[3] = O::mk(d0.x - jd1.x, d0.y - jd1.y);
-            } else {
-                for (int q = 0; q < Rr; ++q) {
-                    C acc = v[0];
-                    for (int r = 1; r < Rr; ++r) {
-                        R sn, cs;
-                        O::sincospi_((R)(2 * sign * ((r * q) % Rr)) / (R)Rr, &sn, &cs);
-                        C t = cmul(v[r], O::mk(cs, sn));
-                        acc.x += t.x;
-                        acc.y += t.y;
-                    }
-                    V[q] = acc;
-                }
-            }
-            const int idxD = (j / Ns) * Ns * Rr + jm;
-            for (int r = 0; r < Rr; ++r) out[(size_t)(idxD + r * Ns) * estride] = V[r];
         }
-        __syncthreads();
-        C *t = src;
-        src = dst;
-        dst = t;
-        which ^= 1;
-        Ns *= Rr;
+        dft_regs<RADIX, C, R>(v, sg);
+        C *out = dst + base + ((j - jm) * RADIX + jm) * inner;
+#pragma unroll
+        for (int r = 0; r < RADIX; ++r) out[r * Ns * inner] = v[r];
     }
-    return which;
 }
 
 // Unnormalised FFT with sign `sign` along every axis of an n^s array held in
-// shared memory (a; b is scratch of the same size), s = 1..3: all lines of an
-// axis at once, line bases (l / inner) * inner * n + l % inner for the axis
-// whose element stride is `inner`.  All threads of the block call it; returns
-// the buffer that holds the result.
+// shared memory (a; b is scratch of the same size, followed by the twiddle
+// table), s = 1..3, radices 8, 4, 2, 3, 5.  All threads of the block call it
+// after filling a (it synchronises first); returns the buffer that holds the
+// result.  What bounds it is the latency of a block's few stages: the former
+// stages, with per-butterfly sincospi, run-time radix loops over arrays in
+// local memory and hardware divisions, took 52 us for the 211 terms of the
+// d = 20 workload (n = 64) and 147 us for 120 three-dimensional terms (n = 20).
 template <typename C, typename R>
 __device__ C *grid_fft(C *a, C *b, int n, int s, int sign) {
-    using O = CplxOps<C, R>;
     int fe = n;
     for (int j = 1; j < s; ++j) fe *= n;
-    C *cur = a, *oth = b;
+    C *tw = nullptr;
+    if (n <= fft_table_max<C>()) {
+        tw = b + fe;
+        for (int k = threadIdx.x; k < n; k += blockDim.x)
+            CplxOps<C, R>::sincospi_((R)(2 * sign * k) / (R)n, &tw[k].y, &tw[k].x);
+    }
+    __syncthreads();
+    const R sg = (R)sign;
+    C *src = a, *dst = b;
     int inner = 1;
-    int rad[24];
-    const int ns = fft_radices(n, rad);
-    for (int ax = s - 1; ax >= 0; --ax) {
-        const int nlines = fe / n;
-        C *src = cur, *dst = oth;
-        int which = 0, Ns = 1;
-        for (int st = 0; st < ns; ++st) {
-            const int Rr = rad[st];
-            const int nb = n / Rr;
-            for (int w = threadIdx.x; w < nlines * nb; w += blockDim.x) {
-                const int l = w / nb, j = w - l * nb;
-                const int base = (l / inner) * inner * n + (l % inner);
-                const C *in = src + base;
-                C *out = dst + base;
-                C v[5];
-                const int jm = j % Ns;
-                for (int r = 0; r < Rr; ++r) {
-                    C x = in[(j + r * nb) * inner];
-                    if (r && jm) {
-                        R sn, cs;
-                        O::sincospi_((R)(2 * sign * r * jm) / (R)(Ns * Rr), &sn, &cs);
-                        x = cmul(x, O::mk(cs, sn));
-                    }
-                    v[r] = x;
-                }
-                C V[5];
-                if (Rr == 2) {
-                    V[0] = O::mk(v[0].x + v[1].x, v[0].y + v[1].y);
-                    V[1] = O::mk(v[0].x - v[1].x, v[0].y - v[1].y);
-                } else if (Rr == 4) {
-                    const C s0 = O::mk(v[0].x + v[2].x, v[0].y + v[2].y);
-                    const C d0 = O::mk(v[0].x - v[2].x, v[0].y - v[2].y);
-                    const C s1 = O::mk(v[1].x + v[3].x, v[1].y + v[3].y);
-                    const C d1 = O::mk(v[1].x - v[3].x, v[1].y - v[3].y);
-                    const C jd1 = sign > 0 ? O::mk(-d1.y, d1.x) : O::mk(d1.y, -d1.x);   // sign i d1
-                    V[0] = O::mk(s0.x + s1.x, s0.y + s1.y);
-                    V[2] = O::mk(s0.x - s1.x, s0.y - s1.y);
-                    V[1] = O::mk(d0.x + jd1.x, d0.y + jd1.y);
-                    V[3] = O::mk(d0.x - jd1.x, d0.y - jd1.y);
-                } else {
-                    for (int q = 0; q < Rr; ++q) {
-                        C acc = v[0];
-                        for (int r = 1; r < Rr; ++r) {
-                            R sn, cs;
-                            O::sincospi_((R)(2 * sign * ((r * q) % Rr)) / (R)Rr, &sn, &cs);
-                            const C t = cmul(v[r], O::mk(cs, sn));
-                            acc.x += t.x;
-                            acc.y += t.y;
-                        }
-                        V[q] = acc;
-                    }
-                }
-                const int idxD = (j / Ns) * Ns * Rr + jm;
-                for (int r = 0; r < Rr; ++r) out[(idxD + r * Ns) * inner] = V[r];
+    for (int ax = 0; ax < s; ++ax) {
+        int left = n, Ns = 1;
+        while (left > 1) {
+            const int radix = left % 8 == 0 ? 8 : left % 4 == 0 ? 4 : left % 2 == 0 ? 2 : left % 3 == 0 ? 3 : 5;
+            switch (radix) {
+                case 8: fft_stage<8, C, R>(src, dst, fe, n, inner, Ns, sg, tw); break;
+                case 4: fft_stage<4, C, R>(src, dst, fe, n, inner, Ns, sg, tw); break;
+                case 2: fft_stage<2, C, R>(src, dst, fe, n, inner, Ns, sg, tw); break;
+                case 3: fft_stage<3, C, R>(src, dst, fe, n, inner, Ns, sg, tw); break;
+                default: fft_stage<5, C, R>(src, dst, fe, n, inner, Ns, sg, tw); break;
             }
             __syncthreads();
             C *t = src;
             src = dst;
             dst = t;
-            which ^= 1;
-            Ns *= Rr;
-        }
-        if (which) {
-            C *t = cur;
-            cur = oth;
-            oth = t;
+            Ns *= radix;
+            left /= radix;
         }
         inner *= n;
     }
-    return cur;
+    return src;
+}
+
+// Block-wide FP64 sum in a fixed order, valid in thread 0 (sh: 32 doubles;
+// blockDim a multiple of 32).
+__device__ __forceinline__ double block_sum_fixed(double v, double *sh) {
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (threadIdx.x < 32) {
+        s = threadIdx.x < (blockDim.x >> 5) ? sh[threadIdx.x] : 0.0;
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    }
+    return s;
+}
+
+// Position of coefficient q of an exponential block on the term's FFT array
+// (k mod n per axis, last axis fastest) and the product of its deconvolution
+// factors (column table on the last axis, row table on the others).
+template <typename R>
+__device__ __forceinline__ int exp_position(int q, int s, int N, int n, const FastDiv &by_Nm, const R *deconv,
+                                            int dc_off, int dr_off, R &D) {
+    int pos = 0, mul = 1;
+    D = (R)1;
+    for (int t = s - 1; t >= 0; --t) {
+        int it;
+        q = by_Nm.div(q, it);
+        const int k = it < N / 2 ? it - N / 2 : it - N / 2 + 1;
+        pos += (k < 0 ? k + n : k) * mul;
+        mul *= n;
+        D *= deconv[(t == s - 1 ? dc_off : dr_off) + it];
+    }
+    return pos;
+}
+
+// Periodic grid of a term into a (n^s values) from its stored grid with halos:
+// entries of the stored grid that repeat a periodic one are added.  `load2`
+// returns the stored values 2 i, 2 i + 1 (rows are even in length); they pass
+// through `stage` (halo_stage_elems), so that global memory is read once, 16
+// bytes or more at a time.  All threads of the block call it.
+__host__ __device__ inline int halo_cols(const Term &T) { return (T.n + 2 * T.hc + 2) & ~1; }   // even row length
+__host__ __device__ inline int halo_stage_elems(const Term &T) { return T.order > 2 ? 0 : T.erows * halo_cols(T); }
+
+template <typename C, typename Load2>
+__device__ __forceinline__ void fold_halo(const Term &T, C *a, C *stage, int fe, Load2 load2) {
+    const int n = T.n, cols = T.order > 2 ? n : halo_cols(T), rows = T.erows, half = cols >> 1;
+    C *dst = T.order > 2 ? a : stage;
+    {
+        const FastDiv by_half(half);
+        for (int i = threadIdx.x; i < rows * half; i += blockDim.x) {
+            int c2;
+            const int r = by_half.div(i, c2);
+            C v0, v1;
+            load2((r * T.stride >> 1) + c2, v0, v1);
+            dst[r * cols + 2 * c2] = v0;
+            dst[r * cols + 2 * c2 + 1] = v1;
+        }
+    }
+    if (T.order > 2) return;
+    __syncthreads();
+    const int ecw = n + 2 * T.hc + 1;
+    const FastDiv by_n(n);
+    for (int e = threadIdx.x; e < fe; e += blockDim.x) {
+        int qc;
+        const int qr = by_n.div(e, qc);
+        C v;
+        v.x = v.y = 0;
+        for (int er = T.order == 2 ? (qr + T.hr >= n ? qr + T.hr - n : qr + T.hr) : 0; er < rows; er += n)
+            for (int ec = qc + T.hc >= n ? qc + T.hc - n : qc + T.hc; ec < ecw; ec += n) {
+                const C u = stage[er * cols + ec];
+                v.x += u.x;
+                v.y += u.y;
+            }
+        a[e] = v;
+    }
 }
 
 }  // namespace agft

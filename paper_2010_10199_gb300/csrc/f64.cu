@@ -22,8 +22,6 @@
 
 namespace agft {
 
-__device__ __forceinline__ int freq_index64(int q, int N) { return q < N / 2 ? q - N / 2 : q - N / 2 + 1; }
-
 // ------------------------------------------------------ window tables ----
 
 __global__ void k_wtab_f64(const double *__restrict__ x, long long M, const int4 *slots, const Window *wins,
@@ -69,7 +67,7 @@ __device__ __forceinline__ void load_w8(const double *wt, int slot, long long M,
 // ------------------------------------------------------------ forward ----
 
 // per active term: zero-extended, deconvolved block, FFT (sign +), grid with halos
-__global__ void trafo_pre_f64(DevPlan P, const double2 *__restrict__ fhat) {
+__global__ void __launch_bounds__(FFT_THREADS) trafo_pre_f64(DevPlan P, const double2 *__restrict__ fhat) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     if (P.skip && *P.skip) return;
     const Term T = P.terms[P.act[blockIdx.x]];
@@ -80,39 +78,34 @@ __global__ void trafo_pre_f64(DevPlan P, const double2 *__restrict__ fhat) {
     double2 *b = a + fe;
     for (int i = threadIdx.x; i < fe; i += blockDim.x) a[i] = make_double2(0.0, 0.0);
     __syncthreads();
-    const int Nm = N - 1;
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis == ANOVA_BASIS_COS; q += blockDim.x) {
-        int k[3];
-        cos_decode(q, s, N, k);
-        const double2 c = fhat[T.coef_off + q];
-        for (int sg = 0; sg < (1 << s); ++sg) {
-            double D = cos_amp(s);
-            const int pos = cos_mirror(k, s, sg, N, n, P.deconvd, T.dc_off, T.dr_off, D);
+    const int len = (int)T.coef_len;
+    if (T.basis == ANOVA_BASIS_COS) {
+        for (int q = threadIdx.x; q < len; q += blockDim.x) {
+            int k[3];
+            cos_decode(q, s, N, k);
+            const double2 c = fhat[T.coef_off + q];
+            for (int sg = 0; sg < (1 << s); ++sg) {
+                double D = cos_amp(s);
+                const int pos = cos_mirror(k, s, sg, N, n, P.deconvd, T.dc_off, T.dr_off, D);
+                a[pos] = make_double2(c.x * D, c.y * D);
+            }
+        }
+    } else {
+        const FastDiv by_Nm(N - 1);
+        for (int q = threadIdx.x; q < len; q += blockDim.x) {
+            double D;
+            const int pos = exp_position(q, s, N, n, by_Nm, P.deconvd, T.dc_off, T.dr_off, D);
+            const double2 c = fhat[T.coef_off + q];
             a[pos] = make_double2(c.x * D, c.y * D);
         }
     }
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis != ANOVA_BASIS_COS; q += blockDim.x) {
-        long long r = q;
-        int pos = 0, mul = 1;
-        double D = 1.0;
-        for (int t = s - 1; t >= 0; --t) {
-            const int it = (int)(r % Nm);
-            r /= Nm;
-            const int k = freq_index64(it, N);
-            pos += (k < 0 ? k + n : k) * mul;
-            mul *= n;
-            D *= (t == s - 1) ? P.deconvd[T.dc_off + it] : P.deconvd[T.dr_off + it];
-        }
-        const double2 c = fhat[T.coef_off + q];
-        a[pos] = make_double2(c.x * D, c.y * D);
-    }
-    __syncthreads();
     const double2 *cur = grid_fft<double2, double>(a, b, n, s, +1);
     double2 *g = (double2 *)P.grids + T.grid_off;
-    const int ecols = T.stride;
-    const long long total = (long long)T.erows * ecols;
-    for (long long e = threadIdx.x; e < total; e += blockDim.x) {
-        const int er = (int)(e / ecols), ec = (int)(e % ecols);
+    const FastDiv by_cols(T.stride);
+    const int total = T.erows * T.stride;
+    for (int e = threadIdx.x; e < total; e += blockDim.x) {
+        int ec;
+        const int er = by_cols.div(e, ec);
         double2 v = make_double2(0.0, 0.0);
         if (s <= 2) {
             if (ec < n + 2 * T.hc + 1) {
@@ -224,11 +217,11 @@ int launch_trafo_f64(Plan &p, const double2 *fhat, double2 *f) {
     }
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
-        cudaFuncSetAttribute(trafo_pre_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(trafo_pre_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
     });
-    const size_t pre_smem = (size_t)p.max_fft_elems * 2 * sizeof(double2);
+    const size_t pre_smem = fft_smem_bytes<double2>(p.max_fft_elems, p.max_n);
     stage_begin(p, ST_PRE);
-    trafo_pre_f64<<<p.n_act, 256, pre_smem, p.stream>>>(v, fhat);
+    trafo_pre_f64<<<p.n_act, FFT_THREADS, pre_smem, p.stream>>>(v, fhat);
     stage_end(p, ST_PRE);
     stage_begin(p, ST_GATHER);
     gather_f64<<<(int)((p.M + 255) / 256), 256, 0, p.stream>>>(v, fhat, f, p.wt64, p.wb64);
@@ -429,10 +422,26 @@ __global__ void reduce_partials_f64(DevPlan P) {
     }
 }
 
-// per active term: fold the halos, FFT (sign -), deconvolve and crop
-__global__ void adjoint_post_f64(DevPlan P, double2 *__restrict__ fhat) {
+// per active term: fold the halos, FFT (sign -), deconvolve and crop; the block
+// behind the terms' adds the empty-set coefficient's partial sums of y
+__global__ void __launch_bounds__(FFT_THREADS) adjoint_post_f64(DevPlan P, double2 *__restrict__ fhat,
+                                                                const double2 *y_part, int n_ypart, int *counter) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ double sh[32];
+    if (blockIdx.x == 0 && threadIdx.x == 0) *counter = 0;
     if (P.skip && *P.skip) return;
+    if ((int)blockIdx.x >= P.n_act) {
+        double sx = 0.0, sy = 0.0;
+        for (int i = threadIdx.x; i < n_ypart; i += blockDim.x) {
+            sx += y_part[i].x;
+            sy += y_part[i].y;
+        }
+        sx = block_sum_fixed(sx, sh);
+        sy = block_sum_fixed(sy, sh);
+        if (threadIdx.x == 0)
+            for (int e = 0; e < P.n_empty; ++e) fhat[P.empty_off[e]] = make_double2(sx, sy);
+        return;
+    }
     const Term T = P.terms[P.act[blockIdx.x]];
     const int n = T.n, s = T.order, N = T.N;
     int fe = n;
@@ -440,63 +449,38 @@ __global__ void adjoint_post_f64(DevPlan P, double2 *__restrict__ fhat) {
     double2 *a = (double2 *)smem_raw;
     double2 *b = a + fe;
     const double2 *g = (const double2 *)P.grids + T.grid_off;
-    for (int e = threadIdx.x; e < fe; e += blockDim.x) {
-        double2 v = make_double2(0.0, 0.0);
-        if (s <= 2) {
-            const int qc = e % n, qr = s == 2 ? e / n : 0;
-            const int ecw = n + 2 * T.hc + 1;
-            for (int dr = -1; dr <= 1; ++dr) {
-                if (s == 1 && dr != 0) continue;
-                const int er = s == 2 ? qr + T.hr + dr * n : 0;
-                if (er < 0 || er >= T.erows) continue;
-                for (int dc = -1; dc <= 1; ++dc) {
-                    const int ec = qc + T.hc + dc * n;
-                    if (ec < 0 || ec >= ecw) continue;
-                    const double2 u = g[(long long)er * T.stride + ec];
-                    v.x += u.x;
-                    v.y += u.y;
-                }
-            }
-        } else {
-            v = g[(long long)(e / n) * T.stride + e % n];
-        }
-        a[e] = v;
-    }
-    __syncthreads();
+    fold_halo(T, a, b, fe, [&](int i, double2 &v0, double2 &v1) {
+        v0 = g[2 * i];
+        v1 = g[2 * i + 1];
+    });
     const double2 *cur = grid_fft<double2, double>(a, b, n, s, -1);
-    const int Nm = N - 1;
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis == ANOVA_BASIS_COS; q += blockDim.x) {
-        int k[3];
-        cos_decode(q, s, N, k);
-        double sx = 0.0, sy = 0.0;
-        for (int sg = 0; sg < (1 << s); ++sg) {
-            double D = cos_amp(s);
-            const double2 v = cur[cos_mirror(k, s, sg, N, n, P.deconvd, T.dc_off, T.dr_off, D)];
-            sx = fma(v.x, D, sx);
-            sy = fma(v.y, D, sy);
+    const int len = (int)T.coef_len;
+    if (T.basis == ANOVA_BASIS_COS) {
+        for (int q = threadIdx.x; q < len; q += blockDim.x) {
+            int k[3];
+            cos_decode(q, s, N, k);
+            double sx = 0.0, sy = 0.0;
+            for (int sg = 0; sg < (1 << s); ++sg) {
+                double D = cos_amp(s);
+                const double2 v = cur[cos_mirror(k, s, sg, N, n, P.deconvd, T.dc_off, T.dr_off, D)];
+                sx = fma(v.x, D, sx);
+                sy = fma(v.y, D, sy);
+            }
+            fhat[T.coef_off + q] = make_double2(sx, sy);
         }
-        fhat[T.coef_off + q] = make_double2(sx, sy);
+        return;
     }
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis != ANOVA_BASIS_COS; q += blockDim.x) {
-        long long rr = q;
-        int pos = 0, mul = 1;
-        double D = 1.0;
-        for (int t = s - 1; t >= 0; --t) {
-            const int it = (int)(rr % Nm);
-            rr /= Nm;
-            const int kk = freq_index64(it, N);
-            pos += (kk < 0 ? kk + n : kk) * mul;
-            mul *= n;
-            D *= (t == s - 1) ? P.deconvd[T.dc_off + it] : P.deconvd[T.dr_off + it];
-        }
-        const double2 v = cur[pos];
+    const FastDiv by_Nm(N - 1);
+    for (int q = threadIdx.x; q < len; q += blockDim.x) {
+        double D;
+        const double2 v = cur[exp_position(q, s, N, n, by_Nm, P.deconvd, T.dc_off, T.dr_off, D)];
         fhat[T.coef_off + q] = make_double2(v.x * D, v.y * D);
     }
 }
 
-// sum of y for the empty-set coefficients: partial sums, then one thread
-__global__ void sum_y_f64_stage1(DevPlan P, const double2 *__restrict__ y, double2 *part) {
-    __shared__ double2 red[256];
+// partial sums of y for the empty-set coefficients
+__global__ void sum_y_f64_partial(DevPlan P, const double2 *__restrict__ y, double2 *part) {
+    __shared__ double sh[32];
     if (P.skip && *P.skip) return;
     double sx = 0.0, sy = 0.0;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P.M; i += (long long)gridDim.x * blockDim.x) {
@@ -504,26 +488,9 @@ __global__ void sum_y_f64_stage1(DevPlan P, const double2 *__restrict__ y, doubl
         sx += v.x;
         sy += v.y;
     }
-    red[threadIdx.x] = make_double2(sx, sy);
-    __syncthreads();
-    for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-        if (threadIdx.x < o) {
-            red[threadIdx.x].x += red[threadIdx.x + o].x;
-            red[threadIdx.x].y += red[threadIdx.x + o].y;
-        }
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) part[blockIdx.x] = red[0];
-}
-
-__global__ void sum_y_f64_stage2(DevPlan P, const double2 *part, int nparts, double2 *fhat) {
-    if (threadIdx.x != 0 || (P.skip && *P.skip)) return;
-    double sx = 0.0, sy = 0.0;
-    for (int i = 0; i < nparts; ++i) {
-        sx += part[i].x;
-        sy += part[i].y;
-    }
-    for (int e = 0; e < P.n_empty; ++e) fhat[P.empty_off[e]] = make_double2(sx, sy);
+    sx = block_sum_fixed(sx, sh);
+    sy = block_sum_fixed(sy, sh);
+    if (threadIdx.x == 0) part[blockIdx.x] = make_double2(sx, sy);
 }
 
 int launch_adjoint_f64(Plan &p, const double2 *y, double2 *fhat) {
@@ -536,30 +503,37 @@ int launch_adjoint_f64(Plan &p, const double2 *y, double2 *fhat) {
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
         cudaFuncSetAttribute(spread_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
-        cudaFuncSetAttribute(adjoint_post_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024);
+        cudaFuncSetAttribute(adjoint_post_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
     });
-    if (p.n_empty > 0) {
-        const int nb = 256;
+    const int n_ypart = p.n_empty > 0 ? 256 : 0;
+    if (n_ypart > 0) {
         stage_begin(p, ST_SUMY);
-        sum_y_f64_stage1<<<nb, 256, 0, st>>>(v, y, (double2 *)p.scratch);
-        sum_y_f64_stage2<<<1, 32, 0, st>>>(v, (const double2 *)p.scratch, nb, fhat);
+        sum_y_f64_partial<<<n_ypart, 256, 0, st>>>(v, y, (double2 *)p.scratch);
         stage_end(p, ST_SUMY);
     }
-    if (p.n_act == 0) return cuda_status(cudaGetLastError());
+    const size_t post_smem = fft_smem_bytes<double2>(p.max_fft_elems, p.max_n, p.max_stage);
+    auto post = [&](int blocks) {
+        if (blocks == 0) return;
+        stage_begin(p, ST_POST);
+        adjoint_post_f64<<<blocks, FFT_THREADS, post_smem, st>>>(v, fhat, (const double2 *)p.scratch, n_ypart,
+                                                                 p.counter);
+        stage_end(p, ST_POST);
+    };
+    if (p.n_act == 0) {
+        post(n_ypart > 0 ? 1 : 0);
+        return cuda_status(cudaGetLastError());
+    }
     const size_t ssm = (size_t)p.max_grid_bytes + 16;
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(4, (size_t)(MAX_SMEM + 1024) / (ssm + 1024)));
     const int ctas = std::max(1, std::min(p.n_items, per_sm * p.sm_count));
     stage_begin(p, ST_SPREAD);
-    cudaMemsetAsync(p.counter, 0, sizeof(int), st);
     spread_f64<<<ctas, 256, ssm, st>>>(v, p.items, y, p.n_items, p.counter, p.max_grid_bytes, p.wt64, p.wb64);
     stage_end(p, ST_SPREAD);
     stage_begin(p, ST_REDUCE);
     const int rb = (int)std::max<long long>(1, std::min<long long>(p.sm_count * 8LL, (p.grid_elems + 255) / 256));
     reduce_partials_f64<<<rb, 256, 0, st>>>(v);
     stage_end(p, ST_REDUCE);
-    stage_begin(p, ST_POST);
-    adjoint_post_f64<<<p.n_act, 256, (size_t)p.max_fft_elems * 2 * sizeof(double2), st>>>(v, fhat);
-    stage_end(p, ST_POST);
+    post(p.n_act + (n_ypart > 0 ? 1 : 0));
     return cuda_status(cudaGetLastError());
 }
 

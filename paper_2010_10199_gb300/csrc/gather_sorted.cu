@@ -15,8 +15,8 @@
 // fixed point, v * 2^e with 2^e chosen from ||fhat||_1 (a bound on every
 // partial sum), so the additions are exact and their order, which the
 // hardware does not fix, cannot change the result: the forward is bitwise
-// reproducible.  A last pass adds acc * 2^-e to f, which already holds the
-// empty set's coefficient and the third-order terms.
+// reproducible.  A last pass writes f, the empty set's coefficient plus
+// acc * 2^-e, and zeroes the accumulators for the next call.
 #include <algorithm>
 #include <cstring>
 
@@ -31,57 +31,16 @@ __device__ __forceinline__ void red_add_u64(unsigned long long *addr, long long 
     asm volatile("red.global.add.u64 [%0], %1;" ::"l"(addr), "l"(v) : "memory");
 }
 
-// fixed-point exponent e for the accumulators: 2^e * 2 sum |fhat| <= 2^62
-// (every partial sum of a node's terms is bounded by sum_k |fhat_k| up to the
-// window error), clamped so that 2^e stays a normal float.  Two passes with
-// a fixed block count, so the sum (and e) never depends on timing.
-constexpr int FPE_BLOCKS = 128;
-
 __device__ __forceinline__ const DevPlan &plan_of(const DevPlan &single, const BatchArgs &B, int prob) {
     return B.plans ? B.plans[prob] : single;
 }
 
-// per problem (blockIdx.y): partial sums of |Re| + |Im| of its coefficients
-__global__ void k_fixed_point_partial(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base,
-                                      double *part_base) {
-    __shared__ double sh[32];
+// per problem (blockIdx.y): f[j] = empty-set coefficient + acc[j] * 2^-e; leaves
+// the accumulators and the launch's item counter at zero for the next call
+__global__ void k_fixed_point_finish(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base,
+                                     float2 *f_base, int *counter) {
     const DevPlan &P = plan_of(single, B, blockIdx.y);
-    if (P.skip && *P.skip) return;
-    const float2 *fhat = fhat_base + P.vec_coef_off;
-    const long long n = P.n_coeffs;
-    double a = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const float2 v = fhat[i];
-        a += fabs((double)v.x) + fabs((double)v.y);
-    }
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += sh[w];
-        part_base[(long long)blockIdx.y * FPE_BLOCKS + blockIdx.x] = s;
-    }
-}
-
-// per problem (blockIdx.x): the exponent from its partial sums
-__global__ void k_fixed_point_exponent(DevPlan single, BatchArgs B, const double *part_base) {
-    const DevPlan &P = plan_of(single, B, blockIdx.x);
-    if (threadIdx.x != 0 || (P.skip && *P.skip)) return;
-    const double *part = part_base + (long long)blockIdx.x * FPE_BLOCKS;
-    double s = 0.0;
-    for (int b = 0; b < FPE_BLOCKS; ++b) s += part[b];
-    int e = 100;
-    // a cosine coefficient stands for 2^s exponential ones of 2^{-s/2} its size
-    // (s <= 3): their absolute sum is at most 2^{3/2} = 2.83 times larger
-    if (s > 0) e = 61 - (int)ceil(log2(s)) - (P.basis == ANOVA_BASIS_COS ? 2 : 0);
-    *P.fexp = max(-100, min(100, e));
-}
-
-// per problem (blockIdx.y): f = empty-set coefficient, accumulators = 0
-__global__ void k_sorted_forward_init(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base,
-                                      float2 *f_base) {
-    const DevPlan &P = plan_of(single, B, blockIdx.y);
+    if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x < 2) counter[threadIdx.x] = 0;
     if (P.skip && *P.skip) return;
     const float2 *fhat = fhat_base + P.vec_coef_off;
     float2 c0 = make_float2(0.f, 0.f);
@@ -90,26 +49,13 @@ __global__ void k_sorted_forward_init(DevPlan single, BatchArgs B, const float2 
         c0.x += c.x;
         c0.y += c.y;
     }
-    float2 *f = f_base + P.vec_node_off;
-    for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < P.M; j += (long long)gridDim.x * blockDim.x) {
-        f[j] = c0;
-        P.facc[2 * j] = 0ULL;
-        P.facc[2 * j + 1] = 0ULL;
-    }
-}
-
-// per problem (blockIdx.y): f[j] += acc[j] * 2^-e
-__global__ void k_fixed_point_finish(DevPlan single, BatchArgs B, float2 *f_base) {
-    const DevPlan &P = plan_of(single, B, blockIdx.y);
-    if (P.skip && *P.skip) return;
     const double sc = ldexp(1.0, -*P.fexp);
     float2 *f = f_base + P.vec_node_off;
-    const long long *acc = (const long long *)P.facc;
+    longlong2 *acc = (longlong2 *)P.facc;
     for (long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x; j < P.M; j += (long long)gridDim.x * blockDim.x) {
-        float2 v = f[j];
-        v.x += (float)((double)acc[2 * j] * sc);
-        v.y += (float)((double)acc[2 * j + 1] * sc);
-        f[j] = v;
+        const longlong2 a = acc[j];
+        acc[j] = make_longlong2(0, 0);
+        f[j] = make_float2(c0.x + (float)((double)a.x * sc), c0.y + (float)((double)a.y * sc));
     }
 }
 
@@ -529,7 +475,7 @@ gather_mma_f32(DevPlan single, BatchArgs B, const int4 *__restrict__ items, int 
 
 int gather_sorted_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P, const float2 *fhat,
                          float2 *f, const int4 *items, int n_items3, int item_end, int *counter,
-                         long long max_grid_bytes, long long max_M, int sm_count, int mr, double *part, bool tc) {
+                         long long max_grid_bytes, long long max_M, int sm_count, int mr, bool tc) {
     const int item_begin = 0;
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
@@ -543,17 +489,15 @@ int gather_sorted_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, 
     // a row idle the GPU at the seam, which costs more than the tensor cores
     // gain (10 % on the d = 10, |u| <= 3 workload).
     const int cuda_end = tc && n_items3 == 0 ? 0 : item_end;
-    const int nb = (int)std::max<long long>(1, std::min<long long>(4LL * sm_count / std::max(1, P) + 1,
-                                                                   (max_M + 255) / 256));
-    k_fixed_point_partial<<<dim3(FPE_BLOCKS, P), 256, 0, st>>>(v, B, fhat, part);
-    k_fixed_point_exponent<<<P, 32, 0, st>>>(v, B, part);
-    k_sorted_forward_init<<<dim3(nb, P), 256, 0, st>>>(v, B, fhat, f);
+    // two nodes per thread of the largest problem: with a batch's uneven problems
+    // sharing few blocks, the largest one's serial loop took 176 us of 32 problems'
+    // pass (four million accumulators), blocks without work cost less
+    const int nb = (int)std::max<long long>(1, (max_M + 511) / 512);
     const size_t smem = (size_t)max_grid_bytes + 32 * sizeof(float4) + 16;
     const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(3, (size_t)(MAX_SMEM + 1024) / (smem + 1024)));
     const size_t smem_mma = (size_t)max_grid_bytes + (GS_THREADS / 32) * GmRing::BYTES + 16;
     const int per_sm_mma = (int)std::max<size_t>(
         1, std::min<size_t>(GM_CTAS_PER_SM, (size_t)(MAX_SMEM + 1024) / (smem_mma + 1024)));
-    if (item_end > item_begin) cudaMemsetAsync(counter, 0, 2 * sizeof(int), st);
     if (cuda_end > item_begin) {
         const int ctas = std::max(1, std::min(cuda_end - item_begin, per_sm * sm_count));
         if (mr <= 3)
@@ -572,7 +516,7 @@ int gather_sorted_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, 
             gather_mma_f32<4><<<ctas, GS_THREADS, smem_mma, st>>>(v, B, items, cuda_end, item_end, counter + 1,
                                                                   max_grid_bytes);
     }
-    k_fixed_point_finish<<<dim3(nb, P), 256, 0, st>>>(v, B, f);
+    k_fixed_point_finish<<<dim3(nb, P), 256, 0, st>>>(v, B, fhat, f, counter);
     return cuda_status(cudaGetLastError());
 }
 
@@ -586,7 +530,7 @@ int launch_gather_sorted_f32(Plan &p, const float2 *fhat, float2 *f) {
     for (int s = 0; s < p.n_terms; ++s)
         if (p.h_terms[s].mr > 0) mr = p.h_terms[s].mr;
     return gather_sorted_launch(p.stream, v, B, 1, fhat, f, p.items, p.n_items3, p.n_items, p.counter,
-                                p.max_grid_bytes, p.M, p.sm_count, mr, (double *)p.scratch, p.cell_tc);
+                                p.max_grid_bytes, p.M, p.sm_count, mr, p.cell_tc);
 }
 
 }  // namespace agft

@@ -134,8 +134,8 @@ struct DevPlan {
     float2 *partials;         // adjoint partial grids [spread_chunks][grid_elems]
     int spread_chunks;        // node chunks of the adjoint (one partial grid each)
     const float4 *srec;       // [slot][M] nodes sorted by grid cell, see SortedNode
-    unsigned long long *facc; // sorted forward: fixed-point accumulators [M][2] (or null)
-    int *fexp;                // and their exponent
+    unsigned long long *facc; // sorted forward: fixed-point accumulators [M][2] (or null), zero between calls
+    int *fexp;                // their exponent, and a block counter (zero between launches)
     long long n_coeffs;
     long long vec_node_off;   // offset of this problem's nodes in batched node vectors
     long long vec_coef_off;   // offset of this problem's coefficients in batched coefficient vectors
@@ -188,6 +188,8 @@ struct Plan {
     long long grid_elems;
     long long max_grid_bytes;
     int max_fft_elems;      // largest n^order
+    int max_n;              // largest n
+    int max_stage;          // largest staged halo grid of the adjoint's fold (elements)
     int pitch2;             // row pitch shared by all order-2 grids
     // active term list (all scheduled terms unless a group mask restricts it)
     int *act;
@@ -204,7 +206,7 @@ struct Plan {
     int4 *h_items;
     int n_items;
     int n_items3;           // the first n_items3 items are those of third-order terms
-    int *counter;           // work-queue counter of the spread
+    int *counter;           // work-queue counters (2), zero between calls
     float4 *srec;           // cell-sorted node records (null: none), n_sorted slots of M
     bool cell_tc;           // order-1/2 spread of sorted records on the tensor cores
     int n_sorted;
@@ -273,12 +275,12 @@ int launch_gather_sorted_f32(Plan &p, const float2 *fhat, float2 *f);
 // with tc and none of those, the gather runs on the tensor cores.
 int gather_sorted_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P, const float2 *fhat,
                          float2 *f, const int4 *items, int n_items3, int item_end, int *counter,
-                         long long max_grid_bytes, long long max_M, int sm_count, int mr, double *part, bool tc);
+                         long long max_grid_bytes, long long max_M, int sm_count, int mr, bool tc);
 int launch_adjoint_f32(Plan &p, const float2 *y, float2 *fhat);
 int adjoint_launch(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P, const float2 *y,
                    float2 *fhat, int n_items, int n_items3, int *counter, int n_blocks, int mr,
-                   long long max_grid_bytes, int max_fft_elems, int sm_count, long long max_grid_elems,
-                   bool any_empty, double2 *scratch, int prec, bool tc);
+                   long long max_grid_bytes, int max_fft_elems, int max_n, int max_stage, int sm_count,
+                   long long max_grid_elems, int max_chunks, bool any_empty, double2 *scratch, int prec, bool tc);
 size_t spread_smem_bytes(long long max_grid_bytes, bool o3, int sp);
 int spread_block_nodes(long long max_grid_bytes);
 // Sorts the nodes by grid cell for every term with sort_slot >= 0 (sort.cu).

@@ -142,7 +142,7 @@ extern "C" int grouped_trafo_noalloc(int d, int64_t M, const float *x_dev, int n
         return n_win++;
     };
     long long goff = 0, maxbytes = 16;
-    int max_fft = 1, n_dec = 0;
+    int max_fft = 1, max_n = 1, n_dec = 0;
     static Term s_sched_terms[NOALLOC_MAX_TERMS];
     for (int s = 0; s < n_sched; ++s) {
         const int i = s_sched[s];
@@ -181,6 +181,7 @@ extern "C" int grouped_trafo_noalloc(int d, int64_t M, const float *x_dev, int n
         for (int j = 0; j < T.order; ++j) fe *= T.n;
         if (fe * 16 > 200 * 1024 || T.grid_bytes > 100 * 1024) return ANOVA_ERR_UNSUPPORTED;
         max_fft = (int)std::max<long long>(max_fft, fe);
+        max_n = std::max(max_n, T.n);
         T.coef_off = s_uoff[i];
         T.coef_len = s_ulen[i];
         T.user_index = i;
@@ -266,6 +267,7 @@ extern "C" int grouped_trafo_noalloc(int d, int64_t M, const float *x_dev, int n
     p.grid_elems = goff;
     p.max_grid_bytes = maxbytes;
     p.max_fft_elems = max_fft;
+    p.max_n = max_n;
     p.pitch2 = pitch2;
     p.err = (int *)(base + o_err);
     p.act = (int *)(base + o_act);

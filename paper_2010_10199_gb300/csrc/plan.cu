@@ -470,6 +470,8 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
         // shared-memory limits of the FFT passes (two copies) and of the spread (one grid)
         if (fe * (f64 ? 32 : 16) > 200 * 1024 || T.grid_bytes > (f64 ? 200 : 100) * 1024) status = ANOVA_ERR_UNSUPPORTED;
         max_fft = (int)std::max<long long>(max_fft, fe);
+        p.max_n = std::max(p.max_n, T.n);
+        p.max_stage = std::max(p.max_stage, halo_stage_elems(T));
         T.coef_off = p.h_user_off[i];
         T.coef_len = p.h_user_len[i];
         T.user_index = i;
@@ -525,9 +527,6 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
         }
         p.n_slots64 = (int)slots64.size();
     }
-    for (int i = 0; i < n_terms; ++i) {
-        (void)i;
-    }
 
     // device allocations
     cudaError_t e = cudaSuccess;
@@ -564,7 +563,8 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
     chk(plan_malloc(&p.counter, 2 * sizeof(int)));
     p.h_items = plan_new<int4>((size_t)std::max(1, p.n_terms) * kmax);
     if (!p.h_items && e == cudaSuccess) e = cudaErrorMemoryAllocation;
-    p.scratch_bytes = 1 << 20;
+    // partial sums: one double per term, or 256 complex ones
+    p.scratch_bytes = std::max<size_t>(1 << 20, sizeof(double) * p.n_terms);
     chk(plan_malloc(&p.scratch, p.scratch_bytes));
     if (p.n_slots64 > 0 && M > 0) {
         chk(plan_malloc(&p.slots64, sizeof(int4) * p.n_slots64));
@@ -600,7 +600,9 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
                         plan_malloc(&p.fexp, sizeof(int) * 4) != cudaSuccess) {
                         cudaGetLastError();   // the forward falls back to the point-major gather
                         if (p.facc) cudaFree(p.facc);
+                        if (p.fexp) cudaFree(p.fexp);
                         p.facc = nullptr;
+                        p.fexp = nullptr;
                     }
                 }
             } else {
@@ -626,6 +628,11 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
         chk(cudaMemcpyAsync(p.empty_off, empties.data(), sizeof(long long) * empties.size(),
                             cudaMemcpyHostToDevice, p.stream));
     chk(cudaMemsetAsync(p.err, 0, sizeof(int) * 4, p.stream));
+    chk(cudaMemsetAsync(p.counter, 0, 2 * sizeof(int), p.stream));
+    if (p.facc) {
+        chk(cudaMemsetAsync(p.facc, 0, sizeof(unsigned long long) * 2 * (size_t)M, p.stream));
+        chk(cudaMemsetAsync(p.fexp, 0, sizeof(int) * 4, p.stream));
+    }
     if (xbytes) {
         long long total = (long long)d * M;
         int blocks = (int)std::min<long long>(4096, (total + 255) / 256);

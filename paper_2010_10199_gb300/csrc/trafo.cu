@@ -19,18 +19,24 @@
 
 namespace agft {
 
-__device__ __forceinline__ int freq_index(int q, int N) { return q < N / 2 ? q - N / 2 : q - N / 2 + 1; }
-
 // ------------------------------------------------------------ pre-pass ----
 
-// grids stored as G (FP32 complex, or a pair of 16-bit floats rounded from the FP32 FFT)
+// One block per active term.  grids stored as G (FP32 complex, or a pair of
+// 16-bit floats rounded from the FP32 FFT).  With fixed-point accumulators
+// (P.fexp) the block also sums |Re| + |Im| of its block of fhat into
+// part[blockIdx.x], and the last block of a problem to finish turns the sums
+// (added in a fixed order) into the accumulators' exponent, which saves two
+// launches on the smallest problems' critical path.
 template <typename G>
 __device__ __forceinline__ void trafo_pre_body(const DevPlan &single, const BatchArgs &B,
-                                               const float2 *__restrict__ fhat_base) {
+                                               const float2 *__restrict__ fhat_base, double *part) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
+    __shared__ double sh[32];
+    __shared__ int s_last;
     const int pb = B.plans ? B.blk_prob[blockIdx.x] : 0;
     const DevPlan &P = B.plans ? B.plans[pb] : single;
-    const int sblk = B.plans ? (int)blockIdx.x - B.blk0[pb] : (int)blockIdx.x;
+    const int blk0 = B.plans ? B.blk0[pb] : 0;
+    const int sblk = (int)blockIdx.x - blk0;
     if (P.skip && *P.skip) return;
     const float2 *fhat = fhat_base + P.vec_coef_off;
     G *grids = (G *)P.grids;
@@ -43,128 +49,45 @@ __device__ __forceinline__ void trafo_pre_body(const DevPlan &single, const Batc
     for (int i = threadIdx.x; i < fe; i += blockDim.x) a[i] = make_float2(0.f, 0.f);
     __syncthreads();
     // zero-extended, deconvolved coefficients at k mod n
-    const int Nm = N - 1;
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis == ANOVA_BASIS_COS; q += blockDim.x) {
+    double l1 = 0.0;
+    const int len = (int)T.coef_len;
+    if (T.basis == ANOVA_BASIS_COS) {
         // cosine term: the coefficient at its 2^s mirrored frequencies
-        int k[3];
-        cos_decode(q, s, N, k);
-        const float2 c = fhat[T.coef_off + q];
-        for (int sg = 0; sg < (1 << s); ++sg) {
-            float D = (float)cos_amp(s);
-            const int pos = cos_mirror(k, s, sg, N, n, P.deconv, T.dc_off, T.dr_off, D);
+        for (int q = threadIdx.x; q < len; q += blockDim.x) {
+            int k[3];
+            cos_decode(q, s, N, k);
+            const float2 c = fhat[T.coef_off + q];
+            l1 += fabs((double)c.x) + fabs((double)c.y);
+            for (int sg = 0; sg < (1 << s); ++sg) {
+                float D = (float)cos_amp(s);
+                const int pos = cos_mirror(k, s, sg, N, n, P.deconv, T.dc_off, T.dr_off, D);
+                a[pos] = make_float2(c.x * D, c.y * D);
+            }
+        }
+    } else {
+        const FastDiv by_Nm(N - 1);
+        for (int q = threadIdx.x; q < len; q += blockDim.x) {
+            float D;
+            const int pos = exp_position(q, s, N, n, by_Nm, P.deconv, T.dc_off, T.dr_off, D);
+            const float2 c = fhat[T.coef_off + q];
+            l1 += fabs((double)c.x) + fabs((double)c.y);
             a[pos] = make_float2(c.x * D, c.y * D);
         }
     }
-    for (long long q = threadIdx.x; q < T.coef_len && T.basis != ANOVA_BASIS_COS; q += blockDim.x) {
-        long long r = q;
-        int pos = 0, mul = 1;
-        float D = 1.f;
-        for (int t = s - 1; t >= 0; --t) {
-            int it = (int)(r % Nm);
-            r /= Nm;
-            int k = freq_index(it, N);
-            int km = k < 0 ? k + n : k;
-            pos += km * mul;
-            mul *= n;
-            D *= (t == s - 1) ? P.deconv[T.dc_off + it] : P.deconv[T.dr_off + it];
-        }
-        float2 c = fhat[T.coef_off + q];
-        a[pos] = make_float2(c.x * D, c.y * D);
-    }
-    __syncthreads();
     // FFT along every axis (sign +): g_q = sum_k ghat_k exp(+2 pi i k q / n)
-    float2 *cur = a, *oth = b;
-    int inner = 1;
-    for (int ax = s - 1; ax >= 0; --ax) {
-        // lines along axis ax: element stride `inner`
-        int rad[24];
-        int ns = fft_radices(n, rad);
-        (void)ns;
-        // smem_fft with generic line bases: handle by looping over outer blocks
-        const int nlines = fe / n;
-        // express lines as (outer, inner) pairs: base = outer * inner * n + in
-        int which;
-        {
-            // Stockham over all lines at once
-            using C = float2;
-            C *src = cur, *dst = oth;
-            which = 0;
-            int Ns = 1;
-            for (int st = 0; st < ns; ++st) {
-                const int Rr = rad[st];
-                const int nb = n / Rr;
-                for (int w = threadIdx.x; w < nlines * nb; w += blockDim.x) {
-                    const int l = w / nb, j = w - l * nb;
-                    const int base = (l / inner) * inner * n + (l % inner);
-                    const C *in = src + base;
-                    C *out = dst + base;
-                    C v[5];
-                    const int jm = j % Ns;
-                    for (int r = 0; r < Rr; ++r) {
-                        C x = in[(j + r * nb) * inner];
-                        if (r && jm) {
-                            float sn, cs;
-                            sincospif((float)(2 * r * jm) / (float)(Ns * Rr), &sn, &cs);
-                            x = cmul(x, make_float2(cs, sn));
-                        }
-                        v[r] = x;
-                    }
-                    C V[5];
-                    if (Rr == 2) {
-                        V[0] = make_float2(v[0].x + v[1].x, v[0].y + v[1].y);
-                        V[1] = make_float2(v[0].x - v[1].x, v[0].y - v[1].y);
-                    } else if (Rr == 4) {
-                        C s0 = make_float2(v[0].x + v[2].x, v[0].y + v[2].y);
-                        C d0 = make_float2(v[0].x - v[2].x, v[0].y - v[2].y);
-                        C s1 = make_float2(v[1].x + v[3].x, v[1].y + v[3].y);
-                        C d1 = make_float2(v[1].x - v[3].x, v[1].y - v[3].y);
-                        C jd1 = make_float2(-d1.y, d1.x);   // +i d1
-                        V[0] = make_float2(s0.x + s1.x, s0.y + s1.y);
-                        V[2] = make_float2(s0.x - s1.x, s0.y - s1.y);
-                        V[1] = make_float2(d0.x + jd1.x, d0.y + jd1.y);
-                        V[3] = make_float2(d0.x - jd1.x, d0.y - jd1.y);
-                    } else {
-                        for (int q = 0; q < Rr; ++q) {
-                            C acc = v[0];
-                            for (int r = 1; r < Rr; ++r) {
-                                float sn, cs;
-                                sincospif((float)(2 * ((r * q) % Rr)) / (float)Rr, &sn, &cs);
-                                C t = cmul(v[r], make_float2(cs, sn));
-                                acc.x += t.x;
-                                acc.y += t.y;
-                            }
-                            V[q] = acc;
-                        }
-                    }
-                    const int idxD = (j / Ns) * Ns * Rr + jm;
-                    for (int r = 0; r < Rr; ++r) out[(idxD + r * Ns) * inner] = V[r];
-                }
-                __syncthreads();
-                C *t = src;
-                src = dst;
-                dst = t;
-                which ^= 1;
-                Ns *= Rr;
-            }
-        }
-        if (which) {
-            float2 *t = cur;
-            cur = oth;
-            oth = t;
-        }
-        inner *= n;
-    }
+    const float2 *cur = grid_fft<float2, float>(a, b, n, s, +1);
     // store with halos
     G *g = grids + T.grid_off;
-    const int ecols = T.stride;
-    const long long total = (long long)T.erows * ecols;
-    for (long long e = threadIdx.x; e < total; e += blockDim.x) {
-        int er = (int)(e / ecols), ec = (int)(e % ecols);
+    const FastDiv by_cols(T.stride);
+    const int total = T.erows * T.stride;
+    for (int e = threadIdx.x; e < total; e += blockDim.x) {
+        int ec;
+        const int er = by_cols.div(e, ec);
         float2 v = make_float2(0.f, 0.f);
         if (s <= 2) {
             if (ec < n + 2 * T.hc + 1) {
-                int qc = wrap(ec - T.hc, n);
-                int qr = s == 2 ? wrap(er - T.hr, n) : 0;
+                const int qc = wrap(ec - T.hc, n);
+                const int qr = s == 2 ? wrap(er - T.hr, n) : 0;
                 v = cur[qr * n + qc];
             }
         } else {
@@ -172,16 +95,49 @@ __device__ __forceinline__ void trafo_pre_body(const DevPlan &single, const Batc
         }
         g[e] = GridEl<G>::store(v.x, v.y);
     }
+    if (!P.fexp) return;
+    // fixed-point exponent e for the accumulators: 2^e * 2 sum |fhat| <= 2^62
+    // (every partial sum of a node's terms is bounded by sum_k |fhat_k| of the
+    // active blocks up to the window error), clamped so that 2^e stays a normal
+    // float.  The sums are added in a fixed order, so e never depends on timing.
+    if (sblk == 0 && threadIdx.x == 0)
+        for (int i = 0; i < P.n_empty; ++i) {
+            const float2 c = fhat[P.empty_off[i]];
+            l1 += fabs((double)c.x) + fabs((double)c.y);
+        }
+    l1 = block_sum_fixed(l1, sh);
+    if (threadIdx.x == 0) {
+        part[blockIdx.x] = l1;
+        __threadfence();
+        s_last = atomicAdd(P.fexp + 1, 1) == P.n_act - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    double sum = 0.0;
+    for (int i = threadIdx.x; i < P.n_act; i += blockDim.x) sum += __ldcg(part + blk0 + i);
+    sum = block_sum_fixed(sum, sh);
+    if (threadIdx.x == 0) {
+        int e = 100;
+        // a cosine coefficient stands for 2^s exponential ones of 2^{-s/2} its size
+        // (s <= 3): their absolute sum is at most 2^{3/2} = 2.83 times larger
+        if (sum > 0) e = 61 - (int)ceil(log2(sum)) - (P.basis == ANOVA_BASIS_COS ? 2 : 0);
+        P.fexp[0] = max(-100, min(100, e));
+        P.fexp[1] = 0;
+    }
 }
 
-__global__ void trafo_pre_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base) {
-    trafo_pre_body<float2>(single, B, fhat_base);
+__global__ void __launch_bounds__(FFT_THREADS)
+trafo_pre_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base, double *part) {
+    trafo_pre_body<float2>(single, B, fhat_base, part);
 }
-__global__ void trafo_pre_f16(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base) {
-    trafo_pre_body<__half2>(single, B, fhat_base);
+__global__ void __launch_bounds__(FFT_THREADS)
+trafo_pre_f16(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base, double *part) {
+    trafo_pre_body<__half2>(single, B, fhat_base, part);
 }
-__global__ void trafo_pre_bf16(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base) {
-    trafo_pre_body<__nv_bfloat162>(single, B, fhat_base);
+__global__ void __launch_bounds__(FFT_THREADS)
+trafo_pre_bf16(DevPlan single, BatchArgs B, const float2 *__restrict__ fhat_base, double *part) {
+    trafo_pre_body<__nv_bfloat162>(single, B, fhat_base, part);
 }
 
 // ------------------------------------------------------- empty plan case --
@@ -206,18 +162,18 @@ int launch_trafo_f32(Plan &p, const float2 *fhat, float2 *f) {
         fill_const_f32<<<blocks, 256, 0, p.stream>>>(f, p.M, fhat, p.empty_off, p.n_empty, p.skip);
         return cuda_status(cudaGetLastError());
     }
-    size_t pre_smem = (size_t)p.max_fft_elems * 2 * sizeof(float2);
+    const size_t pre_smem = fft_smem_bytes<float2>(p.max_fft_elems, p.max_n);
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
-        cudaFuncSetAttribute(trafo_pre_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(trafo_pre_f16, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        cudaFuncSetAttribute(trafo_pre_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(trafo_pre_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
+        cudaFuncSetAttribute(trafo_pre_f16, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
+        cudaFuncSetAttribute(trafo_pre_bf16, cudaFuncAttributeMaxDynamicSharedMemorySize, FFT_MAX_SMEM);
     });
     stage_begin(p, ST_PRE);
     BatchArgs B;
     std::memset(&B, 0, sizeof(B));
     auto pre = p.precision == ANOVA_PREC_F16 ? trafo_pre_f16 : p.precision == ANOVA_PREC_BF16 ? trafo_pre_bf16 : trafo_pre_f32;
-    pre<<<p.n_act, 256, pre_smem, p.stream>>>(v, B, fhat);
+    pre<<<p.n_act, FFT_THREADS, pre_smem, p.stream>>>(v, B, fhat, (double *)p.scratch);
     stage_end(p, ST_PRE);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return cuda_status(e);

@@ -6,8 +6,8 @@
 //      term's stored grid (halos included), then writes it to partial grid z
 //      of the term (z = chunk index).  With cell-sorted node records the sums
 //      of one grid cell's nodes are formed first -- on the tensor cores
-//      (spread_mma_f32, spread3_mma_f32) or in registers on the CUDA cores
-//      (spread_f32 sorted items, spread3_f32) -- and added to the shared grid
+//      (spread_tiles.cu) or in registers on the CUDA cores (spread_f32 sorted
+//      items, spread3_f32) -- and added to the shared grid
 //      once per cell; without records every node's window is added with
 //      shared-memory atomics.
 //   2. adjoint_post: per term, sum the partial grids in a fixed order
@@ -16,6 +16,7 @@
 //      factors and crop the block (I_N minus {0})^{|u|}.
 //   3. empty-set terms: sum_j y_j, partial sums first, added by adjoint_post.
 #include <algorithm>
+#include <cmath>
 #include <cstring>
 
 #include "device.cuh"
@@ -28,14 +29,8 @@ __device__ __forceinline__ void red_add(float *addr, float v) {
     asm volatile("red.shared.add.f32 [%0], %1;" ::"r"(smem_addr(addr)), "f"(v) : "memory");
 }
 
-enum { SK_STAGED = 0, SK_ORDER3 = 1, SK_MMA = 2, SK_MMA3 = 3 };
-// the order-1/2 tensor-core spread: 12 warps per CTA, 2 CTAs per SM (80
-// registers); two grid copies per SM leave each warp room for deep rings
-constexpr int SPREAD_MMA_THREADS = 384;
-constexpr int SPREAD_MMA_CTAS_PER_SM = 2;
-
 constexpr int POST_MAX_CHUNKS = 16;   // chunks per term summed inside adjoint_post_f32
-constexpr int SUM_Y_BLOCKS = 256;     // partial sums of y (at most this many per problem)
+constexpr int SUM_Y_BLOCKS = 608;     // partial sums of y (at most this many per problem)
 
 constexpr int SP_CH = 512;   // nodes staged per block of a work item (order 1/2: SP_CH or SP_CH / 2)
 
@@ -83,28 +78,59 @@ int spread_block_nodes(long long max_grid_bytes) {
     return smem_bound && ctas_for(max_grid_bytes, SP_CH / 2) > ctas_for(max_grid_bytes, SP_CH) ? SP_CH / 2 : SP_CH;
 }
 
-// the tensor-core kernel: grid, one ring per warp, item slot
-static size_t spread_mma_smem_bytes(long long max_grid_bytes);
+int spread_ctas_per_sm(long long max_grid_bytes) { return ctas_for(max_grid_bytes, spread_block_nodes(max_grid_bytes)); }
 
-int spread_ctas_per_sm(long long max_grid_bytes, bool tc) {
-    if (tc) {
-        const size_t per = spread_mma_smem_bytes(max_grid_bytes) + 1024;
-        return (int)std::max<size_t>(1, std::min<size_t>(SPREAD_MMA_CTAS_PER_SM, (size_t)(MAX_SMEM + 1024) / per));
+// Nanoseconds a CTA takes per node of an order-1/2 and of a third-order term, and
+// per work item (grid copies, first cells): measured at d = 20, M = 1e6 and d = 10,
+// M = 5e5.  Only their ratios matter here.
+constexpr double NS_NODE = 3.0, NS_NODE3 = 16.0, NS_ITEM = 4000.0;
+
+// Time of n3 items of d3 followed by n items of d <= d3 on R CTAs that take the next
+// item when they are free.
+static double queue_time(long long n3, double d3, long long n, double d, long long R) {
+    const long long base = n3 / R, rem = n3 % R;
+    const double early = base * d3, late = (base + (rem > 0)) * d3;
+    if (n == 0) return late;
+    for (long long k = n / R;; ++k) {   // an early CTA takes k more items
+        const double t = early + k * d;
+        const long long l = t > early + d3 ? (long long)((t - early - d3) / d + 1e-9) : 0;
+        if ((R - rem) * k + rem * l >= n) return std::max(late, t);
     }
-    return ctas_for(max_grid_bytes, spread_block_nodes(max_grid_bytes));
 }
 
-int spread_chunks_for(long long M, int n_act_total, int kmax, long long max_grid_bytes, int sm_count, bool tc,
-                      bool order3) {
-    // third-order items cost several times an order-1/2 item per node: with
-    // them, finer chunks (three per CTA of 3 per SM, the forward gather's
-    // count) keep the last wave of both kernels short
-    const int per_sm = spread_ctas_per_sm(max_grid_bytes, tc);
-    const long long resident = (long long)(order3 ? std::max(3, per_sm) : per_sm) * sm_count;
-    long long K = (3 * resident + std::max(1, n_act_total) - 1) / std::max(1, n_act_total);
-    K = std::min<long long>(K, (M + 2047) / 2048);
-    K = std::min<long long>(K, kmax);
-    return (int)std::max<long long>(1, K);
+int spread_chunks_for(long long M, int n_terms, int n_terms3, int kmax, long long max_grid_bytes,
+                      long long grid_elems, int sm_count, bool tc) {
+    // the chunk count whose items fill the CTAs of the spread and of the gather
+    // best: at d = 20, M = 1e6 the former rule's 5 chunks per term (three items per
+    // CTA) left the gather's third round of 456 CTAs a third full, 1.76 ms
+    const bool order3 = n_terms3 > 0;
+    const long long Rs = (long long)sm_count * (tc ? spread_tiles_ctas_per_sm(max_grid_bytes, order3)
+                                                   : spread_ctas_per_sm(max_grid_bytes));
+    const long long Rg = (long long)sm_count * (tc ? gather_tiles_ctas_per_sm(max_grid_bytes, order3) : 3);
+    const int n = n_terms - n_terms3;
+    int best = 1;
+    double cost = 0.0;
+    for (int K = 1; K <= kmax; ++K) {
+        const double d3 = NS_NODE3 * M / K + NS_ITEM, d = NS_NODE * M / K + NS_ITEM;
+        const double c = queue_time((long long)n_terms3 * K, d3, (long long)n * K, d, Rs) +
+                         queue_time((long long)n_terms3 * K, d3, (long long)n * K, d, Rg) +
+                         K * grid_elems * 8 / 2500.0;   // partial grids written and read at 5 bytes per ps
+        if (K == 1 || c < 0.995 * cost) {
+            best = K;
+            cost = c;
+        }
+    }
+    return best;
+}
+
+// chunks of problem p of a batch: items of about equal cost, ten per CTA
+int batch_chunks_for(long long M, double total_ns, int kmax, long long ctas) {
+    const double item = std::max(total_ns / (10.0 * ctas), NS_ITEM);
+    return (int)std::max<long long>(1, std::min<long long>(kmax, (long long)std::ceil(NS_NODE * M / item)));
+}
+
+double batch_cost_ns(long long M, int n_terms, int n_terms3) {
+    return M * (NS_NODE * (n_terms - n_terms3) + NS_NODE3 * n_terms3);
 }
 
 int append_spread_items(const Plan &p, int prob, int K, int4 *out, int sel) {
@@ -529,481 +555,21 @@ __device__ __forceinline__ void spread_unsorted_item(const DevPlan &P, const Ter
     cp_async_wait0();
 }
 
-// ---- Tensor-core cell sums (order 1/2 terms with cell-sorted records) ----
-//
-// For the nodes j of one cell the contributions to its window block are
-//     G[r][k] += sum_j y_j psi_row,r(j) psi_col,k(j)   (r < 2 m_row, k < 8).
-// Every tap weight is a degree-7 polynomial in the node's cell offset v, kept
-// in the Chebyshev basis X_i (Window::ch): psi_k = sum_i C[k][i] X_i.  So
-//     G = C_col Mo C_row^T,   Mo[(re/im, i)][l] = sum_j y_j X_i(v_col,j) X_l(v_row,j),
-// and the nodes of a cell only build the 16 x 8 moment matrix Mo: a product
-// A B with A[(re/im, i)][j] = y_j X_i(v_col,j) (16 x n) and B[j][l] =
-// X_l(v_row,j) (n x 8), one mma.m16n8k8 per group of 8 cell-sorted nodes.  A
-// node's 2 x 8 basis values come from one lane (the recurrence: 8 packed FP32
-// operations for both coordinates) through shared memory, where lane (g, t) =
-// (lane / 4, lane % 4) picks up X_g of nodes t and t + 4 (the fragment layout
-// of the PTX ISA for tf32 m16n8k8).  Instead of 16 polynomial evaluations
-// per node (one per lane that holds a tap of it), each node's basis is
-// computed once.  When the cell changes, two more products turn Mo into G,
-// with the contraction index permuted (2t, 2t + 1 -> t, t + 4) so that each
-// D fragment is the next product's operand as it stands, and G goes to the
-// shared grid by shared-memory additions.  Each operand is split x = hi + lo
-// into TF32 parts and a product is hi*hi + hi*lo + lo*hi (relative error near
-// 2^-21); the three products of a group are summed by the tensor core, the
-// groups in FP32 registers.  A group holding nodes of several cells is run
-// once per cell with the other nodes masked.
-
-// Records rec[0, n) of one term for one warp, in steps of STEP = 32 nodes (4
-// groups of 8 for the tensor core; a step lying in one cell takes one test),
-// lane u holding node u of a step.  The warp's ring in shared memory (RING
-// steps of records) is filled by its lanes with cp.async DR steps ahead, and
-// records PF steps ahead are prefetched into L2 (one bulk prefetch per step),
-// so that the ring's copies find them there.  The value y[index] of a node is
-// loaded by its lane into registers DY steps ahead, through L2 only
-// (ld.global.cg: the scattered reads allocate no L1 lines, whose few hundred
-// per SM would otherwise bound the reads in flight, and they cost no
-// shared-memory writes); the lane then computes the node's basis and leaves
-// it, with the value, in shared memory: the basis rows X_0..X_7 of the
-// current step XROW words apart (= 8 mod 32: the four rows a half-warp reads
-// lie in distinct banks), then the step's values.
-// Order 1: B = e_0 (the single grid row), exact in TF32.
-template <int STEP>
-struct MmaRing {
-    static constexpr int RING = 4, DR = 3, DY = 2, PF = 7;   // PF: L2 prefetch distance
-    static constexpr int XROW = 2 * STEP + 8;   // words per basis row (STEP float2 + pad)
-    static constexpr size_t REC_BYTES = (size_t)RING * STEP * 16;                    // float4 records
-    static constexpr size_t X_OFF = REC_BYTES;                                       // basis rows
-    static constexpr size_t YC_OFF = X_OFF + (size_t)NCOEF * XROW * 4;               // + values
-    static constexpr size_t BYTES = YC_OFF + (size_t)STEP * 8;                       // per warp
-    static_assert(DY < DR && DR < RING && STEP == 32 && XROW % 32 == 8, "ring layout");
-};
-
-constexpr int MMA_STEP = 32;   // nodes per ring step of the order-1/2 tensor-core spread
-
-static size_t spread_mma_smem_bytes(long long max_grid_bytes) {
-    return (size_t)max_grid_bytes + MmaRing<MMA_STEP>::BYTES * (SPREAD_MMA_THREADS / 32) + 16;
-}
-
-template <int MR, bool ORD2>
-__device__ __forceinline__ void spread_mma_run(const float4 *__restrict__ rec, const float2 *__restrict__ y, int n,
-                                               float2 *S, int stride, const float *__restrict__ chr,
-                                               const float *__restrict__ chc, float4 *rring, float2 *xs,
-                                               float2 *yc) {
-    using R = MmaRing<MMA_STEP>;
-    constexpr unsigned MMA_RING = R::RING;
-    constexpr int MMA_DR = R::DR, MMA_DY = R::DY, XR = R::XROW / 2;   // basis row stride in float2
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int ns = (n + MMA_STEP - 1) / MMA_STEP;
-    int cur = -1;   // grid offset of the cell being summed
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
-    // d = Mo (re i = g, l = 2t), (re g, 2t + 1), (im g, 2t), (im g, 2t + 1)
-    auto flush = [&]() {
-        // this lane's window coefficients of the two products, split into TF32
-        // parts: the row window's C_row[g][2t], C_row[g][2t + 1] (zero for g >=
-        // 2 m_row; order 1: e_0 e_0^T) and the column window's C_col[g][2t],
-        // C_col[g][2t + 1] (Window::ch rows are taps)
-        unsigned ah[4], al[4], ch0, cl0, ch1, cl1;
-        {
-            float r0 = 0.f, r1 = 0.f;
-            if (ORD2) {
-                if (g < 2 * MR) {
-                    r0 = __ldg(chr + g * NCOEF + 2 * t);
-                    r1 = __ldg(chr + g * NCOEF + 2 * t + 1);
-                }
-            } else {
-                r0 = g == 0 && t == 0 ? 1.f : 0.f;
-            }
-            split_tf32_x2(pk2(r0, r1), ah[0], al[0], ah[2], al[2]);
-            ah[1] = ah[3] = al[1] = al[3] = 0u;
-            split_tf32_x2(pk2(__ldg(chc + g * NCOEF + 2 * t), __ldg(chc + g * NCOEF + 2 * t + 1)), ch0, cl0, ch1,
-                          cl1);
-        }
-        // Q_x[j][i] = sum_l C_row[j][l] Mo_x[i][l]: A = C_row (rows 8..15 zero),
-        // B[k][i] = Mo_x[i][l(k)] with l(t) = 2t, l(t + 4) = 2t + 1
-        unsigned mh[4], ml[4];
-        split_tf32_x2(pk2(d[0], d[1]), mh[0], ml[0], mh[1], ml[1]);
-        split_tf32_x2(pk2(d[2], d[3]), mh[2], ml[2], mh[3], ml[3]);
-        float qr[4] = {0.f, 0.f, 0.f, 0.f}, qi[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_tf32(qr, al, mh[0], mh[1]);
-        mma_tf32(qr, ah, ml[0], ml[1]);
-        mma_tf32(qr, ah, mh[0], mh[1]);
-        mma_tf32(qi, al, mh[2], mh[3]);
-        mma_tf32(qi, ah, ml[2], ml[3]);
-        mma_tf32(qi, ah, mh[2], mh[3]);
-        // q = Q_x[j = g][i = 2t], Q_x[g][2t + 1] (entries 2, 3: zero rows).
-        // G_x^T[j][k] = sum_i Q_x[j][i] C_col[k][i]: A[(x, j)][k'] = Q_x[j][i(k')],
-        // B[k'][k] = C_col[k][i(k')]
-        unsigned qh[4], ql[4];
-        split_tf32_x2(pk2(qr[0], qi[0]), qh[0], ql[0], qh[1], ql[1]);
-        split_tf32_x2(pk2(qr[1], qi[1]), qh[2], ql[2], qh[3], ql[3]);
-        float G[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_tf32(G, ql, ch0, ch1);
-        mma_tf32(G, qh, cl0, cl1);
-        mma_tf32(G, qh, ch0, ch1);
-        // G = (re, row tap g, column tap 2t), (re, g, 2t + 1), (im, g, 2t), (im, g, 2t + 1)
-        if (ORD2 ? g < 2 * MR : g == 0) {
-            float *c = (float *)(S + cur + g * stride + 2 * t);
-            red_add(c, G[0]);
-            red_add(c + 1, G[2]);
-            red_add(c + 2, G[1]);
-            red_add(c + 3, G[3]);
-        }
-        d[0] = d[1] = d[2] = d[3] = 0.f;
-    };
-    // tensor-core products of one group added to e (hi*lo terms first); a01 =
-    // (A[g][t], A[g + 8][t]), a23 = (A[g][t + 4], A[g + 8][t + 4])
-    auto group_mma = [&](float (&e)[4], f32x2 a01, f32x2 a23, unsigned bh0, unsigned bl0, unsigned bh1,
-                         unsigned bl1) {
-        unsigned ah[4], al[4];
-        split_tf32_x2(a01, ah[0], al[0], ah[1], al[1]);
-        split_tf32_x2(a23, ah[2], al[2], ah[3], al[3]);
-        mma_tf32(e, al, bh0, bh1);
-        if (ORD2) mma_tf32(e, ah, bl0, bl1);
-        mma_tf32(e, ah, bh0, bh1);
-    };
-    // basis row 0 is X_0 = 1 for every node
-    xs[lane] = make_float2(1.f, 1.f);
-    float2 y_mid = make_float2(0.f, 0.f), y_cur = y_mid;   // values of steps i + 1, i (DY = 2 in flight)
-    static_assert(MmaRing<MMA_STEP>::DY == 2, "two values in flight");
-    // A fresh tensor-core sum per step (at most eight groups), added to d in
-    // FP32 with rounding to nearest: the tensor core's own accumulation is
-    // not rounded to nearest, and its bias would grow with the cell's node
-    // count.
-    for (int i = -MMA_DR; i < ns; ++i) {
-        // iteration i commits one cp.async group, the records of step i + DR,
-        // and loads the values of step i + DY; steps i < 0 fill the pipeline
-        const int qr = i + MMA_DR, qy = i + MMA_DY, qp = i + R::PF;
-        // the records of step qp into L2 (whole records of the run only)
-        if (lane == 0 && qp < ns && qp >= MMA_DR)
-            prefetch_l2_bulk(rec + MMA_STEP * qp, 16u * (unsigned)min(MMA_STEP, n - MMA_STEP * qp));
-        if (qr < ns) cp_async16(&rring[((unsigned)qr % MMA_RING) * MMA_STEP + lane], rec + min(MMA_STEP * qr + lane, n - 1));
-        cp_async_commit();
-        // this lane's records of steps <= i + DR - 1 (the groups before this one) have landed
-        cp_async_wait_n<1>();
-        // the value of this lane's node of step qy, into registers
-        float2 y_next = make_float2(0.f, 0.f);
-        if (qy >= 0 && qy < ns) y_next = __ldcg(y + __float_as_int(rring[((unsigned)qy % MMA_RING) * MMA_STEP + lane].w));
-        const float2 y_now = y_cur;   // the value of this lane's node of step i
-        y_cur = y_mid;
-        y_mid = y_next;
-        if (i < 0) continue;
-        const int sl0 = ((unsigned)i % MMA_RING) * MMA_STEP;
-        // value and basis values X_1..X_7 of node `lane` of the step, (row,
-        // column) coordinate pairs: X_{k+1} = X_{k-1} + (-1)^k 2 v X_k
-        {
-            const int u = lane;
-            const float4 r = rring[sl0 + u];
-            yc[u] = y_now;
-            const f32x2 v = pk2(r.x, r.y);
-            const f32x2 up = mul2(v, pk2(2.f, 2.f)), um = mul2(v, pk2(-2.f, -2.f));
-            f32x2 xm = pk2(1.f, 1.f), x = v;
-            f32x2 *row = (f32x2 *)(xs + u);
-            row[XR] = x;
-#pragma unroll
-            for (int k = 2; k < NCOEF; ++k) {
-                const f32x2 xn = fma2((k & 1) ? up : um, x, xm);
-                row[k * XR] = xn;
-                xm = x;
-                x = xn;
-            }
-        }
-        __syncwarp();   // records, values and basis rows of step i visible to the warp
-        // two tensor-core sums (even and odd groups), so that two chains of
-        // dependent products are in flight
-        float e[4] = {0.f, 0.f, 0.f, 0.f}, e2[4] = {0.f, 0.f, 0.f, 0.f};
-        const bool whole = MMA_STEP * (i + 1) <= n;   // no group of this step runs past the end
-        // the records are in cell order: if the step's first and last nodes lie in
-        // the cell being summed, all of them do (the same test in every lane)
-        const bool step_in_cell = whole && __float_as_int(rring[sl0].z) == cur &&
-                                  __float_as_int(rring[sl0 + MMA_STEP - 1].z) == cur;
-        // operands of group h: A = y times X_g of the column coordinate of nodes
-        // t, t + 4, B = X_g of their row coordinate
-        struct GroupOp {
-            f32x2 a01, a23;
-            unsigned bh0, bl0, bh1, bl1;
-        };
-        auto operands = [&](int h) {
-            GroupOp o;
-            const float2 x0 = xs[g * XR + 8 * h + t], x1 = xs[g * XR + 8 * h + t + 4];
-            const float2 y0 = yc[8 * h + t], y1 = yc[8 * h + t + 4];
-            o.a01 = pk2(y0.x * x0.y, y0.y * x0.y);
-            o.a23 = pk2(y1.x * x1.y, y1.y * x1.y);
-            if (ORD2) {
-                split_tf32_x2(pk2(x0.x, x1.x), o.bh0, o.bl0, o.bh1, o.bl1);
-            } else {
-                o.bh0 = o.bh1 = g == 0 ? 0x3f800000u : 0u;
-                o.bl0 = o.bl1 = 0u;
-            }
-            return o;
-        };
-        if (step_in_cell) {
-            // every group of the step lies in the cell being summed
-#pragma unroll
-            for (int h = 0; h < MMA_STEP / 8; ++h) {
-                const GroupOp o = operands(h);
-                group_mma((h & 1) ? e2 : e, o.a01, o.a23, o.bh0, o.bl0, o.bh1, o.bl1);
-            }
-        } else {
-#pragma unroll
-            for (int h = 0; h < MMA_STEP / 8; ++h) {
-                const int base = MMA_STEP * i + 8 * h;   // first node of this group (may be past the end)
-                const GroupOp o = operands(h);
-                const int off0 = __float_as_int(rring[sl0 + 8 * h + t].z);
-                const int off1 = __float_as_int(rring[sl0 + 8 * h + t + 4].z);
-                if (__all_sync(0xffffffffu, (whole || base + 8 <= n) && off0 == cur && off1 == cur)) {
-                    // the whole group lies in the cell being summed
-                    group_mma((h & 1) ? e2 : e, o.a01, o.a23, o.bh0, o.bl0, o.bh1, o.bl1);
-                    continue;
-                }
-                // past the end the ring holds the last record again: masked here
-                bool p0 = base + t < n, p1 = base + t + 4 < n;   // nodes t, t + 4 not yet added
-                for (;;) {
-                    const unsigned pm =
-                        (__ballot_sync(0xffffffffu, p0) & 0xfu) | ((__ballot_sync(0xffffffffu, p1) & 0xfu) << 4);
-                    if (!pm) break;
-                    const int f = __ffs(pm) - 1;   // first node not yet added; its cell is next
-                    const int oc = __shfl_sync(0xffffffffu, f < 4 ? off0 : off1, f & 3);
-                    const bool e0 = p0 && off0 == oc, e1 = p1 && off1 == oc;
-                    if (oc != cur) {
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            d[q] += e[q] + e2[q];
-                            e[q] = e2[q] = 0.f;
-                        }
-                        if (cur >= 0) flush();
-                        cur = oc;
-                    }
-                    group_mma(e, e0 ? o.a01 : pk2(0.f, 0.f), e1 ? o.a23 : pk2(0.f, 0.f), o.bh0, o.bl0, o.bh1,
-                              o.bl1);
-                    p0 = p0 && !e0;
-                    p1 = p1 && !e1;
-                }
-            }
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) d[q] += e[q] + e2[q];
-        __syncwarp();   // ring slot i and the basis rows are read before later iterations refill them
-    }
-    cp_async_wait0();
-    if (cur >= 0) flush();
-}
-
-// Sorted item of order 1/2 on the tensor cores: the item's records are cut
-// into 8 contiguous runs (multiples of 8 nodes), one per warp.
-template <int MR>
-__device__ __forceinline__ void spread_mma_item(const DevPlan &P, const Term &T, const float2 *__restrict__ y,
-                                                long long j0, long long j1, float2 *S, unsigned char *stg_raw) {
-    const int warp = threadIdx.x >> 5;
-    constexpr int NW = SPREAD_MMA_THREADS / 32;
-    const long long len = j1 - j0, per = (len + 8 * NW - 1) / (8 * NW) * 8;
-    const long long a = j0 + warp * per, b = min(j1, a + per);
-    if (a >= b) return;
-    const float4 *rec = P.srec + (long long)T.sort_slot * P.M + a;
-    using R = MmaRing<MMA_STEP>;
-    unsigned char *ring = stg_raw + warp * R::BYTES;
-    float4 *rring = (float4 *)ring;
-    float2 *xs = (float2 *)(ring + R::X_OFF);
-    float2 *yc = (float2 *)(ring + R::YC_OFF);
-    const float *chc = &P.windows[T.wc].ch[0][0];
-    if (T.order == 2)
-        spread_mma_run<MR, true>(rec, y, (int)(b - a), S, T.stride, &P.windows[T.wr].ch[0][0], chc, rring, xs, yc);
-    else
-        spread_mma_run<MR, false>(rec, y, (int)(b - a), S, T.stride, nullptr, chc, rring, xs, yc);
-}
-
-// ---- Third-order cell sums on the tensor cores ----
-//
-// For the nodes j of one cell of a term (a, b, c) the window sums are
-//     G[ia][ib][k] += sum_j psi_a,ia(j) psi_b,ib(j) y_j psi_c,k(j).
-// For each row tap ia this is one product A B_ia: A[(k, re/im)][j] =
-// y_j psi_c,k(j) as in the order-2 kernel (shared by all ia) and
-// B_ia[j][ib] = psi_a,ia(j) psi_b,ib(j), 2 m_row mma.m16n8k8 (three TF32
-// products each) per group of 8 nodes.  Column n of B_ia holds second-row tap
-// ib = n / 2 (n even) or n / 2 + 4 (n odd), so the two taps a lane's D
-// fragment covers, t and t + 4, are 4 grid rows apart, which spreads its
-// shared-memory additions over more banks.  Lane (g, t) evaluates column tap
-// g, second-row tap ib(g) and first-row tap g of nodes t, t + 4; shuffles hand
-// each lane the first coordinate's taps of its nodes.  The sums stay in the D
-// fragments (4 per ia) and go to the shared grid (indices modulo n) when the
-// cell changes and after 8 steps of 16 nodes in one cell, which keeps the
-// tensor core's own accumulation chains short.
-constexpr int MMA3_STEP = 16, MMA3_RING = 4, MMA3_DR = 3, MMA3_DY = 1;
-constexpr size_t MMA3_REC_BYTES = (size_t)MMA3_RING * MMA3_STEP * 32;              // two float4 per node
-constexpr size_t MMA3_RING_BYTES = MMA3_REC_BYTES + (size_t)MMA3_RING * MMA3_STEP * 8;  // + float2 values
-static_assert(MMA3_DY < MMA3_DR && MMA3_DR < MMA3_RING && (MMA3_RING & (MMA3_RING - 1)) == 0, "ring depths");
-
-static size_t spread3_mma_smem_bytes(long long max_grid_bytes) {
-    return (size_t)max_grid_bytes + MMA3_RING_BYTES * (SPREAD_THREADS / 32) + 16;
-}
-
-template <int MR>
-__device__ __forceinline__ void spread3_mma_run(const float4 *__restrict__ rec, const float2 *__restrict__ y, int n,
-                                                float2 *S, const Term &T, const f32x2 cbp[NCOEF],
-                                                const float rcf[NCOEF], float4 *rring, float2 *yring) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-    const int ib_g = (g >> 1) + 4 * (g & 1);   // second-row tap of B column g
-    const int nn = T.n, stride = T.stride, mc = T.mc;
-    const int ns = (n + MMA3_STEP - 1) / MMA3_STEP;
-    int cur = -1, cfa = 0, cfb = 0, cfc = 0;   // the cell being summed: number and grid indices
-    float d[2 * MR][4];
-#pragma unroll
-    for (int a = 0; a < 2 * MR; ++a) d[a][0] = d[a][1] = d[a][2] = d[a][3] = 0.f;
-    // d[ia] = (re ib t, re ib t + 4, im ib t, im ib t + 4) of column tap g
-    int chain = 0;   // steps summed into d since the last flush
-    auto flush = [&]() {
-        const int col = wrap(cfc - mc + 1 + g, nn);
-        const int rb0 = wrap(cfb - MR + 1 + t, nn), rb1 = wrap(cfb - MR + 1 + t + 4, nn);
-#pragma unroll
-        for (int a = 0; a < 2 * MR; ++a) {
-            const int ra = wrap(cfa - MR + 1 + a, nn) * nn;
-            float *c0 = (float *)(S + (ra + rb0) * stride + col);
-            red_add(c0, d[a][0]);
-            red_add(c0 + 1, d[a][2]);
-            if (t + 4 < 2 * MR) {
-                float *c1 = (float *)(S + (ra + rb1) * stride + col);
-                red_add(c1, d[a][1]);
-                red_add(c1 + 1, d[a][3]);
-            }
-            d[a][0] = d[a][1] = d[a][2] = d[a][3] = 0.f;
-        }
-        chain = 0;
-    };
-    for (int i = -MMA3_DR; i < ns; ++i) {
-        // iteration i commits one cp.async group: the records of step i + MMA3_DR
-        // and the values of step i + MMA3_DY; lanes 0..15 copy one node each
-        if (lane < MMA3_STEP) {
-            const int qr = i + MMA3_DR, qy = i + MMA3_DY;
-            if (qr < ns) {
-                const float4 *src = rec + 2 * min(MMA3_STEP * qr + lane, n - 1);
-                float4 *dst = &rring[((qr & (MMA3_RING - 1)) * MMA3_STEP + lane) * 2];
-                cp_async16(dst, src);
-                cp_async16(dst + 1, src + 1);
-            }
-            if (qy >= 0 && qy < ns) {
-                cp_async_wait_n<MMA3_DR - MMA3_DY - 1>();
-                const int j = __float_as_int(rring[((qy & (MMA3_RING - 1)) * MMA3_STEP + lane) * 2].w);
-                cp_async8(&yring[(qy & (MMA3_RING - 1)) * MMA3_STEP + lane], y + j);
-            }
-        }
-        cp_async_commit();
-        if (i < 0) continue;
-        cp_async_wait_n<MMA3_DY>();
-        __syncwarp();
-#pragma unroll
-        for (int h = 0; h < MMA3_STEP / 8; ++h) {
-            const int base = MMA3_STEP * i + 8 * h;   // first node of this group (may be past the end)
-            const int sl = (i & (MMA3_RING - 1)) * MMA3_STEP + 8 * h;
-            const float4 q0 = rring[2 * (sl + t)], c0 = rring[2 * (sl + t) + 1];
-            const float4 q1 = rring[2 * (sl + t + 4)], c1 = rring[2 * (sl + t + 4) + 1];
-            const float2 y0 = yring[sl + t], y1 = yring[sl + t + 4];
-            // column tap g and second-row tap ib(g) (the B column) of nodes t,
-            // t + 4, one packed Horner per node; first-row tap g here, handed
-            // round below
-            const bool gok = ib_g < 2 * MR;
-            float wc0, wc1, wb0, wb1;
-            horner8_x2(cbp, q0.z, q0.y, wc0, wb0);
-            horner8_x2(cbp, q1.z, q1.y, wc1, wb1);
-            wb0 = gok ? wb0 : 0.f;
-            wb1 = gok ? wb1 : 0.f;
-            const float wa0 = horner8(rcf, q0.x), wa1 = horner8(rcf, q1.x);
-            const int key0 = __float_as_int(c0.w), key1 = __float_as_int(c1.w);
-            bool p0 = base + t < n, p1 = base + t + 4 < n;   // nodes t, t + 4 not yet added
-            const bool fast = __all_sync(0xffffffffu, p0 && p1 && key0 == cur && key1 == cur);
-            for (;;) {
-                bool e0 = p0, e1 = p1;
-                if (!fast) {
-                    const unsigned pm =
-                        (__ballot_sync(0xffffffffu, p0) & 0xfu) | ((__ballot_sync(0xffffffffu, p1) & 0xfu) << 4);
-                    if (!pm) break;
-                    const int f = __ffs(pm) - 1;   // first node not yet added; its cell is next
-                    const int src = f & 3;
-                    const bool second = f >= 4;
-                    const int oc = __shfl_sync(0xffffffffu, second ? key1 : key0, src);
-                    e0 = p0 && key0 == oc;
-                    e1 = p1 && key1 == oc;
-                    if (oc != cur) {
-                        if (cur >= 0) flush();
-                        cur = oc;
-                        cfa = __shfl_sync(0xffffffffu, __float_as_int(second ? c1.x : c0.x), src);
-                        cfb = __shfl_sync(0xffffffffu, __float_as_int(second ? c1.y : c0.y), src);
-                        cfc = __shfl_sync(0xffffffffu, __float_as_int(second ? c1.z : c0.z), src);
-                    }
-                }
-                unsigned ah[4], al[4];
-                split_tf32_x2(e0 ? mul2(pk2(y0.x, y0.y), pk2(wc0, wc0)) : pk2(0.f, 0.f), ah[0], al[0], ah[1], al[1]);
-                split_tf32_x2(e1 ? mul2(pk2(y1.x, y1.y), pk2(wc1, wc1)) : pk2(0.f, 0.f), ah[2], al[2], ah[3], al[3]);
-                const f32x2 wb = pk2(wb0, wb1);
-#pragma unroll
-                for (int a = 0; a < 2 * MR; ++a) {
-                    // first coordinate's tap a of nodes t, t + 4 from lane (a, t)
-                    const float va0 = __shfl_sync(0xffffffffu, wa0, 4 * a + t);
-                    const float va1 = __shfl_sync(0xffffffffu, wa1, 4 * a + t);
-                    unsigned bh0, bl0, bh1, bl1;
-                    split_tf32_x2(mul2(pk2(va0, va1), wb), bh0, bl0, bh1, bl1);
-                    mma_tf32(d[a], al, bh0, bh1);
-                    mma_tf32(d[a], ah, bl0, bl1);
-                    mma_tf32(d[a], ah, bh0, bh1);
-                }
-                if (fast) break;
-                p0 = p0 && !e0;
-                p1 = p1 && !e1;
-            }
-        }
-        // at most 8 steps per tensor-core chain
-        if (cur >= 0 && ++chain == 8) flush();
-        __syncwarp();   // ring slot i is read before a later iteration refills it
-    }
-    cp_async_wait0();
-    if (cur >= 0) flush();
-}
-
-template <int MR>
-__device__ __forceinline__ void spread3_mma_item(const DevPlan &P, const Term &T, const float2 *__restrict__ y,
-                                                 long long j0, long long j1, float2 *S, unsigned char *stg_raw) {
-    const int warp = threadIdx.x >> 5, g = (threadIdx.x & 31) >> 2;
-    // (column tap g, second-row tap of B column g) pairs, first-row tap g
-    f32x2 cbp[NCOEF];
-    float rcf[NCOEF];
-    {
-        const int ib = (g >> 1) + 4 * (g & 1);
-        const float *cs = P.windows[T.wc].c[g];
-        const float *rs = P.windows[T.wr].c[min(g, 2 * MR - 1)];
-        const float *bs = P.windows[T.wr].c[min(ib, 2 * MR - 1)];
-#pragma unroll
-        for (int q = 0; q < NCOEF; ++q) {
-            cbp[q] = pk2(__ldg(cs + q), __ldg(bs + q));
-            rcf[q] = __ldg(rs + q);
-        }
-    }
-    constexpr int NW = SPREAD_THREADS / 32;
-    const long long len = j1 - j0, per = (len + 8 * NW - 1) / (8 * NW) * 8;
-    const long long a = j0 + warp * per, b = min(j1, a + per);
-    if (a >= b) return;
-    unsigned char *ring = stg_raw + warp * MMA3_RING_BYTES;
-    spread3_mma_run<MR>(P.srec + (long long)T.sort_slot * P.M + 2 * a, y, (int)(b - a), S, T, cbp, rcf,
-                        (float4 *)ring, (float2 *)(ring + MMA3_REC_BYTES));
-}
-
 // One work item (x = problem, y = active term, z = node chunk, w = chunks per
 // term) spreads nodes [M z / w, M (z+1) / w) of one term (in the term's cell
 // order if the plan keeps sorted copies and the term has order <= 2, else in
 // the original order) into a shared-memory copy of the term's stored grid
 // (halos included) and writes it to partial grid z of its problem.  CTAs take
-// items from a global counter.
-// KIND: SK_STAGED (order 1/2 on the CUDA cores), SK_ORDER3, SK_MMA (order 1/2
-// with records on the tensor cores; no staging area)
-template <int MR, typename G, int KIND, int SP, int NT = SPREAD_THREADS>
+// items from a global counter.  O3: third-order items.
+template <int MR, typename G, bool O3, int SP>
 __device__ __forceinline__ void spread_items(const DevPlan &single, const BatchArgs &B,
                                              const float2 *__restrict__ y_base, int item_begin, int item_end,
                                              int *counter, long long max_grid_bytes) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float2 *S = (float2 *)smem_raw;
     unsigned char *stg_raw = smem_raw + max_grid_bytes;
-    constexpr bool O3 = KIND == SK_ORDER3;
-    int &s_item = *(int *)(stg_raw + (KIND == SK_MMA    ? MmaRing<MMA_STEP>::BYTES * (NT / 32)
-                                      : KIND == SK_MMA3 ? MMA3_RING_BYTES * (NT / 32)
-                                      : O3              ? SP3_STAGE_BYTES
-                                                        : sp_stage_bytes(SP)));
+    constexpr int NT = SPREAD_THREADS;
+    int &s_item = *(int *)(stg_raw + (O3 ? SP3_STAGE_BYTES : sp_stage_bytes(SP)));
     const int tid = threadIdx.x;
     const int k = tid & 7;
     for (;;) {
@@ -1025,24 +591,23 @@ __device__ __forceinline__ void spread_items(const DevPlan &single, const BatchA
         // window coefficients of this lane: row tap k for lanes r = 1 of an
         // order-2 term (see node_weights), column tap k otherwise
         float wcf[NCOEF];
-        if constexpr (KIND != SK_MMA && KIND != SK_MMA3) {
+        {
             const bool row = T.order == 2 && (tid & 8);
             const float *wsrc = row ? P.windows[T.wr].c[min(k, 2 * MR - 1)] : P.windows[T.wc].c[k];
 #pragma unroll
             for (int i = 0; i < NCOEF; ++i) wcf[i] = __ldg(wsrc + i);
         }
+        // in a batch whose other problems have no room for sorted nodes, a problem
+        // may hold node tiles, which only the tensor-core kernels read
+        const bool sorted = T.sort_slot >= 0 && P.srec && !P.tile_cell;
         __syncthreads();   // grid zeroed before any addition
-        if constexpr (KIND == SK_MMA) {
-            spread_mma_item<MR>(P, T, y, j0, j1, S, stg_raw);
-        } else if constexpr (KIND == SK_MMA3) {
-            spread3_mma_item<MR>(P, T, y, j0, j1, S, stg_raw);
-        } else if constexpr (O3) {
-            if (T.sort_slot >= 0 && P.srec)
+        if constexpr (O3) {
+            if (sorted)
                 spread_sorted_item3<MR>(P, T, y, j0, j1, S, stg_raw, wcf);
             else
                 spread_unsorted_item<MR, true, SP>(P, T, y, j0, j1, S, stg_raw, wcf);
         } else {
-            if (T.sort_slot >= 0 && P.srec)
+            if (sorted)
                 spread_sorted_item<MR, SP>(P, T, y, j0, j1, S, stg_raw, wcf);
             else
                 spread_unsorted_item<MR, false, SP>(P, T, y, j0, j1, S, stg_raw, wcf);
@@ -1065,32 +630,14 @@ template <int MR, typename G, int SP>
 __global__ void __launch_bounds__(SPREAD_THREADS, SP == SP_CH ? 3 : SPREAD_MAX_CTAS_PER_SM)
 spread_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, int item_begin, int item_end,
            int *counter, long long max_grid_bytes) {
-    spread_items<MR, G, SK_STAGED, SP>(single, B, y_base, item_begin, item_end, counter, max_grid_bytes);
-}
-
-// order-1/2 items of plans with cell-sorted records, on the tensor cores, in
-// steps of STEP nodes
-template <int MR, typename G>
-__global__ void __launch_bounds__(SPREAD_MMA_THREADS, SPREAD_MMA_CTAS_PER_SM)
-spread_mma_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, int item_begin, int item_end,
-               int *counter, long long max_grid_bytes) {
-    spread_items<MR, G, SK_MMA, MMA_STEP, SPREAD_MMA_THREADS>(single, B, y_base, item_begin, item_end, counter,
-                                                              max_grid_bytes);
-}
-
-// third-order items of plans with cell-sorted records, on the tensor cores
-template <int MR, typename G>
-__global__ void __launch_bounds__(SPREAD_THREADS, 2)
-spread3_mma_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, int item_begin, int item_end,
-                int *counter, long long max_grid_bytes) {
-    spread_items<MR, G, SK_MMA3, 0>(single, B, y_base, item_begin, item_end, counter, max_grid_bytes);
+    spread_items<MR, G, false, SP>(single, B, y_base, item_begin, item_end, counter, max_grid_bytes);
 }
 
 template <int MR, typename G>
 __global__ void __launch_bounds__(SPREAD_THREADS, 2)
 spread3_f32(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, int item_begin, int item_end,
             int *counter, long long max_grid_bytes) {
-    spread_items<MR, G, SK_ORDER3, SP_CH / 2>(single, B, y_base, item_begin, item_end, counter, max_grid_bytes);
+    spread_items<MR, G, true, SP_CH / 2>(single, B, y_base, item_begin, item_end, counter, max_grid_bytes);
 }
 
 template <typename G>
@@ -1169,6 +716,7 @@ adjoint_post_f32(DevPlan single, BatchArgs B, float2 *__restrict__ fhat_base, in
     const DevPlan &P = B.plans ? B.plans[pb] : single;
     const int sblk = B.plans ? (int)blockIdx.x - B.blk0[pb] : (int)blockIdx.x;
     if (P.skip && *P.skip) return;
+    if (sblk == 0 && threadIdx.x == 0) P.err[ERR_YMAX] = 0;
     float2 *__restrict__ fhat = fhat_base + P.vec_coef_off;
     const Term T = P.terms[P.act[sblk]];
     const int n = T.n, s = T.order, N = T.N;
@@ -1228,18 +776,30 @@ adjoint_post_f32(DevPlan single, BatchArgs B, float2 *__restrict__ fhat_base, in
 }
 
 // partial sums of y for the empty-set coefficients, one per block (of the
-// problem blockIdx.y); adjoint_post_f32 adds them
-__global__ void sum_y_partial(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, double2 *part_base) {
+// problem blockIdx.y), which adjoint_post_f32 adds; with find_max also the
+// largest |Re|, |Im| of y as float bits (NaN above all), for the scale of the
+// third-order terms' FP16 operands
+__global__ void sum_y_partial(DevPlan single, BatchArgs B, const float2 *__restrict__ y_base, double2 *part_base,
+                              bool find_max) {
     __shared__ double sh[32];
     const DevPlan &P = B.plans ? B.plans[blockIdx.y] : single;
-    if (P.n_empty == 0 || (P.skip && *P.skip)) return;
+    if (P.skip && *P.skip) return;
     const float2 *__restrict__ y = y_base + P.vec_node_off;
     double sx = 0, sy = 0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < P.M; i += (long long)gridDim.x * blockDim.x) {
-        const float2 v = y[i];
+    unsigned m = 0u;
+    const long long M = P.M, step = (long long)gridDim.x * blockDim.x;
+#pragma unroll 4
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < M; i += step) {
+        const float2 v = __ldg(y + i);
         sx += v.x;
         sy += v.y;
+        m = max(m, max(__float_as_uint(v.x) & 0x7fffffffu, __float_as_uint(v.y) & 0x7fffffffu));
     }
+    if (find_max) {
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((threadIdx.x & 31) == 0 && m) atomicMax((unsigned *)P.err + ERR_YMAX, m);
+    }
+    if (P.n_empty == 0) return;
     sx = block_sum_fixed(sx, sh);
     sy = block_sum_fixed(sy, sh);
     if (threadIdx.x == 0) part_base[(long long)blockIdx.y * gridDim.x + blockIdx.x] = make_double2(sx, sy);
@@ -1255,10 +815,6 @@ static void adjoint_attrs() {
         cudaFuncSetAttribute(spread_f32<3, G, SP_CH / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
         cudaFuncSetAttribute(spread_f32<4, G, SP_CH / 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
         cudaFuncSetAttribute(spread3_f32<3, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
-        cudaFuncSetAttribute(spread3_mma_f32<3, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
-        cudaFuncSetAttribute(spread3_mma_f32<4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
-        cudaFuncSetAttribute(spread_mma_f32<3, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
-        cudaFuncSetAttribute(spread_mma_f32<4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
         cudaFuncSetAttribute(spread3_f32<4, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, MAX_SMEM);
     });
 }
@@ -1270,38 +826,25 @@ template <typename G>
 static void adjoint_kernels(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P,
                             const float2 *y, float2 *fhat, int n_items, int n_items3, int *counter, int n_blocks,
                             int mr, long long sgrid, int max_fft_elems, int max_n, int max_stage, int sm_count,
-                            long long max_grid_elems, int max_chunks, const double2 *y_part, int n_ypart, bool tc) {
+                            long long max_grid_elems, int max_chunks, const double2 *y_part, int n_ypart, int prec,
+                            bool tc) {
     adjoint_attrs<G>();
-    const int sp = spread_block_nodes(sgrid);
-    const size_t ssm = spread_smem_bytes(sgrid, false, sp), ssm3 = spread_smem_bytes(sgrid, true, sp);
-    const int per_sm = spread_ctas_per_sm(sgrid, false);
     if (n_blocks > 0) {
         if (prof) stage_begin(*prof, ST_SPREAD);
-        if (n_items3 > 0 && tc) {
-            const size_t sm3 = spread3_mma_smem_bytes(sgrid);
-            const int per3 = (int)std::max<size_t>(1, std::min<size_t>(2, (size_t)(MAX_SMEM + 1024) / (sm3 + 1024)));
-            const int c3 = std::max(1, std::min(n_items3, per3 * sm_count));
-            auto k = mr <= 3 ? spread3_mma_f32<3, G> : spread3_mma_f32<4, G>;
-            k<<<c3, SPREAD_THREADS, sm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
+        const int sp = spread_block_nodes(sgrid), per_sm = spread_ctas_per_sm(sgrid);
+        if (tc) {
+            spread_tiles_launch(st, v, B, y, n_items, n_items3 > 0, counter, sgrid, sm_count, mr, prec);
         } else if (n_items3 > 0) {
             const int c3 = std::max(1, std::min(n_items3, std::min(per_sm, 2) * sm_count));
-            if (mr <= 3)
-                spread3_f32<3, G><<<c3, SPREAD_THREADS, ssm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
-            else
-                spread3_f32<4, G><<<c3, SPREAD_THREADS, ssm3, st>>>(v, B, y, 0, n_items3, counter, sgrid);
+            auto k = mr <= 3 ? spread3_f32<3, G> : spread3_f32<4, G>;
+            k<<<c3, SPREAD_THREADS, spread_smem_bytes(sgrid, true, sp), st>>>(v, B, y, 0, n_items3, counter, sgrid);
         }
-        if (n_items > n_items3 && tc) {
-            const size_t sm = spread_mma_smem_bytes(sgrid);
-            const int per = (int)std::max<size_t>(
-                1, std::min<size_t>(SPREAD_MMA_CTAS_PER_SM, (size_t)(MAX_SMEM + 1024) / (sm + 1024)));
-            const int c = std::max(1, std::min(n_items - n_items3, per * sm_count));
-            auto k = mr <= 3 ? spread_mma_f32<3, G> : spread_mma_f32<4, G>;
-            k<<<c, SPREAD_MMA_THREADS, sm, st>>>(v, B, y, n_items3, n_items, counter + 1, sgrid);
-        } else if (n_items > n_items3) {
+        if (!tc && n_items > n_items3) {
             const int c = std::max(1, std::min(n_items - n_items3, per_sm * sm_count));
             auto k = mr <= 3 ? (sp == SP_CH ? spread_f32<3, G, SP_CH> : spread_f32<3, G, SP_CH / 2>)
                              : (sp == SP_CH ? spread_f32<4, G, SP_CH> : spread_f32<4, G, SP_CH / 2>);
-            k<<<c, SPREAD_THREADS, ssm, st>>>(v, B, y, n_items3, n_items, counter + 1, sgrid);
+            k<<<c, SPREAD_THREADS, spread_smem_bytes(sgrid, false, sp), st>>>(v, B, y, n_items3, n_items, counter + 1,
+                                                                             sgrid);
         }
         if (prof) stage_end(*prof, ST_SPREAD);
     }
@@ -1327,11 +870,12 @@ int adjoint_launch(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArg
                    float2 *fhat, int n_items, int n_items3, int *counter, int n_blocks, int mr,
                    long long max_grid_bytes, int max_fft_elems, int max_n, int max_stage, int sm_count, long long max_grid_elems,
                    int max_chunks, bool any_empty, double2 *scratch, int prec, bool tc) {
+    const bool find_max = tc && n_items3 > 0;
     // enough blocks to fill the chip, shared among the problems
-    const int n_ypart = any_empty ? std::max(8, SUM_Y_BLOCKS / P) : 0;
-    if (any_empty) {
+    const int ny = std::max(32, SUM_Y_BLOCKS / P), n_ypart = any_empty ? ny : 0;
+    if (any_empty || find_max) {
         if (prof) stage_begin(*prof, ST_SUMY);
-        sum_y_partial<<<dim3(n_ypart, P), 256, 0, st>>>(v, B, y, scratch);
+        sum_y_partial<<<dim3(ny, P), 256, 0, st>>>(v, B, y, scratch, find_max);
         if (prof) stage_end(*prof, ST_SUMY);
     }
     auto run = prec == ANOVA_PREC_F16    ? adjoint_kernels<__half2>
@@ -1339,7 +883,7 @@ int adjoint_launch(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArg
                                          : adjoint_kernels<float2>;
     const long long sgrid = prec == ANOVA_PREC_F32 ? max_grid_bytes : 2 * max_grid_bytes;
     run(prof, st, v, B, P, y, fhat, n_items, n_items3, counter, n_blocks, mr, sgrid, max_fft_elems, max_n, max_stage,
-        sm_count, max_grid_elems, max_chunks, scratch, n_ypart, tc);
+        sm_count, max_grid_elems, max_chunks, scratch, n_ypart, prec, tc);
     return cuda_status(cudaGetLastError());
 }
 

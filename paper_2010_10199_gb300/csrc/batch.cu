@@ -245,7 +245,6 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
     b->node_off.assign(n_problems + 1, 0);
     b->coef_off.assign(n_problems + 1, 0);
     std::vector<int> tile_prob, tile0, blk_prob, blk0;
-    int total_act = 0;
     int pitch = -1;
     bool mixed_pitch = false;
     for (int p = 0; p < n_problems; ++p) {
@@ -275,7 +274,6 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
         tile0.push_back(b->n_tiles);
         for (int t = 0; t < tiles; ++t) tile_prob.push_back(p);
         b->n_tiles += tiles;
-        total_act += pl.n_act;
         blk0.push_back(b->n_blocks);
         for (int t = 0; t < pl.n_act; ++t) blk_prob.push_back(p);
         b->n_blocks += pl.n_act;
@@ -298,19 +296,21 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
         b->sm_count = pl.sm_count;
     }
     b->pitch = mixed_pitch || pitch < 0 ? 0 : pitch;
-    // spread items: every problem's active terms split into K_p node chunks,
-    // K_p sized for all problems sharing the GPU
+    // spread items: every problem's active terms split into K_p node chunks of about
+    // the same size for all problems (one chunk per term each, the largest problem's
+    // items ran alone at the end)
     std::vector<int4> items;
     std::vector<int> Ks(n_problems);
-    bool order3 = false;
-    for (int p = 0; p < n_problems; ++p) {
-        const Plan &pl = b->plans[p]->p;
-        for (int i = 0; i < pl.n_act; ++i) order3 = order3 || pl.h_terms[pl.h_act[i]].order == 3;
-    }
+    auto third = [](const Plan &pl) {
+        int n3 = 0;
+        for (int i = 0; i < pl.n_act; ++i) n3 += pl.h_terms[pl.h_act[i]].order == 3;
+        return n3;
+    };
+    double total_ns = 0.0;
+    for (anova_plan_t h : b->plans) total_ns += batch_cost_ns(h->p.M, h->p.n_act, third(h->p));
     for (int p = 0; p < n_problems; ++p) {
         Plan &pl = b->plans[p]->p;
-        Ks[p] = spread_chunks_for(pl.M, total_act, pl.spread_kmax, b->max_grid_bytes, b->sm_count, b->cell_tc,
-                                  order3);
+        Ks[p] = batch_chunks_for(pl.M, total_ns, pl.spread_kmax, 2LL * b->sm_count);
         b->views[p].spread_chunks = Ks[p];
         b->max_chunks = std::max(b->max_chunks, Ks[p]);
     }
@@ -331,9 +331,9 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
     if (e == cudaSuccess) e = cudaMalloc(&b->d_items, sizeof(int4) * std::max<size_t>(1, items.size()));
     if (e == cudaSuccess) e = cudaMalloc(&b->counter, 2 * sizeof(int));
     if (e == cudaSuccess) e = cudaMemsetAsync(b->counter, 0, 2 * sizeof(int), b->stream);
-    // partial sums: 256 complex ones per problem, or a double per block of the FFT passes
+    // partial sums: at most 608 or 32 complex ones per problem, or a double per block of the FFT passes
     if (e == cudaSuccess)
-        e = cudaMalloc(&b->scratch, std::max(sizeof(double2) * 256 * n_problems, sizeof(double) * b->n_blocks));
+        e = cudaMalloc(&b->scratch, std::max(sizeof(double2) * (608 + 32 * (size_t)n_problems), sizeof(double) * b->n_blocks));
     if (e != cudaSuccess) {
         free_batch(b);
         return cuda_status(e);

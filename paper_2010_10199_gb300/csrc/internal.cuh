@@ -39,6 +39,7 @@ constexpr int MAX_SMEM = 227 * 1024;
 struct Window {
     float c[2 * MAXM][NCOEF];
     float ch[2 * MAXM][NCOEF];
+    float pb[2 * MAXM][NCOEF];   // the same polynomials in the product basis (tiles.cuh)
     int m;
     float b;          // shape parameter pi (2 - 1/sigma)
     float inv_psi0;   // 1 / psi(0)
@@ -65,6 +66,8 @@ struct Term {
     int hr, hc;         // halo widths (rows, columns): stored index = periodic index + halo
     int erows;          // stored rows (order 2: n + 2 hr + 1; order 1: 1; order 3: n^2, no halo)
     int sort_slot;      // slot of this term's cell-sorted node copy (-1: none)
+    long long rec_off;  // node tiles: first record (float4 units) and first tile
+    long long tile_off;
     long long grid_off;   // element offset in the grid buffer
     long long grid_bytes; // bytes (multiple of 16)
     long long coef_off;   // offset in the coefficient vector
@@ -102,7 +105,9 @@ inline ActRec make_act_rec(const Term &T, int term, int newgroup) {
     return a;
 }
 
-// A node in the cell order of one term (16 bytes, stored as float4):
+// A node in the cell order of one term, plans whose cell products run on the
+// CUDA cores and FP64 plans (16 bytes, stored as float4; the tensor-core kernels'
+// tiles: tiles.cuh):
 //   x: 2 tau_row - 1 (order 2; 0 for order 1), y: 2 tau_col - 1, the window
 //   polynomial arguments of the node's fractional grid positions;
 //   z (int bits): stored-grid offset of the first tap, i_row * stride + i_col
@@ -133,7 +138,9 @@ struct DevPlan {
     const float2 *grids;      // stored grids of this problem
     float2 *partials;         // adjoint partial grids [spread_chunks][grid_elems]
     int spread_chunks;        // node chunks of the adjoint (one partial grid each)
-    const float4 *srec;       // [slot][M] nodes sorted by grid cell, see SortedNode
+    const float4 *srec;       // nodes sorted by grid cell: [slot][M] records, or node tiles if tile_cell is set
+    const int *tile_cell;     // cell of every tile (null: srec holds records)
+    const int *tile_count;    // tiles per scheduled term
     unsigned long long *facc; // sorted forward: fixed-point accumulators [M][2] (or null), zero between calls
     int *fexp;                // their exponent, and a block counter (zero between launches)
     long long n_coeffs;
@@ -154,6 +161,10 @@ struct BatchArgs {
     const int *blk_prob;      // pre/post: problem of each (problem, active term) block
     const int *blk0;          // first block of each problem
 };
+
+// words of DevPlan::err: the error code of bounded waits; the largest |Re|, |Im| of
+// the adjoint's input (float bits, zero between calls)
+enum { ERR_CODE = 0, ERR_YMAX = 2 };
 
 constexpr int N_STAGES = 7;
 struct Profiler;   // per-stage CUDA-event timing (profile.cu)
@@ -176,7 +187,8 @@ struct Plan {
     long long *h_user_off;  // per user term: coefficient offset
     long long *h_user_len;
     int *h_user_n, *h_user_mc, *h_user_mr, *h_user_order;
-    // device buffers
+    // device memory: parts of arena, the sorted copies and accumulators of arena_opt
+    void *arena, *arena_opt;
     void *x;                // FP32 or FP64 nodes [d][M]
     Term *terms;
     Window *windows;
@@ -208,7 +220,9 @@ struct Plan {
     int n_items3;           // the first n_items3 items are those of third-order terms
     int *counter;           // work-queue counters (2), zero between calls
     float4 *srec;           // cell-sorted node records (null: none), n_sorted slots of M
-    bool cell_tc;           // order-1/2 spread of sorted records on the tensor cores
+    bool cell_tc;           // srec holds node tiles: cell products on the tensor cores
+    int *tile_cell;         // tiles: their cells, and the tiles per scheduled term
+    int *tile_count;
     int n_sorted;
     unsigned long long *facc;   // sorted forward: fixed-point accumulators [M][2]
     int *fexp;              // and their exponent
@@ -265,16 +279,15 @@ enum { ST_PRE = 0, ST_GATHER = 1, ST_SPREAD = 2, ST_REDUCE = 3, ST_POST = 4, ST_
 // kernels launched by the entry points (trafo.cu / adjoint.cu)
 int launch_trafo_f32(Plan &p, const float2 *fhat, float2 *f);
 int launch_gather_f32(Plan &p, const float2 *fhat, float2 *f);
-// Sorted forward (gather_sorted.cu): order-1/2 terms over the cell-sorted
-// records, accumulated into f with atomics; f must hold the other terms' sum.
+// Sorted forward (gather_sorted.cu), every term over its cell-sorted records:
+// f = empty-set coefficient + all terms.
 int launch_gather_sorted_f32(Plan &p, const float2 *fhat, float2 *f);
 // The same for one problem (B.plans == null) or a batch of P problems, every one
-// with records and accumulators: f = empty-set coefficient + all terms.
-// Sorted forward of one problem or a batch: fixed-point passes around the
-// gather of items [0, item_end); the first n_items3 are third-order items;
-// with tc and none of those, the gather runs on the tensor cores.
+// with records and accumulators: the gather of items [0, n_items), the first
+// n_items3 of them third-order ones, and the fixed-point pass after it.  tc: the
+// plans hold node tiles, the gather runs on the tensor cores.
 int gather_sorted_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P, const float2 *fhat,
-                         float2 *f, const int4 *items, int n_items3, int item_end, int *counter,
+                         float2 *f, const int4 *items, int n_items3, int n_items, int *counter,
                          long long max_grid_bytes, long long max_M, int sm_count, int mr, bool tc);
 int launch_adjoint_f32(Plan &p, const float2 *y, float2 *fhat);
 int adjoint_launch(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArgs &B, int P, const float2 *y,
@@ -289,14 +302,23 @@ int sort_nodes_by_cell(Plan &p);
 int build_window_tables_f64(Plan &p);
 int launch_trafo_f64(Plan &p, const double2 *fhat, double2 *f);
 int launch_adjoint_f64(Plan &p, const double2 *y, double2 *fhat);
-// CTAs per SM of the order-1/2 spread kernel (tc: the tensor-core one)
-int spread_ctas_per_sm(long long max_grid_bytes, bool tc);
-// Node chunks per term for a spread over n_act_total active terms (all
-// problems of a launch) on sm_count SMs: about three items per resident
-// spread CTA (with third-order terms, order3, per CTA of 3 per SM at least),
-// at most kmax, at least 2048 nodes per chunk.
-int spread_chunks_for(long long M, int n_act_total, int kmax, long long max_grid_bytes, int sm_count, bool tc,
-                      bool order3);
+// Node tiles (gather_tiles.cu, spread_tiles.cu, sort.cu).
+void gather_tiles_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, const int4 *items, int n_items,
+                         bool order3, int *counter, long long max_grid_bytes, int sm_count, int mr);
+void spread_tiles_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, const float2 *y, int n_items,
+                         bool order3, int *counter, long long sgrid, int sm_count, int mr, int prec);
+int spread_tiles_ctas_per_sm(long long sgrid, bool order3);
+int gather_tiles_ctas_per_sm(long long max_grid_bytes, bool order3);
+// CTAs per SM of the order-1/2 spread kernel on the CUDA cores
+int spread_ctas_per_sm(long long max_grid_bytes);
+// Node chunks per term for a problem of n_terms active terms, n_terms3 of them
+// third-order, at most kmax.
+int spread_chunks_for(long long M, int n_terms, int n_terms3, int kmax, long long max_grid_bytes,
+                      long long grid_elems, int sm_count, bool tc);
+// The same for one problem of a batch whose problems cost total_ns (the sum of
+// batch_cost_ns) on ctas CTAs.
+double batch_cost_ns(long long M, int n_terms, int n_terms3);
+int batch_chunks_for(long long M, double total_ns, int kmax, long long ctas);
 // Appends the spread work items of one problem, K chunks per active term:
 // those of the third-order terms (sel = 3) or of the others, order 2 before
 // order 1 (sel = 0).  Returns the count.

@@ -13,6 +13,7 @@
 
 #include "device.cuh"
 #include "internal.cuh"
+#include "tiles.cuh"
 
 namespace agft {
 
@@ -58,7 +59,7 @@ void window_polys(Window &w, int m, double b) {
     const int P = NCOEF;
     double psi0 = kb_window(0.0, m, b);
     for (int j = 0; j < 2 * MAXM; ++j)
-        for (int i = 0; i < P; ++i) w.c[j][i] = w.ch[j][i] = 0.0f;
+        for (int i = 0; i < P; ++i) w.c[j][i] = w.ch[j][i] = w.pb[j][i] = 0.0f;
     for (int j = 0; j < 2 * m; ++j) {
         double fv[NCOEF], a[NCOEF];
         for (int i = 0; i < P; ++i) {
@@ -72,6 +73,12 @@ void window_polys(Window &w, int m, double b) {
             a[k] = (k == 0 ? 1.0 : 2.0) * s / P;
             w.ch[j][k] = (float)(((k >> 1) & 1) ? -a[k] : a[k]);   // s_k a_k
         }
+        // product basis: T_3 = 2 v T_2 - v, T_5 = 2 v T_4 - T_3, T_6 = 2 T_2 T_4 - T_2,
+        // T_7 = 4 v T_2 T_4 - T_5 - T_3 - T_1
+        static_assert(NCOEF == 8, "product basis of degree 7");
+        const double pb[NCOEF] = {a[0], a[1] - a[3] + a[5] - a[7], a[2] - a[6], 2 * (a[3] - a[5]),
+                                  a[4], 2 * (a[5] - a[7]), 2 * a[6], 4 * a[7]};
+        for (int k = 0; k < P; ++k) w.pb[j][k] = (float)pb[k];
         // sum a_k T_k(v) -> monomials, T_{k+1} = 2 v T_k - T_{k-1}
         double Tm1[NCOEF] = {0}, T0[NCOEF] = {0}, mono[NCOEF] = {0};
         T0[0] = 1.0;
@@ -148,6 +155,7 @@ __global__ void wrap_nodes_f64(const double *in, double *out, long long total, d
 // list.  Uploaded on the plan's stream.
 int set_active_terms(Plan &p, const unsigned char *user_mask) {
     static thread_local std::vector<ActRec> recs, recs3;
+    static thread_local std::vector<unsigned char> stage;
     recs.clear();
     recs3.clear();
     int n = 0;
@@ -168,21 +176,25 @@ int set_active_terms(Plan &p, const unsigned char *user_mask) {
     p.n_items = 0;
     p.n_items3 = 0;
     if (n == 0) return ANOVA_OK;
-    bool order3 = false;
-    for (int i = 0; i < n; ++i) order3 = order3 || p.h_terms[p.h_act[i]].order == 3;
-    p.spread_K = spread_chunks_for(p.M, n, p.spread_kmax, p.max_grid_bytes, p.sm_count, p.cell_tc, order3);
+    int n3 = 0;
+    for (int i = 0; i < n; ++i) n3 += p.h_terms[p.h_act[i]].order == 3;
+    p.spread_K = spread_chunks_for(p.M, n, n3, p.spread_kmax, p.max_grid_bytes, p.grid_elems, p.sm_count,
+                                     p.cell_tc);
     if (p.h_items) {
         p.n_items3 = append_spread_items(p, 0, p.spread_K, p.h_items, 3);
         p.n_items = p.n_items3 + append_spread_items(p, 0, p.spread_K, p.h_items + p.n_items3, 0);
     }
-    cudaError_t e = cudaMemcpyAsync(p.act, p.h_act, sizeof(int) * n, cudaMemcpyHostToDevice, p.stream);
-    if (e == cudaSuccess)
-        e = cudaMemcpyAsync(p.act_rec, recs.data(), sizeof(ActRec) * n, cudaMemcpyHostToDevice, p.stream);
-    if (e == cudaSuccess && p.n_items)
-        e = cudaMemcpyAsync(p.items, p.h_items, sizeof(int4) * p.n_items, cudaMemcpyHostToDevice, p.stream);
-    if (e == cudaSuccess && p.n_act3 && p.act_rec3)
-        e = cudaMemcpyAsync(p.act_rec3, recs3.data(), sizeof(ActRec) * p.n_act3, cudaMemcpyHostToDevice, p.stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);   // recs is reused by the next call
+    // act, act_rec, act_rec3 and items adjoin: one copy, staged
+    unsigned char *base = (unsigned char *)p.act;
+    const size_t o1 = (unsigned char *)p.act_rec - base, o2 = (unsigned char *)p.act_rec3 - base,
+                 o3 = (unsigned char *)p.items - base, end = o3 + sizeof(int4) * p.n_items;
+    stage.resize(end);
+    std::memcpy(stage.data(), p.h_act, sizeof(int) * n);
+    std::memcpy(stage.data() + o1, recs.data(), sizeof(ActRec) * n);
+    if (p.n_act3) std::memcpy(stage.data() + o2, recs3.data(), sizeof(ActRec) * p.n_act3);
+    if (p.n_items) std::memcpy(stage.data() + o3, p.h_items, sizeof(int4) * p.n_items);
+    cudaError_t e = cudaMemcpyAsync(base, stage.data(), end, cudaMemcpyHostToDevice, p.stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);   // the staging is reused by the next call
     return cuda_status(e);
 }
 
@@ -210,6 +222,8 @@ DevPlan dev_view(const Plan &p) {
     v.partials = (float2 *)p.partials;
     v.spread_chunks = p.spread_K;
     v.srec = p.srec;
+    v.tile_cell = p.tile_cell;
+    v.tile_count = p.tile_count;
     v.facc = p.facc;
     v.fexp = p.fexp;
     v.n_coeffs = p.n_coeffs;
@@ -238,15 +252,40 @@ cudaError_t plan_malloc_raw(void **ptr, size_t bytes) {
     return cudaMalloc(ptr, bytes);
 }
 
+// Parts of one device allocation, each 256-byte aligned.  A part counts as an
+// allocation of its own for anova_debug_fail_allocation.
+struct Arena {
+    struct Part {
+        void **ptr;
+        size_t off;
+    };
+    std::vector<Part> parts;
+    size_t bytes = 0;
+    bool failed = false;
+    template <typename T>
+    void want(T **ptr, size_t n) {   // n = 0: *ptr stays null
+        if (n == 0) return;
+        failed = alloc_fault() || failed;
+        parts.push_back({(void **)ptr, bytes});
+        bytes = (bytes + n + 255) & ~(size_t)255;
+    }
+    cudaError_t commit(void **base) {
+        cudaError_t e = failed ? cudaErrorMemoryAllocation : cudaMalloc(base, bytes);
+        if (e != cudaSuccess) {
+            *base = nullptr;
+            return e;
+        }
+        for (const Part &q : parts) *q.ptr = (unsigned char *)*base + q.off;
+        return e;
+    }
+};
+
 static void free_plan(Plan &p) {
     profiler_free(p);
     if (p.solver && p.solver_free) p.solver_free(p.solver);
     p.solver = nullptr;
-    void *bufs[] = {p.x, p.terms, p.windows, p.deconv, p.deconvd, p.empty_off, p.grids, p.partials,
-                    p.err, p.scratch, p.act, p.act_rec, p.act_rec3, p.items, p.counter, p.srec, p.wt64, p.wb64, p.slots64,
-                    p.facc, p.fexp};
-    for (void *b : bufs)
-        if (b) cudaFree(b);
+    if (p.arena) cudaFree(p.arena);
+    if (p.arena_opt) cudaFree(p.arena_opt);
     delete[] p.h_terms;
     delete[] p.h_user_off;
     delete[] p.h_user_len;
@@ -528,26 +567,16 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
         p.n_slots64 = (int)slots64.size();
     }
 
-    // device allocations
+    // Device memory: the parts of one allocation (and a second for the optional
+    // sorted copies).  A plan's twenty cudaMalloc and cudaFree calls took 1.3 ms, two
+    // thirds of the life of a plan that evaluates 1e5 new nodes once.
     cudaError_t e = cudaSuccess;
     auto chk = [&](cudaError_t r) {
         if (r != cudaSuccess && e == cudaSuccess) e = r;
     };
-    size_t xbytes = (size_t)d * M * (p.precision == ANOVA_PREC_F64 ? 8 : 4);
-    if (xbytes) chk(plan_malloc(&p.x, xbytes));
-    chk(plan_malloc(&p.terms, sizeof(Term) * std::max(1, p.n_terms)));
-    chk(plan_malloc(&p.windows, sizeof(Window) * std::max<size_t>(1, wins.size())));
-    chk(plan_malloc(&p.deconv, sizeof(float) * std::max<size_t>(1, dec.size())));
-    chk(plan_malloc(&p.deconvd, sizeof(double) * std::max<size_t>(1, decd.size())));
-    chk(plan_malloc(&p.empty_off, sizeof(long long) * std::max<size_t>(1, empties.size())));
-    const size_t esize = p.precision == ANOVA_PREC_F64 ? 16 : (p.precision == ANOVA_PREC_F32 ? 8 : 4);   // bytes per grid element
-    chk(plan_malloc(&p.grids, (size_t)std::max<long long>(1, p.grid_elems) * esize));
-    chk(plan_malloc(&p.err, sizeof(int) * 4));
-    chk(plan_malloc(&p.act, sizeof(int) * std::max(1, p.n_terms)));
-    chk(plan_malloc(&p.act_rec, sizeof(ActRec) * std::max(1, p.n_terms)));
-    chk(plan_malloc(&p.act_rec3, sizeof(ActRec) * std::max(1, p.n_terms)));
-    p.h_act = plan_new<int>(std::max(1, p.n_terms));
-    if (!p.h_act && e == cudaSuccess) e = cudaErrorMemoryAllocation;
+    const bool f64 = p.precision == ANOVA_PREC_F64;
+    const size_t esize = f64 ? 16 : (p.precision == ANOVA_PREC_F32 ? 8 : 4);   // bytes per grid element
+    const size_t xbytes = (size_t)d * M * (f64 ? 8 : 4), nt1 = (size_t)std::max(1, p.n_terms);
     // adjoint partial grids: one per node chunk of a term (work items of the
     // spread are (term, chunk) pairs), bounded to 8 GB
     long long k_cap = std::max<long long>(1, (8LL << 30) / std::max<long long>(1, p.grid_elems * 8));
@@ -557,86 +586,123 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
     p.spread_kmax = kmax;
     p.gather_ctas = (int)std::min<long long>((long long)p.sm_count,
                                              std::max<long long>(1, (M + GATHER_TILE - 1) / GATHER_TILE));
-    if (e == cudaSuccess && p.n_terms > 0)
-        chk(plan_malloc(&p.partials, (size_t)kmax * (size_t)p.grid_elems * esize));
-    chk(plan_malloc(&p.items, sizeof(int4) * (size_t)std::max(1, p.n_terms) * kmax));
-    chk(plan_malloc(&p.counter, 2 * sizeof(int)));
-    p.h_items = plan_new<int4>((size_t)std::max(1, p.n_terms) * kmax);
-    if (!p.h_items && e == cudaSuccess) e = cudaErrorMemoryAllocation;
     // partial sums: one double per term, or 256 complex ones
     p.scratch_bytes = std::max<size_t>(1 << 20, sizeof(double) * p.n_terms);
-    chk(plan_malloc(&p.scratch, p.scratch_bytes));
-    if (p.n_slots64 > 0 && M > 0) {
-        chk(plan_malloc(&p.slots64, sizeof(int4) * p.n_slots64));
-        chk(plan_malloc(&p.wt64, sizeof(double) * 8 * (size_t)p.n_slots64 * M));
-        chk(plan_malloc(&p.wb64, sizeof(int) * (size_t)p.n_slots64 * M));
-        if (e == cudaSuccess)
-            chk(cudaMemcpyAsync(p.slots64, slots64.data(), sizeof(int4) * p.n_slots64, cudaMemcpyHostToDevice,
-                                p.stream));
+    Arena mem;
+    mem.want(&p.terms, sizeof(Term) * nt1);
+    mem.want(&p.windows, sizeof(Window) * std::max<size_t>(1, wins.size()));
+    mem.want(&p.deconv, sizeof(float) * std::max<size_t>(1, dec.size()));
+    mem.want(&p.deconvd, sizeof(double) * std::max<size_t>(1, decd.size()));
+    mem.want(&p.empty_off, sizeof(long long) * std::max<size_t>(1, empties.size()));
+    mem.want(&p.slots64, sizeof(int4) * slots64.size());
+    const size_t table_bytes = mem.bytes;
+    mem.want(&p.act, sizeof(int) * nt1);
+    mem.want(&p.act_rec, sizeof(ActRec) * nt1);
+    mem.want(&p.act_rec3, sizeof(ActRec) * nt1);
+    mem.want(&p.items, sizeof(int4) * nt1 * kmax);
+    mem.want(&p.err, sizeof(int) * 4);
+    mem.want(&p.counter, 2 * sizeof(int));
+    mem.want(&p.x, xbytes);
+    mem.want(&p.grids, (size_t)std::max<long long>(1, p.grid_elems) * esize);
+    mem.want(&p.scratch, p.scratch_bytes);
+    mem.want(&p.partials, p.n_terms > 0 ? (size_t)kmax * (size_t)p.grid_elems * esize : 0);
+    if (M > 0) {
+        mem.want(&p.wt64, sizeof(double) * 8 * (size_t)p.n_slots64 * M);
+        mem.want(&p.wb64, sizeof(int) * (size_t)p.n_slots64 * M);
     }
-    // cell-sorted node records (16 bytes per node for a term of order <= 2, 32
-    // for order 3; FP64 plans sort order <= 2 only), if they fit in half the
-    // free device memory.  sort_slot counts units of M records of 16 bytes.
-    if (e == cudaSuccess && o.node_sort >= 0 && M > 0) {
-        auto units = [&](const Term &T) { return T.order <= 2 ? 1 : (p.precision == ANOVA_PREC_F64 ? 0 : 2); };
-        int ns = 0;
-        for (int s = 0; s < p.n_terms; ++s) ns += units(p.h_terms[s]);
-        size_t free_b = 0, total_b = 0;
-        const size_t need = (size_t)ns * (size_t)M * sizeof(float4);
-        if (ns > 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need <= free_b / 2) {
-            if (plan_malloc(&p.srec, need) == cudaSuccess) {
-                int slot = 0;
-                for (int s = 0; s < p.n_terms; ++s) {
-                    const int u = units(p.h_terms[s]);
-                    if (u) {
-                        p.h_terms[s].sort_slot = slot;
-                        slot += u;
-                    }
-                }
-                p.n_sorted = ns;
-                p.cell_tc = p.precision != ANOVA_PREC_F64 && o.cell_kernel == 0;
-                if (p.precision == ANOVA_PREC_F32) {
-                    if (plan_malloc(&p.facc, sizeof(unsigned long long) * 2 * (size_t)M) != cudaSuccess ||
-                        plan_malloc(&p.fexp, sizeof(int) * 4) != cudaSuccess) {
-                        cudaGetLastError();   // the forward falls back to the point-major gather
-                        if (p.facc) cudaFree(p.facc);
-                        if (p.fexp) cudaFree(p.fexp);
-                        p.facc = nullptr;
-                        p.fexp = nullptr;
-                    }
-                }
-            } else {
-                cudaGetLastError();
-                p.srec = nullptr;
-            }
-        }
-    }
+    p.h_act = plan_new<int>(nt1);
+    p.h_items = plan_new<int4>(nt1 * kmax);
+    if (!p.h_act || !p.h_items) return ANOVA_ERR_NOMEM;
+    e = mem.commit(&p.arena);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return cuda_status(e);
     }
-    chk(cudaMemcpyAsync(p.terms, p.h_terms, sizeof(Term) * p.n_terms, cudaMemcpyHostToDevice, p.stream));
-    if (!wins.empty())
-        chk(cudaMemcpyAsync(p.windows, wins.data(), sizeof(Window) * wins.size(), cudaMemcpyHostToDevice,
-                            p.stream));
-    if (!dec.empty()) {
-        chk(cudaMemcpyAsync(p.deconv, dec.data(), sizeof(float) * dec.size(), cudaMemcpyHostToDevice, p.stream));
-        chk(cudaMemcpyAsync(p.deconvd, decd.data(), sizeof(double) * decd.size(), cudaMemcpyHostToDevice,
-                            p.stream));
+    // cell-sorted node copies, if they fit in half the free device memory: node
+    // tiles (tiles.cuh) for the tensor-core kernels, else records of 16 bytes per
+    // node (32 for order 3; FP64 plans sort order <= 2 only), whose sort_slot
+    // counts units of M records of 16 bytes
+    if (o.node_sort >= 0 && M > 0 && p.n_terms > 0) {
+        const bool tiles = !f64 && o.cell_kernel == 0;
+        long long n_rec = 0, n_tiles = 0;   // float4 records, tiles
+        std::vector<int> slot(p.n_terms, -1);
+        for (int s = 0; s < p.n_terms; ++s) {
+            Term &T = p.h_terms[s];
+            if (tiles) {
+                long long cells = T.n;
+                for (int j = 1; j < T.order; ++j) cells *= T.n;
+                const long long cap = tile_capacity(M, cells);
+                T.rec_off = n_rec;
+                T.tile_off = n_tiles;
+                slot[s] = s;
+                n_rec += cap * tile_f4(T.order);
+                n_tiles += cap;
+            } else {
+                const int u = T.order <= 2 ? 1 : (f64 ? 0 : 2);
+                if (u) slot[s] = (int)(n_rec / M);
+                n_rec += (long long)u * M;
+            }
+        }
+        if (tiles) {
+            n_rec += TILE_SLACK * tile_f4(3);
+            n_tiles += TILE_SLACK;
+        }
+        size_t free_b = 0, total_b = 0;
+        const size_t need = (size_t)n_rec * sizeof(float4) + (size_t)n_tiles * sizeof(int);
+        if (n_rec > 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need <= free_b / 2) {
+            auto sorted_parts = [&](Arena &A) {
+                A.want(&p.srec, (size_t)n_rec * sizeof(float4));
+                A.want(&p.tile_cell, (size_t)n_tiles * sizeof(int));
+                A.want(&p.tile_count, tiles ? sizeof(int) * p.n_terms : 0);
+            };
+            Arena opt;
+            sorted_parts(opt);
+            bool ok = !opt.failed, acc = p.precision == ANOVA_PREC_F32;
+            if (ok && acc) {
+                opt.want(&p.facc, sizeof(unsigned long long) * 2 * (size_t)M);
+                opt.want(&p.fexp, sizeof(int) * 4);
+                if (opt.failed || opt.commit(&p.arena_opt) != cudaSuccess) acc = false;
+            }
+            if (ok && !acc) {   // without accumulators the forward is the point-major gather
+                cudaGetLastError();
+                p.facc = nullptr;
+                p.fexp = nullptr;
+                Arena only;
+                sorted_parts(only);
+                ok = !only.failed && only.commit(&p.arena_opt) == cudaSuccess;
+            }
+            if (ok) {
+                for (int s = 0; s < p.n_terms; ++s) p.h_terms[s].sort_slot = slot[s];
+                p.n_sorted = tiles ? p.n_terms : (int)(n_rec / M);
+                p.cell_tc = tiles;
+            } else {
+                cudaGetLastError();
+                p.srec = nullptr;
+                p.tile_cell = p.tile_count = nullptr;
+            }
+        }
     }
-    if (!empties.empty())
-        chk(cudaMemcpyAsync(p.empty_off, empties.data(), sizeof(long long) * empties.size(),
-                            cudaMemcpyHostToDevice, p.stream));
-    chk(cudaMemsetAsync(p.err, 0, sizeof(int) * 4, p.stream));
-    chk(cudaMemsetAsync(p.counter, 0, 2 * sizeof(int), p.stream));
-    if (p.facc) {
-        chk(cudaMemsetAsync(p.facc, 0, sizeof(unsigned long long) * 2 * (size_t)M, p.stream));
-        chk(cudaMemsetAsync(p.fexp, 0, sizeof(int) * 4, p.stream));
+    {   // the tables in one copy
+        std::vector<unsigned char> host(table_bytes);
+        auto put = [&](const void *dev, const void *src, size_t bytes) {
+            if (bytes) std::memcpy(host.data() + ((const unsigned char *)dev - (const unsigned char *)p.arena), src, bytes);
+        };
+        put(p.terms, p.h_terms, sizeof(Term) * p.n_terms);
+        put(p.windows, wins.data(), sizeof(Window) * wins.size());
+        put(p.deconv, dec.data(), sizeof(float) * dec.size());
+        put(p.deconvd, decd.data(), sizeof(double) * decd.size());
+        put(p.empty_off, empties.data(), sizeof(long long) * empties.size());
+        put(p.slots64, slots64.data(), sizeof(int4) * slots64.size());
+        chk(cudaMemcpyAsync(p.arena, host.data(), table_bytes, cudaMemcpyHostToDevice, p.stream));
+        chk(cudaStreamSynchronize(p.stream));   // `host` leaves scope
     }
+    // counter and error words, and the accumulators and their exponent, adjoin
+    chk(cudaMemsetAsync(p.err, 0, (char *)(p.counter + 2) - (char *)p.err, p.stream));
+    if (p.facc) chk(cudaMemsetAsync(p.facc, 0, (char *)(p.fexp + 4) - (char *)p.facc, p.stream));
     if (xbytes) {
         long long total = (long long)d * M;
         int blocks = (int)std::min<long long>(4096, (total + 255) / 256);
-        if (p.precision == ANOVA_PREC_F64)
+        if (f64)
             wrap_nodes_f64<<<blocks, 256, 0, p.stream>>>((const double *)x_dev, (double *)p.x, total,
                                                           cosine ? 0.5 : 1.0);
         else

@@ -15,6 +15,7 @@
 
 #include "device.cuh"
 #include "internal.cuh"
+#include "tiles.cuh"
 
 namespace agft {
 
@@ -170,8 +171,226 @@ __global__ void k_cell_scatter64(const Term *terms, const int *wb, long long M, 
     }
 }
 
+// ---- node tiles (tiles.cuh) ----
+//
+// A counting sort per term with the node range cut into S slices, one block
+// each.  The blocks' histograms are kept, and the scan turns them into every
+// block's first place in every cell, so that the scatter counts in shared memory
+// only.  Scattered writes are what bounds it: they run at DRAM speed in partial
+// sectors once the terms in work outgrow L2.  So for order <= 2 the scatter writes
+// only the 4-byte indices (a third of the tiles' sectors; big blocks keep few terms
+// in work) and a second pass, in tile order, reads the coordinates through L2 and
+// writes whole lines.
+constexpr int SORT_THREADS = 512;
+
+__device__ __forceinline__ int tile_bin(const Term &T, int fr, int fr1, int fc) {
+    return T.order == 3 ? (fr1 * T.n + fc) * T.n + fr : (T.order == 2 ? fr * T.n + fc : fc);
+}
+
+// hist[(term S + slice) max_bins + cell] = nodes of the slice in the cell
+__global__ void __launch_bounds__(SORT_THREADS)
+k_tile_count(const Term *terms, const float *x, long long M, int *hist, int max_bins) {
+    extern __shared__ int bins[];
+    const Term &T = terms[blockIdx.y];
+    const int nb = cell_bins(T), S = gridDim.x, n = T.n, order = T.order;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) bins[b] = 0;
+    __syncthreads();
+    const float *xr = x + (long long)(order >= 2 ? T.row0 : T.col) * M;
+    const float *xr1 = x + (long long)(order == 3 ? T.row1 : T.col) * M;
+    const float *xc = x + (long long)T.col * M;
+    const long long j1 = M * (blockIdx.x + 1) / S;
+    for (long long j = M * blockIdx.x / S + threadIdx.x; j < j1; j += blockDim.x) {
+        float t;
+        const int fc = grid_pos(xc[j], n, t);
+        const int fr = order >= 2 ? grid_pos(xr[j], n, t) : 0, fr1 = order == 3 ? grid_pos(xr1[j], n, t) : 0;
+        atomicAdd(&bins[tile_bin(T, fr, fr1, fc)], 1);
+    }
+    __syncthreads();
+    int *out = hist + ((long long)blockIdx.y * S + blockIdx.x) * max_bins;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) out[b] = bins[b];
+}
+
+constexpr int SORT_MAX_SLICES = 16;
+
+// One block per term: first places of every slice in every cell (in place of the
+// histograms), (first tile, nodes) of every cell and the number of tiles.
+__global__ void __launch_bounds__(1024) k_tile_scan(const Term *terms, int *hist, int S, int max_bins, int2 *cell_info,
+                                                    int *tile_count) {
+    __shared__ int wsum[32];
+    const Term &T = terms[blockIdx.x];
+    const int nb = cell_bins(T);
+    int *h = hist + (long long)blockIdx.x * S * max_bins;
+    int2 *info = cell_info + (long long)blockIdx.x * max_bins;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    int carry = 0;
+    for (int b0 = 0; b0 < nb; b0 += blockDim.x) {
+        const int b = b0 + threadIdx.x;
+        int k[SORT_MAX_SLICES], count = 0;
+#pragma unroll
+        for (int s = 0; s < SORT_MAX_SLICES; ++s) k[s] = s < S && b < nb ? h[(long long)s * max_bins + b] : 0;
+#pragma unroll
+        for (int s = 0; s < SORT_MAX_SLICES; ++s) count += k[s];
+        const int tiles = (count + TILE - 1) / TILE;
+        int v = tiles;   // inclusive scan across the block
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += u;
+        }
+        if (lane == 31) wsum[wid] = v;
+        __syncthreads();
+        if (wid == 0) {
+            int w = wsum[lane];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, w, o);
+                if (lane >= o) w += u;
+            }
+            wsum[lane] = w;
+        }
+        __syncthreads();
+        const int tile0 = carry + v - tiles + (wid > 0 ? wsum[wid - 1] : 0);
+        carry += wsum[31];
+        __syncthreads();   // wsum is read before the next round
+        if (b >= nb) continue;
+        info[b] = make_int2(tile0, count);
+        int place = tile0 * TILE;
+#pragma unroll
+        for (int s = 0; s < SORT_MAX_SLICES; ++s) {
+            if (s < S) h[(long long)s * max_bins + b] = place;
+            place += k[s];
+        }
+    }
+    if (threadIdx.x == 0) tile_count[blockIdx.x] = carry;
+}
+
+// the slice's nodes to their places (order <= 2: the indices); each block also
+// writes the tiles' cells and the padding of its share of the term's cells
+__global__ void __launch_bounds__(SORT_THREADS)
+k_tile_scatter(const Term *terms, const float *x, long long M, const int *hist, const int2 *cell_info, int max_bins,
+               float4 *srec, int *tile_cell) {
+    extern __shared__ int bins[];
+    const Term &T = terms[blockIdx.y];
+    const int nb = cell_bins(T), S = gridDim.x, n = T.n, order = T.order;
+    const int *in = hist + ((long long)blockIdx.y * S + blockIdx.x) * max_bins;
+    for (int b = threadIdx.x; b < nb; b += blockDim.x) bins[b] = in[b];
+    __syncthreads();
+    const float *xr = x + (long long)(order >= 2 ? T.row0 : T.col) * M;
+    const float *xr1 = x + (long long)(order == 3 ? T.row1 : T.col) * M;
+    const float *xc = x + (long long)T.col * M;
+    float4 *rec = srec + T.rec_off;
+    const long long j1 = M * (blockIdx.x + 1) / S;
+    auto index_at = [&](int pos) -> int & {   // node number pos of a term of order <= 2
+        return ((int *)(rec + (long long)(pos >> 4) * tile_f4(2) + 8))[(pos & 7) * 2 + ((pos >> 3) & 1)];
+    };
+    for (long long j = M * blockIdx.x / S + threadIdx.x; j < j1; j += blockDim.x) {
+        float tc, tr, tr1;
+        const int fc = grid_pos(xc[j], n, tc);
+        const int fr = order >= 2 ? grid_pos(xr[j], n, tr) : 0, fr1 = order == 3 ? grid_pos(xr1[j], n, tr1) : 0;
+        const int pos = atomicAdd(&bins[tile_bin(T, fr, fr1, fc)], 1);
+        if (order == 3)
+            rec[pos] = make_float4(2.f * tr - 1.f, 2.f * tr1 - 1.f, 2.f * tc - 1.f, __int_as_float((int)j));
+        else
+            index_at(pos) = (int)j;
+    }
+    int *cells = tile_cell + T.tile_off;
+    const int2 *info = cell_info + (long long)blockIdx.y * max_bins;
+    const int b1 = (int)((long long)nb * (blockIdx.x + 1) / S);
+    for (int b = (int)((long long)nb * blockIdx.x / S) + threadIdx.x; b < b1; b += blockDim.x) {
+        const int2 c = info[b];   // first tile, nodes
+        int cell = b;
+        if (order == 2) cell = b / n * T.stride + b % n;
+        if (order == 3) cell = b % n | b / (n * n) << 8 | b / n % n << 16;   // a, b, c
+        for (int i = 0; i * TILE < c.y; ++i) cells[c.x + i] = cell | (c.y - i * TILE <= TILE / 2 ? TILE_HALF : 0);
+        for (int k = c.y; k % TILE; ++k) {
+            if (order == 3)
+                rec[c.x * TILE + k] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
+            else
+                index_at(c.x * TILE + k) = -1;
+        }
+    }
+}
+
+// order <= 2: the window arguments of the tiles' nodes, a lane per node and two
+// tiles per warp; lane p < 8 of a tile writes the pair (p, p + 8)
+__global__ void __launch_bounds__(256) k_tile_fill(const Term *terms, const float *__restrict__ x, long long M,
+                                                   float4 *srec, const int *tile_count) {
+    const Term &T = terms[blockIdx.y];
+    if (T.order == 3) return;
+    const int nt = tile_count[blockIdx.y], n = T.n, lane = threadIdx.x & 31, p = lane & 15;
+    const bool two = T.order == 2;
+    const float *xr = x + (long long)(two ? T.row0 : T.col) * M, *xc = x + (long long)T.col * M;
+    float4 *rec = srec + T.rec_off;
+    const int warps = gridDim.x * (blockDim.x >> 5);
+    for (int i0 = 2 * (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)); i0 < nt; i0 += 2 * warps) {
+        const int i = i0 + (lane >> 4);
+        float4 *tile = rec + (long long)i * tile_f4(2);
+        const int j = i < nt ? ((const int *)(tile + 8))[(p & 7) * 2 + (p >> 3)] : -1;
+        float vr = 0.f, vc = 0.f;
+        if (j >= 0) {
+            float t;
+            grid_pos(xc[j], n, t);
+            vc = 2.f * t - 1.f;
+            if (two) {
+                grid_pos(xr[j], n, t);
+                vr = 2.f * t - 1.f;
+            }
+        }
+        const float vr8 = __shfl_down_sync(0xffffffffu, vr, 8), vc8 = __shfl_down_sync(0xffffffffu, vc, 8);
+        if (p < 8 && i < nt) tile[p] = make_float4(vr, vr8, vc, vc8);
+    }
+}
+
+static int sort_tiles(Plan &p) {
+    int max_bins = 1;
+    for (int s = 0; s < p.n_terms; ++s) {
+        const Term &T = p.h_terms[s];
+        max_bins = std::max(max_bins, T.order == 3 ? T.n * T.n * T.n : (T.order == 2 ? T.n * T.n : T.n));
+    }
+    // slices of at least 16384 nodes (a block also moves a histogram)
+    const int S = (int)std::max<long long>(1, std::min<long long>(SORT_MAX_SLICES, p.M / 16384));
+    const size_t n_bins = (size_t)p.n_terms * max_bins;
+    // (first tile, nodes) per cell, then the slices' histograms: in the partial
+    // grids, which hold nothing yet, where they fit
+    int2 *info = nullptr, *own = nullptr;
+    const size_t need = sizeof(int2) * n_bins + sizeof(int) * n_bins * S;
+    cudaError_t e = cudaSuccess;
+    if (need <= (size_t)p.spread_kmax * (size_t)p.grid_elems * (p.precision == ANOVA_PREC_F32 ? 8 : 4)) {
+        info = (int2 *)p.partials;
+    } else {
+        e = plan_malloc(&own, need);
+        if (e != cudaSuccess) return cuda_status(e);
+        info = own;
+    }
+    const size_t bytes = sizeof(int) * (size_t)max_bins;
+    if (bytes > 48 * 1024) {
+        e = cudaFuncSetAttribute(k_tile_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_tile_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    }
+    if (e == cudaSuccess) {
+        const dim3 grid(S, p.n_terms);
+        const float *x = (const float *)p.x;
+        int *hist = (int *)(info + n_bins);
+        k_tile_count<<<grid, SORT_THREADS, bytes, p.stream>>>(p.terms, x, p.M, hist, max_bins);
+        k_tile_scan<<<p.n_terms, 1024, 0, p.stream>>>(p.terms, hist, S, max_bins, info, p.tile_count);
+        k_tile_scatter<<<grid, SORT_THREADS, bytes, p.stream>>>(p.terms, x, p.M, hist, info, max_bins, p.srec,
+                                                                p.tile_cell);
+        // about 16 steps per warp
+        const int fb = (int)std::max<long long>(1, std::min<long long>(256, p.M / 4096));
+        k_tile_fill<<<dim3(fb, p.n_terms), 256, 0, p.stream>>>(p.terms, x, p.M, p.srec, p.tile_count);
+        e = cudaGetLastError();
+    }
+    if (own) {
+        if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);
+        cudaFree(own);
+    }
+    return cuda_status(e);
+}
+
 int sort_nodes_by_cell(Plan &p) {
     if (!p.srec || p.n_sorted == 0 || p.M == 0) return ANOVA_OK;
+    if (p.cell_tc) return sort_tiles(p);
     int max_bins = 1;
     for (int s = 0; s < p.n_terms; ++s) {
         const Term &T = p.h_terms[s];

@@ -888,6 +888,7 @@ int adjoint_launch(Plan *prof, cudaStream_t st, const DevPlan &v, const BatchArg
 }
 
 int launch_adjoint_f32(Plan &p, const float2 *y, float2 *fhat) {
+    if (p.direct) return launch_direct_adjoint(p, y, fhat);
     DevPlan v = dev_view(p);
     BatchArgs B;
     std::memset(&B, 0, sizeof(B));

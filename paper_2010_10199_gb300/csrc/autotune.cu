@@ -145,7 +145,7 @@ int anova_plan_autotune(anova_plan_options *opts, int d, int64_t M, const void *
     ro.window_m_row = 4;
     ro.eps = 1e-8;
     anova_plan_t ref = nullptr;
-    int rc = anova_plan_create(&ref, d, M, x_dev, n_terms, term_dims, bandwidth, &ro, stream);
+    int rc = plan_create(&ref, d, M, x_dev, n_terms, term_dims, bandwidth, &ro, stream, false);
     if (rc) return rc;
     const long long n = anova_num_coeffs(ref);
     TuneBuffers T;
@@ -200,7 +200,7 @@ int anova_plan_autotune(anova_plan_options *opts, int d, int64_t M, const void *
     auto trial = [&](const anova_plan_options &o) -> int {
         Cand c{o, INFINITY, INFINITY, false};
         anova_plan_t p = nullptr;
-        int r = anova_plan_create(&p, d, M, x_dev, n_terms, term_dims, bandwidth, &o, stream);
+        int r = plan_create(&p, d, M, x_dev, n_terms, term_dims, bandwidth, &o, stream, false);
         if (r == ANOVA_ERR_UNSUPPORTED || r == ANOVA_ERR_NOMEM) {
             cudaGetLastError();
             done.push_back(c);   // not buildable: recorded, never chosen

@@ -253,7 +253,7 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
             return ANOVA_ERR_INVALID;
         }
         anova_plan_t h = nullptr;
-        int rc = anova_plan_create(&h, d[p], M[p], x_dev[p], n_terms[p], term_dims[p], bandwidth[p], &o, stream);
+        int rc = plan_create(&h, d[p], M[p], x_dev[p], n_terms[p], term_dims[p], bandwidth[p], &o, stream, false);
         if (rc) {
             free_batch(b);
             return rc;

@@ -115,6 +115,19 @@ inline ActRec make_act_rec(const Term &T, int term, int newgroup) {
 //   w (int bits): the node's original index.
 // Built in sort.cu by the same FP32 operations the unsorted kernels apply.
 
+// Direct summation (direct.cu): a term as its kernels need it, and an adjoint item.
+struct DirectTerm {
+    int order, K;            // K: frequencies per axis
+    int col, row0, row1;
+    int coef_off;
+    int group, pad;          // frequency or row group of the unit
+};
+struct DirectItem {
+    int act, chunk, chunks, pad;   // active term (-1: the empty set), node chunk of chunks
+    DirectTerm term;
+};
+constexpr int DA_MAX_ACC = 192;                // partial sums of an adjoint item
+
 // Device-visible view of a plan (passed by value to kernels).
 struct DevPlan {
     int d;
@@ -123,6 +136,7 @@ struct DevPlan {
     int n_empty;              // empty-set terms
     const float *x;           // [d][M] FP32 nodes (or null)
     const double *xd;         // [d][M] FP64 nodes (or null)
+    const float2 *z;          // [d][M] exp(2 pi i x), plans summed directly (or null)
     const Term *terms;
     const Window *windows;
     const float *deconv;      // deconvolution factors
@@ -226,6 +240,19 @@ struct Plan {
     int n_sorted;
     unsigned long long *facc;   // sorted forward: fixed-point accumulators [M][2]
     int *fexp;              // and their exponent
+    // plans of small bandwidths, summed directly (direct.cu)
+    bool direct;
+    float2 *z;              // [d][M] exp(2 pi i x)
+    float *direct_part;     // partial sums of the adjoint's items
+    int *direct_count;      // finished blocks per active term and of the empty set, zero between calls
+    int direct_kt;          // powers per coordinate of the forward's table
+    int direct_npl, direct_split;   // forward: nodes per lane, sets of terms per node block
+    float2 *direct_fpart;   // their sums [direct_split][M] (one set: null), finished CTAs per node block
+    int *direct_fcount;
+    bool direct_big;        // adjoint: the kernel for many sums per item
+    DirectTerm *direct_units, *h_units;    // forward work units of the active terms
+    DirectItem *direct_items, *h_ditems;   // adjoint work items (n_items of them)
+    int n_direct_units;
     // FP64 plans: window weights per (window, coordinate) slot and node, the
     // precomputed form of psi (taps 0..2m-1, zero padded to 8), and the first
     // tap's grid index floor(n x + n/2) in [0, n)
@@ -298,6 +325,31 @@ size_t spread_smem_bytes(long long max_grid_bytes, bool o3, int sp);
 int spread_block_nodes(long long max_grid_bytes);
 // Sorts the nodes by grid cell for every term with sort_slot >= 0 (sort.cu).
 int sort_nodes_by_cell(Plan &p);
+// Direct summation (direct.cu).
+constexpr int DIRECT_MAX_SMEM = 100 * 1024;   // forward: two CTAs per SM
+constexpr int DIRECT_MAX_CHUNKS = 64, DIRECT_MAX_BLOCKS = 8192;   // adjoint
+constexpr int DIRECT_RESIDENT = 4, DIRECT_RESIDENT_BIG = 2;       // its blocks per SM
+constexpr int DIRECT_MAX_SPLITS = 16;         // forward: sets of terms per node block
+constexpr double DIRECT_FIXED_NS = 8400.0, NFFT_FIXED_NS = 33000.0;   // launches and latencies of a transform
+bool direct_term(const Term &T);
+double direct_term_ns(const Term &T, long long M);
+double nfft_term_ns(const Term &T, long long M);
+size_t direct_smem(int d, int kt, int npl, bool cosine);
+int direct_npl(int d, int kt, long long M, bool cosine);
+int direct_splits(long long n_units, long long M, int npl, int sm_count);
+inline long long direct_max_chunks(long long M) { return std::min<long long>(DIRECT_MAX_CHUNKS, std::max<long long>(1, M / 256)); }
+int direct_unit_list(const Plan &p, DirectTerm *out);
+bool direct_big(const Term &T);
+int direct_axis(const Term &T);
+int direct_groups(const Term &T);
+int direct_items(const Plan &p, DirectItem *out);
+int build_unit_table(Plan &p);
+int launch_direct_trafo(Plan &p, const float2 *fhat, float2 *f);
+int launch_direct_adjoint(Plan &p, const float2 *y, float2 *fhat);
+// anova_plan_create; allow_direct: small bandwidths may be summed directly (a batch's
+// kernels and the tuner's candidates need the NFFT)
+int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
+                const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct);
 // FP64 path (f64.cu): window tables, forward and adjoint transforms.
 int build_window_tables_f64(Plan &p);
 int launch_trafo_f64(Plan &p, const double2 *fhat, double2 *f);

@@ -175,24 +175,41 @@ int set_active_terms(Plan &p, const unsigned char *user_mask) {
     p.n_act3 = (int)recs3.size();
     p.n_items = 0;
     p.n_items3 = 0;
-    if (n == 0) return ANOVA_OK;
+    if (p.direct) {
+        p.n_items = direct_items(p, p.h_ditems);
+        p.n_direct_units = direct_unit_list(p, p.h_units);
+    } else if (n == 0) {
+        return ANOVA_OK;
+    }
     int n3 = 0;
     for (int i = 0; i < n; ++i) n3 += p.h_terms[p.h_act[i]].order == 3;
-    p.spread_K = spread_chunks_for(p.M, n, n3, p.spread_kmax, p.max_grid_bytes, p.grid_elems, p.sm_count,
+    if (!p.direct) p.spread_K = spread_chunks_for(p.M, n, n3, p.spread_kmax, p.max_grid_bytes, p.grid_elems, p.sm_count,
                                      p.cell_tc);
-    if (p.h_items) {
+    if (p.h_items && !p.direct) {
         p.n_items3 = append_spread_items(p, 0, p.spread_K, p.h_items, 3);
         p.n_items = p.n_items3 + append_spread_items(p, 0, p.spread_K, p.h_items + p.n_items3, 0);
     }
-    // act, act_rec, act_rec3 and items adjoin: one copy, staged
+    // act, act_rec, act_rec3 and items (summed directly: units and items) adjoin: one
+    // copy, staged
     unsigned char *base = (unsigned char *)p.act;
-    const size_t o1 = (unsigned char *)p.act_rec - base, o2 = (unsigned char *)p.act_rec3 - base,
-                 o3 = (unsigned char *)p.items - base, end = o3 + sizeof(int4) * p.n_items;
-    stage.resize(end);
-    std::memcpy(stage.data(), p.h_act, sizeof(int) * n);
-    std::memcpy(stage.data() + o1, recs.data(), sizeof(ActRec) * n);
-    if (p.n_act3) std::memcpy(stage.data() + o2, recs3.data(), sizeof(ActRec) * p.n_act3);
-    if (p.n_items) std::memcpy(stage.data() + o3, p.h_items, sizeof(int4) * p.n_items);
+    size_t end = 0;
+    auto put = [&](const void *dev, const void *src, size_t bytes) {
+        if (bytes == 0) return;
+        const size_t at = (const unsigned char *)dev - base;
+        end = std::max(end, at + bytes);
+        if (stage.size() < end) stage.resize(end);
+        std::memcpy(stage.data() + at, src, bytes);
+    };
+    put(p.act, p.h_act, sizeof(int) * n);
+    put(p.act_rec, recs.data(), sizeof(ActRec) * n);
+    put(p.act_rec3, recs3.data(), sizeof(ActRec) * p.n_act3);
+    if (p.direct) {
+        put(p.direct_units, p.h_units, sizeof(DirectTerm) * p.n_direct_units);
+        put(p.direct_items, p.h_ditems, sizeof(DirectItem) * p.n_items);
+    } else {
+        put(p.items, p.h_items, sizeof(int4) * p.n_items);
+    }
+    if (end == 0) return ANOVA_OK;
     cudaError_t e = cudaMemcpyAsync(base, stage.data(), end, cudaMemcpyHostToDevice, p.stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);   // the staging is reused by the next call
     return cuda_status(e);
@@ -206,6 +223,7 @@ DevPlan dev_view(const Plan &p) {
     v.n_empty = p.n_empty;
     v.x = p.precision == ANOVA_PREC_F64 ? nullptr : (const float *)p.x;
     v.xd = p.precision == ANOVA_PREC_F64 ? (const double *)p.x : nullptr;
+    v.z = p.z;
     v.terms = p.terms;
     v.windows = p.windows;
     v.deconv = p.deconv;
@@ -295,6 +313,8 @@ static void free_plan(Plan &p) {
     delete[] p.h_user_order;
     delete[] p.h_act;
     delete[] p.h_items;
+    delete[] p.h_units;
+    delete[] p.h_ditems;
 }
 
 }  // namespace agft
@@ -319,9 +339,10 @@ const char *anova_status_string(int s) {
 
 const char *anova_version(void) { return "anova-gft 0.1 (sm_103a)"; }
 
-static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms,
-                       const int32_t *term_dims, const int32_t *bandwidth, const anova_plan_options *opts,
-                       void *stream) {
+}  // extern "C"
+
+static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
+                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct) {
     if (!out) return ANOVA_ERR_INVALID;
     *out = nullptr;
     cudaGetLastError();   // do not report an earlier, unrelated error
@@ -583,6 +604,34 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
     int kmax = (int)std::min<long long>(std::min<long long>(SPREAD_MAX_K, k_cap),
                                         std::max<long long>(1, (M + 2047) / 2048));
     if (o.n_ctas > 0) kmax = std::min(o.n_ctas, SPREAD_MAX_K);
+    // small bandwidths in every term: the sums themselves, where they are faster
+    // (default options only: the others ask for a path of the NFFT)
+    long long d_groups = p.n_empty > 0 ? 1 : 0, d_units = 0;
+    if (allow_direct && p.precision == ANOVA_PREC_F32 && o.node_sort == 0 && o.cell_kernel == 0 &&
+        o.n_ctas <= 0 && M > 0 && p.n_terms > 0) {
+        double t_direct = DIRECT_FIXED_NS, t_nfft = NFFT_FIXED_NS;
+        p.direct = true;
+        for (int s = 0; s < p.n_terms && p.direct; ++s) {
+            const Term &T = p.h_terms[s];
+            p.direct = direct_term(T);
+            t_direct += direct_term_ns(T, M);
+            t_nfft += nfft_term_ns(T, M);
+            d_groups += direct_groups(T);
+            d_units += T.order == 1 ? direct_groups(T) : 1;
+            p.direct_big = p.direct_big || direct_big(T);
+            if (T.order > 1) p.direct_kt = std::max(p.direct_kt, direct_axis(T));
+        }
+        p.direct = p.direct && t_direct < t_nfft && direct_smem(d, p.direct_kt, 1, cosine) <= DIRECT_MAX_SMEM;
+    }
+    if (p.direct) {
+        p.direct_npl = direct_npl(d, p.direct_kt, M, cosine);
+        p.direct_split = direct_splits(d_units, M, p.direct_npl, p.sm_count);
+    }
+    const size_t f_blocks = p.direct ? (size_t)((M + 32 * p.direct_npl - 1) / (32 * p.direct_npl)) : 0;
+    if (p.direct) kmax = 1;
+    const size_t n_ditems = p.direct ? (size_t)std::max(d_groups, std::min<long long>(DIRECT_MAX_BLOCKS, d_groups * direct_max_chunks(M)))
+                                     : 0;
+    const size_t n_items = p.direct ? 1 : nt1 * kmax;
     p.spread_kmax = kmax;
     p.gather_ctas = (int)std::min<long long>((long long)p.sm_count,
                                              std::max<long long>(1, (M + GATHER_TILE - 1) / GATHER_TILE));
@@ -599,19 +648,34 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
     mem.want(&p.act, sizeof(int) * nt1);
     mem.want(&p.act_rec, sizeof(ActRec) * nt1);
     mem.want(&p.act_rec3, sizeof(ActRec) * nt1);
-    mem.want(&p.items, sizeof(int4) * nt1 * kmax);
+    mem.want(&p.items, sizeof(int4) * n_items);
+    mem.want(&p.direct_units, p.direct ? sizeof(DirectTerm) * d_units : 0);
+    mem.want(&p.direct_items, sizeof(DirectItem) * n_ditems);
     mem.want(&p.err, sizeof(int) * 4);
     mem.want(&p.counter, 2 * sizeof(int));
+    mem.want(&p.direct_fcount, sizeof(int) * f_blocks);
+    mem.want(&p.direct_count, p.direct ? sizeof(int) * (nt1 + 1) : 0);
     mem.want(&p.x, xbytes);
-    mem.want(&p.grids, (size_t)std::max<long long>(1, p.grid_elems) * esize);
+    if (p.direct) {
+        mem.want(&p.z, sizeof(float2) * (size_t)d * M);
+        mem.want(&p.direct_part, sizeof(float) * DA_MAX_ACC * n_ditems);
+        mem.want(&p.direct_fpart, p.direct_split > 1 ? sizeof(float2) * (size_t)p.direct_split * M : 0);
+    } else {
+        mem.want(&p.grids, (size_t)std::max<long long>(1, p.grid_elems) * esize);
+        mem.want(&p.partials, p.n_terms > 0 ? (size_t)kmax * (size_t)p.grid_elems * esize : 0);
+    }
     mem.want(&p.scratch, p.scratch_bytes);
-    mem.want(&p.partials, p.n_terms > 0 ? (size_t)kmax * (size_t)p.grid_elems * esize : 0);
     if (M > 0) {
         mem.want(&p.wt64, sizeof(double) * 8 * (size_t)p.n_slots64 * M);
         mem.want(&p.wb64, sizeof(int) * (size_t)p.n_slots64 * M);
     }
     p.h_act = plan_new<int>(nt1);
-    p.h_items = plan_new<int4>(nt1 * kmax);
+    p.h_items = plan_new<int4>(n_items);
+    if (p.direct) {
+        p.h_units = plan_new<DirectTerm>(d_units);
+        p.h_ditems = plan_new<DirectItem>(n_ditems);
+        if (!p.h_units || !p.h_ditems) return ANOVA_ERR_NOMEM;
+    }
     if (!p.h_act || !p.h_items) return ANOVA_ERR_NOMEM;
     e = mem.commit(&p.arena);
     if (e != cudaSuccess) {
@@ -622,7 +686,7 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
     // tiles (tiles.cuh) for the tensor-core kernels, else records of 16 bytes per
     // node (32 for order 3; FP64 plans sort order <= 2 only), whose sort_slot
     // counts units of M records of 16 bytes
-    if (o.node_sort >= 0 && M > 0 && p.n_terms > 0) {
+    if (o.node_sort >= 0 && M > 0 && p.n_terms > 0 && !p.direct) {
         const bool tiles = !f64 && o.cell_kernel == 0;
         long long n_rec = 0, n_tiles = 0;   // float4 records, tiles
         std::vector<int> slot(p.n_terms, -1);
@@ -696,8 +760,9 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
         chk(cudaMemcpyAsync(p.arena, host.data(), table_bytes, cudaMemcpyHostToDevice, p.stream));
         chk(cudaStreamSynchronize(p.stream));   // `host` leaves scope
     }
-    // counter and error words, and the accumulators and their exponent, adjoin
-    chk(cudaMemsetAsync(p.err, 0, (char *)(p.counter + 2) - (char *)p.err, p.stream));
+    // error and counter words, and the accumulators and their exponent, adjoin
+    char *words = p.direct ? (char *)(p.direct_count + nt1 + 1) : (char *)(p.counter + 2);
+    chk(cudaMemsetAsync(p.err, 0, words - (char *)p.err, p.stream));
     if (p.facc) chk(cudaMemsetAsync(p.facc, 0, (char *)(p.fexp + 4) - (char *)p.facc, p.stream));
     if (xbytes) {
         long long total = (long long)d * M;
@@ -711,6 +776,7 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
         chk(cudaGetLastError());
     }
     if (e == cudaSuccess && p.precision == ANOVA_PREC_F64) chk(cuda_err_of(build_window_tables_f64(p)));
+    if (e == cudaSuccess && p.direct) chk(cuda_err_of(build_unit_table(p)));
     if (e == cudaSuccess) chk(cuda_err_of(sort_nodes_by_cell(p)));
     if (e == cudaSuccess) chk(cuda_err_of(set_active_terms(p, nullptr)));
     chk(cudaStreamSynchronize(p.stream));
@@ -724,16 +790,23 @@ static int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, i
     return ANOVA_OK;
 }
 
-int anova_plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms,
-                      const int32_t *term_dims, const int32_t *bandwidth, const anova_plan_options *opts,
-                      void *stream) {
+int agft::plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
+                      const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct) {
     try {
-        return plan_create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream);
+        return create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, allow_direct);
     } catch (const std::bad_alloc &) {
         return ANOVA_ERR_NOMEM;
     } catch (...) {
         return ANOVA_ERR_CUDA;
     }
+}
+
+extern "C" {
+
+int anova_plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms,
+                      const int32_t *term_dims, const int32_t *bandwidth, const anova_plan_options *opts,
+                      void *stream) {
+    return plan_create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, true);
 }
 
 int anova_debug_fail_allocation(int k) {

@@ -162,6 +162,7 @@ int launch_trafo_f32(Plan &p, const float2 *fhat, float2 *f) {
         fill_const_f32<<<blocks, 256, 0, p.stream>>>(f, p.M, fhat, p.empty_off, p.n_empty, p.skip);
         return cuda_status(cudaGetLastError());
     }
+    if (p.direct) return launch_direct_trafo(p, fhat, f);
     const size_t pre_smem = fft_smem_bytes<float2>(p.max_fft_elems, p.max_n);
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {

@@ -346,14 +346,14 @@ def run_mine(args, rank, world, local_rank):
     rs = 8 if f64 else 4
     grid_bytes = grid_bytes * esz // 8
     if gms / max(gl, 1) >= sms / max(sl, 1):
-        # FP32 plans without third-order terms run the gather on the tensor cores
-        kname, kms, klaunch = ("gather_f64" if f64 else "gather_sorted_f32" if args.cell_kernel else "gather_mma_f32"), \
+        # FP32 plans run the gather on the tensor cores
+        kname, kms, klaunch = ("gather_f64" if f64 else "gather_sorted_f32" if args.cell_kernel else "gather_tiles"), \
             gms / max(gl, 1), gl
         # nodes read (one real per coordinate), f written, grids and coefficients read once
         alg_bytes = rs * d * M + esz * M + grid_bytes + esz * n
     else:
-        # FP32 plans run the order-1/2 spread on the tensor cores (cell-sorted records)
-        kname, kms, klaunch = ("spread_f64" if f64 else "spread_f32" if args.cell_kernel else "spread_mma_f32"), \
+        # and the spread likewise (cell-aligned node tiles)
+        kname, kms, klaunch = ("spread_f64" if f64 else "spread_f32" if args.cell_kernel else "spread_tiles"), \
             sms / max(sl, 1), sl
         # nodes and y read, one grid written
         alg_bytes = rs * d * M + esz * M + grid_bytes
@@ -393,10 +393,10 @@ def run_mine(args, rank, world, local_rank):
                     "peak_source": peak_kind}}
 
     launches = 0
-    # the FP32 forward stage launches the fixed-point passes around the sorted gather
-    # (partial sums, exponent, initialisation, gather, finish)
-    per_stage_kernels = {"trafo_pre": 1, "gather": 1 if f64 else 5, "spread": 1, "reduce_partials": 1,
-                         "adjoint_post": 1, "empty_sum": 2, "solver_vec": 1}
+    # the FP32 forward stage launches the gather and the pass that converts its
+    # fixed-point sums
+    per_stage_kernels = {"trafo_pre": 1, "gather": 1 if f64 else 2, "spread": 1, "reduce_partials": 1,
+                         "adjoint_post": 1, "empty_sum": 1, "solver_vec": 1}
     for name, (_, cnt) in prof.items():
         launches += cnt * per_stage_kernels.get(name, 1)
 
@@ -660,8 +660,8 @@ def batch_result(args, local_rank) -> dict:
             "value": t_sl / t_bl, "unit": "x", "higher_is_better": True,
             "workload": f"64 problems, M {min(Ms)}..{max(Ms)} (total {sum(Ms)}), d 5..15, |u|<=2, N=32 (1D) / 16x16 (2D)",
             "lsqr": "lambda 1e-3, 30 iterations, one LSQR per problem with its own FP64 scalars",
-            "kernels": "per launch all problems: trafo_pre, fixed-point passes around gather_mma_f32, spread_mma_f32, "
-                       "reduce_partials, adjoint_post (cell-sorted records per problem)",
+            "kernels": "per launch all problems: trafo_pre, gather_tiles, the fixed-point sums' conversion, spread_tiles, "
+                       "adjoint_post (cell-aligned node tiles per problem)",
             "results": {"batched_pair_s": t_bp, "sequential_pair_s": t_sp, "pair_speedup": t_sp / t_bp,
                         "batched_lsqr_s": t_bl, "sequential_lsqr_s": t_sl, "lsqr_speedup": t_sl / t_bl,
                         "batched_pairs_per_s": 1.0 / t_bp},

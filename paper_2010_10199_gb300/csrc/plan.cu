@@ -687,7 +687,11 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     // node (32 for order 3; FP64 plans sort order <= 2 only), whose sort_slot
     // counts units of M records of 16 bytes
     if (o.node_sort >= 0 && M > 0 && p.n_terms > 0 && !p.direct) {
-        const bool tiles = !f64 && o.cell_kernel == 0;
+        bool tiles = !f64 && o.cell_kernel == 0;
+        for (int s = 0; s < p.n_terms && tiles; ++s) {   // a tile's places are 32-bit
+            const Term &T = p.h_terms[s];
+            tiles = tile_capacity(M, T.order == 1 ? T.n : (long long)T.n * T.n * (T.order == 3 ? T.n : 1)) * TILE < (1LL << 31);
+        }
         long long n_rec = 0, n_tiles = 0;   // float4 records, tiles
         std::vector<int> slot(p.n_terms, -1);
         for (int s = 0; s < p.n_terms; ++s) {

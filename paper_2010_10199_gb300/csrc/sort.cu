@@ -177,10 +177,11 @@ __global__ void k_cell_scatter64(const Term *terms, const int *wb, long long M, 
 // each.  The blocks' histograms are kept, and the scan turns them into every
 // block's first place in every cell, so that the scatter counts in shared memory
 // only.  Scattered writes are what bounds it: they run at DRAM speed in partial
-// sectors once the terms in work outgrow L2.  So for order <= 2 the scatter writes
-// only the 4-byte indices (a third of the tiles' sectors; big blocks keep few terms
-// in work) and a second pass, in tile order, reads the coordinates through L2 and
-// writes whole lines.
+// sectors once the terms in work outgrow L2.  So for order <= 2 a block first sorts
+// its slice's node numbers in shared memory and writes them by cells, runs of 15 at
+// d = 20, M = 1e6, where a write per node took 4.8 ms instead of 1.4; only the
+// 4-byte indices are written, and a second pass, in tile order, reads the coordinates
+// through L2 and writes whole lines.
 constexpr int SORT_THREADS = 512;
 
 __device__ __forceinline__ int tile_bin(const Term &T, int fr, int fr1, int fc) {
@@ -264,51 +265,128 @@ __global__ void __launch_bounds__(1024) k_tile_scan(const Term *terms, int *hist
     if (threadIdx.x == 0) tile_count[blockIdx.x] = carry;
 }
 
-// the slice's nodes to their places (order <= 2: the indices); each block also
-// writes the tiles' cells and the padding of its share of the term's cells
+// the tiles' cells and the padding of the block's share of a term's cells
+template <typename Pad>
+__device__ __forceinline__ void tile_cells(const Term &T, int nb, const int2 *info, int *cells, Pad pad) {
+    const int n = T.n, S = gridDim.x, b1 = (int)((long long)nb * (blockIdx.x + 1) / S);
+    for (int b = (int)((long long)nb * blockIdx.x / S) + threadIdx.x; b < b1; b += blockDim.x) {
+        const int2 c = info[b];   // first tile, nodes
+        int cell = b;
+        if (T.order == 2) cell = b / n * T.stride + b % n;
+        if (T.order == 3) cell = b % n | b / (n * n) << 8 | b / n % n << 16;   // a, b, c
+        for (int i = 0; i * TILE < c.y; ++i) cells[c.x + i] = cell | (c.y - i * TILE <= TILE / 2 ? TILE_HALF : 0);
+        for (int k = c.y; k % TILE; ++k) pad(c.x * TILE + k);
+    }
+}
+
+// order 3: the slice's nodes to their places
 __global__ void __launch_bounds__(SORT_THREADS)
 k_tile_scatter(const Term *terms, const float *x, long long M, const int *hist, const int2 *cell_info, int max_bins,
                float4 *srec, int *tile_cell) {
     extern __shared__ int bins[];
     const Term &T = terms[blockIdx.y];
-    const int nb = cell_bins(T), S = gridDim.x, n = T.n, order = T.order;
+    if (T.order != 3) return;
+    const int nb = cell_bins(T), S = gridDim.x, n = T.n;
     const int *in = hist + ((long long)blockIdx.y * S + blockIdx.x) * max_bins;
     for (int b = threadIdx.x; b < nb; b += blockDim.x) bins[b] = in[b];
     __syncthreads();
-    const float *xr = x + (long long)(order >= 2 ? T.row0 : T.col) * M;
-    const float *xr1 = x + (long long)(order == 3 ? T.row1 : T.col) * M;
-    const float *xc = x + (long long)T.col * M;
+    const float *xr = x + (long long)T.row0 * M, *xr1 = x + (long long)T.row1 * M, *xc = x + (long long)T.col * M;
     float4 *rec = srec + T.rec_off;
     const long long j1 = M * (blockIdx.x + 1) / S;
-    auto index_at = [&](int pos) -> int & {   // node number pos of a term of order <= 2
-        return ((int *)(rec + (long long)(pos >> 4) * tile_f4(2) + 8))[(pos & 7) * 2 + ((pos >> 3) & 1)];
-    };
     for (long long j = M * blockIdx.x / S + threadIdx.x; j < j1; j += blockDim.x) {
         float tc, tr, tr1;
-        const int fc = grid_pos(xc[j], n, tc);
-        const int fr = order >= 2 ? grid_pos(xr[j], n, tr) : 0, fr1 = order == 3 ? grid_pos(xr1[j], n, tr1) : 0;
+        const int fc = grid_pos(xc[j], n, tc), fr = grid_pos(xr[j], n, tr), fr1 = grid_pos(xr1[j], n, tr1);
         const int pos = atomicAdd(&bins[tile_bin(T, fr, fr1, fc)], 1);
-        if (order == 3)
-            rec[pos] = make_float4(2.f * tr - 1.f, 2.f * tr1 - 1.f, 2.f * tc - 1.f, __int_as_float((int)j));
-        else
-            index_at(pos) = (int)j;
+        rec[pos] = make_float4(2.f * tr - 1.f, 2.f * tr1 - 1.f, 2.f * tc - 1.f, __int_as_float((int)j));
     }
-    int *cells = tile_cell + T.tile_off;
+    tile_cells(T, nb, cell_info + (long long)blockIdx.y * max_bins, tile_cell + T.tile_off,
+               [&](int pos) { rec[pos] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1)); });
+}
+
+// order <= 2: the slice's node numbers to their places, in parts of at most `cap`
+// nodes (16-bit numbers) that are sorted by cell in shared memory: [cells] ends of the
+// part's runs, [cells] next places, [cap] numbers.  A slice of one part takes its counts
+// from the histograms.
+constexpr int PLACE_THREADS = 1024, PLACE_MAX = 65536;
+__global__ void __launch_bounds__(PLACE_THREADS)
+k_tile_place(const Term *terms, const float *x, long long M, const int *hist, const int2 *cell_info, int max_bins,
+             int place_bins, int cap, float4 *srec, int *tile_cell) {
+    extern __shared__ int sm[];
+    __shared__ int wsum[32];
+    const Term &T = terms[blockIdx.y];
+    if (T.order == 3) return;
+    const int nb = cell_bins(T), S = gridDim.x, n = T.n, order = T.order, tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
+    int *ends = sm, *place = sm + place_bins;
+    unsigned short *list = (unsigned short *)(place + place_bins);
+    const int *in = hist + ((long long)blockIdx.y * S + blockIdx.x) * max_bins;
     const int2 *info = cell_info + (long long)blockIdx.y * max_bins;
-    const int b1 = (int)((long long)nb * (blockIdx.x + 1) / S);
-    for (int b = (int)((long long)nb * blockIdx.x / S) + threadIdx.x; b < b1; b += blockDim.x) {
-        const int2 c = info[b];   // first tile, nodes
-        int cell = b;
-        if (order == 2) cell = b / n * T.stride + b % n;
-        if (order == 3) cell = b % n | b / (n * n) << 8 | b / n % n << 16;   // a, b, c
-        for (int i = 0; i * TILE < c.y; ++i) cells[c.x + i] = cell | (c.y - i * TILE <= TILE / 2 ? TILE_HALF : 0);
-        for (int k = c.y; k % TILE; ++k) {
-            if (order == 3)
-                rec[c.x * TILE + k] = make_float4(0.f, 0.f, 0.f, __int_as_float(-1));
-            else
-                index_at(c.x * TILE + k) = -1;
+    const float *xr = x + (long long)(order >= 2 ? T.row0 : T.col) * M, *xc = x + (long long)T.col * M;
+    int *out = (int *)(srec + T.rec_off + 8);   // indices of tile 0
+    auto put = [&](int pos, int id) { out[(long long)(pos >> 4) * (tile_f4(2) * 4) + (pos & 7) * 2 + ((pos >> 3) & 1)] = id; };
+    const long long j0 = M * blockIdx.x / S, len = M * (blockIdx.x + 1) / S - j0;
+    const int parts = (int)((len + cap - 1) / cap);
+    for (int b = tid; b < nb; b += PLACE_THREADS) place[b] = in[b];
+    for (int c = 0; c < parts; ++c) {
+        const long long a = j0 + len * c / parts;
+        const int m = (int)(j0 + len * (c + 1) / parts - a);
+        auto bin = [&](int i) {
+            float t;
+            const int fc = grid_pos(xc[a + i], n, t), fr = order >= 2 ? grid_pos(xr[a + i], n, t) : 0;
+            return tile_bin(T, fr, 0, fc);
+        };
+        if (parts == 1) {
+            for (int b = tid; b < nb; b += PLACE_THREADS)
+                ends[b] = ((int)blockIdx.x + 1 < S ? in[max_bins + b] : info[b].x * TILE + info[b].y) - in[b];
+        } else {
+            for (int b = tid; b < nb; b += PLACE_THREADS) {
+                if (c > 0) place[b] += ends[b] - (b > 0 ? ends[b - 1] : 0);
+            }
+            __syncthreads();
+            for (int b = tid; b < nb; b += PLACE_THREADS) ends[b] = 0;
+            __syncthreads();
+            for (int i = tid; i < m; i += PLACE_THREADS) atomicAdd(&ends[bin(i)], 1);
         }
+        __syncthreads();
+        {   // counts to first numbers: a thread's consecutive cells, then the threads
+            const int per = (nb + PLACE_THREADS - 1) / PLACE_THREADS, b0 = min(nb, tid * per), b1 = min(nb, b0 + per);
+            int sum = 0;
+            for (int b = b0; b < b1; ++b) sum += ends[b];
+            int v = sum;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(0xffffffffu, v, o);
+                if (lane >= o) v += u;
+            }
+            if (lane == 31) wsum[wid] = v;
+            __syncthreads();
+            if (wid == 0) {
+                int w = wsum[lane];
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const int u = __shfl_up_sync(0xffffffffu, w, o);
+                    if (lane >= o) w += u;
+                }
+                wsum[lane] = w;
+            }
+            __syncthreads();
+            int at = v - sum + (wid > 0 ? wsum[wid - 1] : 0);
+            for (int b = b0; b < b1; ++b) {
+                const int k = ends[b];
+                ends[b] = at;
+                at += k;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < m; i += PLACE_THREADS) list[atomicAdd(&ends[bin(i)], 1)] = (unsigned short)i;
+        __syncthreads();
+        // 16 lanes per cell's run
+        for (int b = tid >> 4; b < nb; b += PLACE_THREADS / 16) {
+            const int first = b > 0 ? ends[b - 1] : 0, k = ends[b] - first, at = place[b];
+            for (int i = tid & 15; i < k; i += 16) put(at + i, (int)a + list[first + i]);
+        }
+        __syncthreads();
     }
+    tile_cells(T, nb, info, tile_cell + T.tile_off, [&](int pos) { put(pos, -1); });
 }
 
 // order <= 2: the window arguments of the tiles' nodes, a lane per node and two
@@ -342,10 +420,14 @@ __global__ void __launch_bounds__(256) k_tile_fill(const Term *terms, const floa
 }
 
 static int sort_tiles(Plan &p) {
-    int max_bins = 1;
+    int max_bins = 1, place_bins = 0, n3 = 0;   // place_bins: of the terms of order <= 2
     for (int s = 0; s < p.n_terms; ++s) {
         const Term &T = p.h_terms[s];
         max_bins = std::max(max_bins, T.order == 3 ? T.n * T.n * T.n : (T.order == 2 ? T.n * T.n : T.n));
+        if (T.order == 3)
+            ++n3;
+        else
+            place_bins = std::max(place_bins, T.order == 2 ? T.n * T.n : T.n);
     }
     // slices of at least 16384 nodes (a block also moves a histogram)
     const int S = (int)std::max<long long>(1, std::min<long long>(SORT_MAX_SLICES, p.M / 16384));
@@ -363,22 +445,32 @@ static int sort_tiles(Plan &p) {
         info = own;
     }
     const size_t bytes = sizeof(int) * (size_t)max_bins;
-    if (bytes > 48 * 1024) {
-        e = cudaFuncSetAttribute(k_tile_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-        if (e == cudaSuccess)
-            e = cudaFuncSetAttribute(k_tile_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    }
+    static std::atomic<unsigned long long> attr_seen{0};
+    once_per_device(attr_seen, [] {
+        cudaFuncSetAttribute(k_tile_count, cudaFuncAttributeMaxDynamicSharedMemorySize, TILES_MAX_SMEM);
+        cudaFuncSetAttribute(k_tile_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, TILES_MAX_SMEM);
+        cudaFuncSetAttribute(k_tile_place, cudaFuncAttributeMaxDynamicSharedMemorySize, TILES_MAX_SMEM);
+    });
+    // a part's numbers beside the cells' ends and places (at most 100 KB: 12800 cells)
+    const size_t cells = 2 * sizeof(int) * (size_t)place_bins;
+    const int cap = (int)std::min<long long>({(long long)PLACE_MAX, (long long)((TILES_MAX_SMEM - cells) / 2), (p.M + S - 1) / S});
+    const size_t place_bytes = cells + sizeof(unsigned short) * (size_t)cap;
     if (e == cudaSuccess) {
         const dim3 grid(S, p.n_terms);
         const float *x = (const float *)p.x;
         int *hist = (int *)(info + n_bins);
         k_tile_count<<<grid, SORT_THREADS, bytes, p.stream>>>(p.terms, x, p.M, hist, max_bins);
         k_tile_scan<<<p.n_terms, 1024, 0, p.stream>>>(p.terms, hist, S, max_bins, info, p.tile_count);
-        k_tile_scatter<<<grid, SORT_THREADS, bytes, p.stream>>>(p.terms, x, p.M, hist, info, max_bins, p.srec,
-                                                                p.tile_cell);
-        // about 16 steps per warp
-        const int fb = (int)std::max<long long>(1, std::min<long long>(256, p.M / 4096));
-        k_tile_fill<<<dim3(fb, p.n_terms), 256, 0, p.stream>>>(p.terms, x, p.M, p.srec, p.tile_count);
+        if (n3 > 0)
+            k_tile_scatter<<<grid, SORT_THREADS, bytes, p.stream>>>(p.terms, x, p.M, hist, info, max_bins, p.srec,
+                                                                    p.tile_cell);
+        if (n3 < p.n_terms) {
+            k_tile_place<<<grid, PLACE_THREADS, place_bytes, p.stream>>>(p.terms, x, p.M, hist, info, max_bins,
+                                                                         place_bins, cap, p.srec, p.tile_cell);
+            // about 16 steps per warp
+            const int fb = (int)std::max<long long>(1, std::min<long long>(256, p.M / 4096));
+            k_tile_fill<<<dim3(fb, p.n_terms), 256, 0, p.stream>>>(p.terms, x, p.M, p.srec, p.tile_count);
+        }
         e = cudaGetLastError();
     }
     if (own) {

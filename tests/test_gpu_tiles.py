@@ -57,3 +57,19 @@ def test_tiles_against_the_sums(gft, counts, bw, chunks, m_row):
     xo = f32_nodes(x)
     assert np.abs(f - ndft.trafo(xo, terms, bws, fhat)).max() <= tol * np.abs(fhat).sum()
     assert np.abs(g - ndft.adjoint(xo, terms, bws, y)).max() <= tol * np.abs(y).sum()
+
+
+@pytest.mark.parametrize("M", [16383, 16385, 32769, 1048576, 1048577, 1300001])
+def test_sort_slices_and_parts(gft, M):
+    """One to sixteen slices, of one part and of two (more than 65536 nodes): the same
+    plan over records, which are sorted node by node; both hold 1e-5 of the sums."""
+    import torch
+    x = to_dev(inputs.uniform(31, M, 2 * M).reshape(2, M) - 0.5, torch.float32)
+    terms, bws = [(), (0,), (1,), (0, 1)], [0, 100, 64, 32]
+    out = []
+    for kernel in (0, 1):
+        P = gft.Plan(x, terms, bws, n_ctas=16, cell_kernel=kernel)
+        fhat, y = cplx_dev(inputs.complex_normal(5, 2, P.n_coeffs)), cplx_dev(inputs.complex_normal(5, 4, M))
+        out.append((host(P.trafo(fhat)), host(P.adjoint(y))))
+    for a, b in zip(*out):
+        assert np.linalg.norm(a - b) <= 2e-5 * np.linalg.norm(b)

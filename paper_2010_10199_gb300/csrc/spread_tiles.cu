@@ -27,6 +27,22 @@ __device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
     return d;
 }
 
+// Adds a lane's (g, t) window taps G (moments_to_window) to the elements c0 and c1 of
+// the shared grid.  Lanes whose grid rows fall into the same banks (rows g of a pitch
+// that is 8 mod 16: g of one parity) start at different words: one bank per lane
+// instead of four lanes per bank, a quarter of the additions' shared-memory wavefronts
+// (2.6e7 -> 6.6e6 at d = 20, M = 3e5; third order, d = 10, M = 5e5: 3.36 -> 3.16 ms).
+__device__ __forceinline__ void add_taps(float2 *c0, float2 *c1, const float (&G)[4], int g) {
+    float v[4] = {G[0], G[2], G[1], G[3]}, u[4], w[4];
+    const int s = g >> 1;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) u[q] = s & 1 ? v[(q + 1) & 3] : v[q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) w[q] = s & 2 ? u[(q + 2) & 3] : u[q];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) red_add_f32((float *)((q + s) & 2 ? c1 : c0) + ((q + s) & 1), w[q]);
+}
+
 // Window block of a cell from its moments: G = C_col Mo C_row^T, with lane (g, t)
 // holding d = Mo (re i = g, l = 2t), (re g, 2t + 1), (im g, 2t), (im g, 2t + 1) and
 // the coefficients cr0, cr1 = C_row[g][2t], C_row[g][2t + 1] (zero where no row g
@@ -69,17 +85,20 @@ __device__ __forceinline__ void moments_to_window(const float (&d)[4], float cr0
 // basis alone; the values pass through shared memory to the lanes that hold them
 // as fragments (lane (g, t): index g of nodes 2t, 2t + 1 of a group, 16 bytes of A
 // and 8 of B per read, rows padded to keep the reads free of bank conflicts).
-// The records and y[index] are loaded to registers two steps and one step ahead; a
-// bulk prefetch brings the records into L2 before that.  Each tile gets a fresh
+// The records, y[index] and the tiles' cells are loaded to registers two steps, one step
+// and one step ahead (the cells when needed: d = 20, M = 1e6 2.25 ms instead of 2.01; the
+// values two steps ahead: 2.12); a bulk prefetch brings the records into L2 before that.  Each tile gets a fresh
 // tensor-core sum, added to the cell's in FP32 with rounding to nearest: the
 // tensor core's own accumulation is not rounded to nearest, and its bias would
 // grow with the cell's node count.  Order 1: B = e_0 (the single grid row).
-// Row 0 of B, X_0 = 1, is one row for all warps.
+// Row 0 of B, X_0 = 1, is one row for all warps; a warp's buffer is a multiple of 128
+// bytes, so that the row keeps its place in the banks' order for each of them.
 constexpr int ST_AROW = 40, ST_BROW = 40;   // row strides: float2 (320 bytes) and float (160 bytes)
 constexpr size_t ST_A_BYTES = NCOEF * ST_AROW * sizeof(float2);
 constexpr size_t ST_B_BYTES = (NCOEF - 1) * ST_BROW * sizeof(float);
 constexpr size_t ST_ONE_BYTES = ST_BROW * sizeof(float);
-constexpr size_t ST_WARP_BYTES = ST_A_BYTES + ST_B_BYTES;
+constexpr size_t ST_WARP_BYTES = (ST_A_BYTES + ST_B_BYTES + 127) / 128 * 128;
+static_assert(ST_A_BYTES % 128 == 0 && ST_ONE_BYTES == ST_BROW * sizeof(float), "row 0 of B lies a row's pitch before row 1");
 
 template <int MR, bool ORD2>
 __device__ __forceinline__ void spread_run12(const float4 *__restrict__ rec, const int *__restrict__ cells, int nt,
@@ -101,11 +120,8 @@ __device__ __forceinline__ void spread_run12(const float4 *__restrict__ rec, con
         float G[4];
         moments_to_window(d, cr0, cr1, __ldg(chc + g * NCOEF + 2 * t), __ldg(chc + g * NCOEF + 2 * t + 1), G);
         if (ORD2 ? g < 2 * MR : g == 0) {
-            float *c = (float *)(S + cur + g * stride + 2 * t);
-            red_add_f32(c, G[0]);
-            red_add_f32(c + 1, G[2]);
-            red_add_f32(c + 2, G[1]);
-            red_add_f32(c + 3, G[3]);
+            float2 *c = S + cur + g * stride + 2 * t;
+            add_taps(c, c + 1, G, g);
         }
         d[0] = d[1] = d[2] = d[3] = 0.f;
     };
@@ -129,8 +145,11 @@ __device__ __forceinline__ void spread_run12(const float4 *__restrict__ rec, con
     auto load_y = [&](int id) { return id >= 0 ? __ldcg(y + id) : make_float2(0.f, 0.f); };
     Rec r0 = load(0), r1 = load(min(1, ns - 1));
     float2 y0 = load_y(r0.id);
+    int n0 = __ldg(cells), n1 = __ldg(cells + 1);
     for (int s = 0; s < ns; ++s) {
-        const int c0 = __ldg(cells + 2 * s), c1 = 2 * s + 1 < nt ? __ldg(cells + 2 * s + 1) : (c0 & ~TILE_HALF);
+        const int c0 = n0, c1 = 2 * s + 1 < nt ? n1 : (c0 & ~TILE_HALF);
+        n0 = __ldg(cells + 2 * s + 2);   // the next step's (inside the buffer past the run's end)
+        n1 = __ldg(cells + 2 * s + 3);
         if (lane == 0 && 2 * s + PF + 2 <= nt) prefetch_l2_bulk(rec + (long long)(2 * s + PF) * F4, 2 * F4 * 16);
         const float2 yv = y0;
         const float vr = r0.vr, vc = r0.vc;
@@ -267,11 +286,9 @@ __device__ __forceinline__ void spread_run3(const float4 *__restrict__ rec, cons
         moments_to_window(m, cr0, cr1, __ldg(&wc->pb[g][2 * t]), __ldg(&wc->pb[g][2 * t + 1]), G);
         if (g < NP) {
             float2 *row = S + (wrap(wrap(fa - MR + 1, n), n) * n + wrap(fb - MR + 1 + g, n)) * stride;
-            float *c0 = (float *)(row + wrap(fc - mc + 1 + 2 * t, n)), *c1 = (float *)(row + wrap(fc - mc + 2 + 2 * t, n));
-            red_add_f32(c0, G[0] * inv_ys);
-            red_add_f32(c0 + 1, G[2] * inv_ys);
-            red_add_f32(c1, G[1] * inv_ys);
-            red_add_f32(c1 + 1, G[3] * inv_ys);
+#pragma unroll
+            for (int q = 0; q < 4; ++q) G[q] *= inv_ys;
+            add_taps(row + wrap(fc - mc + 1 + 2 * t, n), row + wrap(fc - mc + 2 + 2 * t, n), G, g);
         }
     };
     int cur = -1;
@@ -307,8 +324,10 @@ __device__ __forceinline__ void spread_run3(const float4 *__restrict__ rec, cons
     cp_async_wait_n<2>();
     __syncwarp();
     load_y(0);
+    int ncell = __ldg(cells);
     for (int i = 0; i < nt; ++i) {
-        const int cell = __ldg(cells + i) & ~TILE_HALF;
+        const int cell = ncell & ~TILE_HALF;
+        ncell = __ldg(cells + i + 1);   // the next tile's (inside the buffer past the run's end)
         if (lane == 0 && i + PF < nt) prefetch_l2_bulk(rec + (long long)(i + PF) * TILE, TILE * 16);
         float2 yv[4];
 #pragma unroll

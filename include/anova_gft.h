@@ -473,6 +473,15 @@ int grouped_trafo_noalloc(int d, int64_t M, const float *x_dev, int n_terms, con
  */
 int anova_debug_fail_allocation(int k);
 
+/*
+ * anova_debug_batch_form -- the form in which a batch's kernels read the nodes of
+ * problems kept in the given forms (host only, for tests; no counterpart in the
+ * paper): 0 in their own order, 1 cell-sorted records, 2 node tiles.  Problems of
+ * different forms are read in their own order: no kernel reads two.
+ * ANOVA_ERR_INVALID for no problems.
+ */
+int anova_debug_batch_form(const int32_t *forms, int n_problems);
+
 /* Human-readable name of a status code (static string). */
 const char *anova_status_string(int status);
 

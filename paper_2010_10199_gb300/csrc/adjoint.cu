@@ -597,8 +597,8 @@ __device__ __forceinline__ void spread_items(const DevPlan &single, const BatchA
 #pragma unroll
             for (int i = 0; i < NCOEF; ++i) wcf[i] = __ldg(wsrc + i);
         }
-        // in a batch whose other problems have no room for sorted nodes, a problem
-        // may hold node tiles, which only the tensor-core kernels read
+        // in a batch whose problems differ in form, a problem may hold node tiles, which
+        // only the tensor-core kernels read
         const bool sorted = T.sort_slot >= 0 && P.srec && !P.tile_cell;
         __syncthreads();   // grid zeroed before any addition
         if constexpr (O3) {

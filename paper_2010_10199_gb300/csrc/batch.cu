@@ -43,8 +43,8 @@ struct Batch {
         max_n = 1, max_stage = 0, max_chunks = 1, sm_count = 152;
     long long max_grid_bytes = 16, max_grid_elems = 0;
     bool any_empty = false;
-    bool sorted_fwd = true;   // every problem has cell-sorted records for all its terms
-    bool cell_tc = true;      // every problem runs its order-1/2 spread on the tensor cores
+    bool sorted_fwd = false;  // every problem has sorted nodes of one form, and accumulators
+    bool cell_tc = false;     // every problem has node tiles
     long long max_M = 0;
     double2 *scratch = nullptr;
     // batched LSQR workspace
@@ -69,6 +69,12 @@ static void free_batch(Batch *b) {
     if (b->e1) cudaEventDestroy(b->e1);
     for (anova_plan_t p : b->plans) anova_plan_destroy(p);
     delete b;
+}
+
+int batch_form(const int *forms, int n) {
+    for (int p = 1; p < n; ++p)
+        if (forms[p] != forms[0]) return FORM_NONE;
+    return n > 0 ? forms[0] : FORM_NONE;
 }
 
 static int upload_views(Batch &b) {
@@ -229,6 +235,10 @@ struct anova_batch_s {
 
 extern "C" {
 
+int anova_debug_batch_form(const int32_t *forms, int n_problems) {
+    return forms && n_problems > 0 ? batch_form(forms, n_problems) : ANOVA_ERR_INVALID;
+}
+
 int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const int64_t *M, const float *const *x_dev,
                        const int *n_terms, const int32_t *const *term_dims, const int32_t *const *bandwidth,
                        const anova_plan_options *opts, void *stream) {
@@ -244,7 +254,8 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
     b->stream = (cudaStream_t)stream;
     b->node_off.assign(n_problems + 1, 0);
     b->coef_off.assign(n_problems + 1, 0);
-    std::vector<int> tile_prob, tile0, blk_prob, blk0;
+    std::vector<int> tile_prob, tile0, blk_prob, blk0, forms;
+    bool accumulators = true;
     int pitch = -1;
     bool mixed_pitch = false;
     for (int p = 0; p < n_problems; ++p) {
@@ -290,11 +301,14 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
         b->max_grid_bytes = std::max(b->max_grid_bytes, pl.max_grid_bytes);
         b->max_grid_elems = std::max(b->max_grid_elems, pl.grid_elems);
         b->any_empty = b->any_empty || pl.n_empty > 0;
-        b->sorted_fwd = b->sorted_fwd && pl.srec && pl.facc && pl.n_act3 == 0;
-        b->cell_tc = b->cell_tc && pl.srec && pl.cell_tc;
+        forms.push_back(node_form(pl));
+        accumulators = accumulators && pl.facc && pl.n_act3 == 0;
         b->max_M = std::max(b->max_M, pl.M);
         b->sm_count = pl.sm_count;
     }
+    const int form = batch_form(forms.data(), n_problems);
+    b->sorted_fwd = form != FORM_NONE && accumulators;
+    b->cell_tc = form == FORM_TILES;
     b->pitch = mixed_pitch || pitch < 0 ? 0 : pitch;
     // spread items: every problem's active terms split into K_p node chunks of about
     // the same size for all problems (one chunk per term each, the largest problem's

@@ -181,6 +181,18 @@ struct BatchArgs {
 enum { ERR_CODE = 0, ERR_YMAX = 2 };
 
 constexpr int N_STAGES = 7;
+// How a plan keeps its nodes, and so which kernels read them.
+enum NodeForm {
+    FORM_NONE = 0,      // no sorted copy: point-major gather, spread with per-node atomics
+    FORM_RECORDS = 1,   // cell-sorted records: CUDA cores
+    FORM_TILES = 2,     // node tiles: tensor cores
+    FORM_DIRECT = 3     // no grid either: direct sums
+};
+// The form in which a batch's kernels can read all its problems' nodes: tiles and
+// records are laid out differently, and a kernel reads one of them, so a batch that
+// holds both runs over the nodes in their own order.
+int batch_form(const int *forms, int n);
+
 struct Profiler;   // per-stage CUDA-event timing (profile.cu)
 
 struct Plan {
@@ -270,6 +282,9 @@ struct Plan {
 };
 
 DevPlan dev_view(const Plan &p);
+inline int node_form(const Plan &p) {
+    return p.direct ? FORM_DIRECT : !p.srec ? FORM_NONE : p.cell_tc ? FORM_TILES : FORM_RECORDS;
+}
 int set_active_terms(Plan &p, const unsigned char *user_mask);
 inline cudaError_t cuda_err_of(int status) {
     return status == ANOVA_OK ? cudaSuccess : status == ANOVA_ERR_NOMEM ? cudaErrorMemoryAllocation : cudaErrorUnknown;

@@ -474,6 +474,15 @@ int grouped_trafo_noalloc(int d, int64_t M, const float *x_dev, int n_terms, con
 int anova_debug_fail_allocation(int k);
 
 /*
+ * anova_debug_plan_form -- how a plan keeps its nodes, and so which kernels run its
+ * transforms (for tests; no counterpart in the paper): 0 in their own order
+ * (point-major gather, spread with per-node atomics), 1 cell-sorted records (CUDA
+ * cores), 2 node tiles (tensor cores), 3 no grids: the sums are computed directly.
+ * ANOVA_ERR_INVALID for NULL.
+ */
+int anova_debug_plan_form(anova_plan_t plan);
+
+/*
  * anova_debug_batch_form -- the form in which a batch's kernels read the nodes of
  * problems kept in the given forms (host only, for tests; no counterpart in the
  * paper): 0 in their own order, 1 cell-sorted records, 2 node tiles.  Problems of

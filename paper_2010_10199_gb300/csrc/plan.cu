@@ -826,6 +826,8 @@ void anova_plan_destroy(anova_plan_t plan) {
     delete plan;
 }
 
+int anova_debug_plan_form(anova_plan_t plan) { return plan ? node_form(plan->p) : ANOVA_ERR_INVALID; }
+
 int64_t anova_num_coeffs(anova_plan_t plan) { return plan ? plan->p.n_coeffs : -1; }
 
 int anova_term_offset(anova_plan_t plan, int u, int64_t *off, int64_t *len) {

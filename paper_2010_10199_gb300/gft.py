@@ -158,6 +158,10 @@ def load(path: str | None = None):
     lib.anova_sobol_indices.restype = ctypes.c_int
     lib.anova_l2_error.argtypes = [vp, vp, vp, ctypes.c_double, ctypes.POINTER(ctypes.c_double)]
     lib.anova_l2_error.restype = ctypes.c_int
+    lib.anova_debug_plan_form.argtypes = [vp]
+    lib.anova_debug_plan_form.restype = ctypes.c_int
+    lib.anova_debug_batch_form.argtypes = [i32p, ctypes.c_int]
+    lib.anova_debug_batch_form.restype = ctypes.c_int
     lib.anova_debug_fail_allocation.argtypes = [ctypes.c_int]
     lib.anova_debug_fail_allocation.restype = ctypes.c_int
     lib.anova_status_string.argtypes = [ctypes.c_int]
@@ -338,6 +342,13 @@ def anova_l2_error(h, fhat_ptr, c_ptr, norm2):
                                                    ctypes.c_void_p(int(c_ptr) or None), float(norm2),
                                                    ctypes.byref(err)))
     return err.value
+
+
+FORM_OWN_ORDER, FORM_RECORDS, FORM_TILES, FORM_DIRECT = 0, 1, 2, 3
+
+
+def anova_debug_plan_form(h) -> int:
+    return int(load().anova_debug_plan_form(h))
 
 
 def anova_debug_fail_allocation(k: int):

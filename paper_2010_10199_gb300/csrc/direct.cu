@@ -371,10 +371,19 @@ direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f,
 
 // ------------------------------------------------------------ adjoint ----
 
-// Block sums of R values per thread (R padded to a multiple of 32 with zeros in v)
-// into out[0, R): each warp halves the values it keeps per exchange.
+// A thread adds at most DA_CHAIN nodes in FP32; the block's sums over such runs are added
+// in FP64.  An FP32 chain's error grows with the root of its length: at d = 6, N = 16/8,
+// M = 1e6 one chain of 601 nodes left 4.8e-7, where the NFFT has 2.8e-7.  One exchange of
+// the block's sums per run is 2 % of its products at most.  Items of more than a run have
+// kernels of their own (RUNS): the loop over runs cost 13 registers and 1.5 % at the
+// solvers' sizes, which have one.
+constexpr int DA_CHAIN = 128, DA_RUN = DA_CHAIN * DA_THREADS;
+
+// Block sums of R values per thread (R padded to a multiple of 32 with zeros in v):
+// each warp halves the values it keeps per exchange.  The sums of all calls from the
+// `first` to the `last` go to out[0, R); tot: [R], the sums so far.
 template <int R>
-__device__ __forceinline__ void block_sums(float (&v)[R], float *out, float *sh) {
+__device__ __forceinline__ void block_sums(float (&v)[R], float *out, float *sh, double *tot, bool first, bool last) {
     static_assert(R % 32 == 0, "padded");
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
@@ -395,17 +404,26 @@ __device__ __forceinline__ void block_sums(float (&v)[R], float *out, float *sh)
         float s = 0.f;
 #pragma unroll
         for (int w = 0; w < DA_THREADS / 32; ++w) s += sh[w * R + i];
-        out[i] = s;
+        if (first && last) {
+            out[i] = s;
+        } else {
+            const double t = first ? (double)s : tot[i] + s;   // the thread's own value
+            if (last)
+                out[i] = (float)t;
+            else
+                tot[i] = t;
+        }
     }
+    if (!last) __syncthreads();   // sh is read before the next run's sums
 }
 
 // ROWS rows of a term of order ORD over nodes [a, b): all of them, or those of index
 // `ia` of a third-order term's first axis.  Per row and innermost
 // pair the sums of u.x c, u.y s, u.y c, u.x s (u = y times the conjugate outer powers,
 // (c, s) the innermost power); cosine: u.x c, u.y c per function.
-template <int K, bool COS, int ORD>
+template <int K, bool COS, int ORD, bool RUNS>
 __device__ __forceinline__ void adjoint_rows(const DevPlan &P, const DirectTerm &T, const float2 *__restrict__ y,
-                                             long long a, long long b, float *out, float *sh) {
+                                             long long a, long long b, float *out, float *sh, double *tot) {
     constexpr int ROWS = group_rows<COS>(ORD, K), PER = COS ? 2 : 4, R = (ROWS * K * PER + 31) / 32 * 32;
     constexpr int N = axis_coefs<COS>(K);
     constexpr bool ALL = ORD == 3 && ROWS == N * N;
@@ -443,84 +461,95 @@ __device__ __forceinline__ void adjoint_rows(const DevPlan &P, const DirectTerm 
         if (ORD == 3) na = __ldg(za + i);
     };
     load(j);
-    for (; j < b; j += DA_THREADS) {
-        const float2 yv = ny, z = nz, zrow = nr, zfirst = na;
-        load(j + DA_THREADS);
-        float2 e[K], pw[2 * K], pa[2 * K], ya = yv;
-        e[0] = z;
+    for (long long r1 = RUNS ? min(b, a + DA_RUN) : b;; r1 = min(b, r1 + DA_RUN)) {
+        for (; j < r1; j += DA_THREADS) {
+            const float2 yv = ny, z = nz, zrow = nr, zfirst = na;
+            load(j + DA_THREADS);
+            float2 e[K], pw[2 * K], pa[2 * K], ya = yv;
+            e[0] = z;
 #pragma unroll
-        for (int k = 1; k < K; ++k) e[k] = cmul(e[k - 1], z);
-        conj_powers(zrow, pw);
-        if (ORD == 3) {
-            conj_powers(zfirst, pa);
-            if (!ALL) {   // the one index of the first axis
-                float2 w = pa[0];
+            for (int k = 1; k < K; ++k) e[k] = cmul(e[k - 1], z);
+            conj_powers(zrow, pw);
+            if (ORD == 3) {
+                conj_powers(zfirst, pa);
+                if (!ALL) {   // the one index of the first axis
+                    float2 w = pa[0];
 #pragma unroll
-                for (int k = 1; k < N; ++k)
-                    if (k == ia) w = pa[k];
-                ya = COS ? make_float2(yv.x * w.x, yv.y * w.x) : cmul(yv, w);
+                    for (int k = 1; k < N; ++k)
+                        if (k == ia) w = pa[k];
+                    ya = COS ? make_float2(yv.x * w.x, yv.y * w.x) : cmul(yv, w);
+                }
             }
-        }
 #pragma unroll
-        for (int r = 0; r < ROWS; ++r) {
-            const float2 w = pw[ALL ? r % N : r];
-            if (ALL && r % N == 0) ya = COS ? make_float2(yv.x * pa[r / N].x, yv.y * pa[r / N].x) : cmul(yv, pa[r / N]);
-            const float2 u = COS ? make_float2(ya.x * w.x, ya.y * w.x) : cmul(ya, w);
+            for (int r = 0; r < ROWS; ++r) {
+                const float2 w = pw[ALL ? r % N : r];
+                if (ALL && r % N == 0) ya = COS ? make_float2(yv.x * pa[r / N].x, yv.y * pa[r / N].x) : cmul(yv, pa[r / N]);
+                const float2 u = COS ? make_float2(ya.x * w.x, ya.y * w.x) : cmul(ya, w);
 #pragma unroll
-            for (int k = 0; k < K; ++k) {
-                float *v = acc + (r * K + k) * PER;
-                if (COS) {
-                    v[0] = fmaf(u.x, e[k].x, v[0]);
-                    v[1] = fmaf(u.y, e[k].x, v[1]);
-                } else {
-                    v[0] = fmaf(u.x, e[k].x, v[0]);
-                    v[1] = fmaf(u.y, e[k].y, v[1]);
-                    v[2] = fmaf(u.y, e[k].x, v[2]);
-                    v[3] = fmaf(u.x, e[k].y, v[3]);
+                for (int k = 0; k < K; ++k) {
+                    float *v = acc + (r * K + k) * PER;
+                    if (COS) {
+                        v[0] = fmaf(u.x, e[k].x, v[0]);
+                        v[1] = fmaf(u.y, e[k].x, v[1]);
+                    } else {
+                        v[0] = fmaf(u.x, e[k].x, v[0]);
+                        v[1] = fmaf(u.y, e[k].y, v[1]);
+                        v[2] = fmaf(u.y, e[k].x, v[2]);
+                        v[3] = fmaf(u.x, e[k].y, v[3]);
+                    }
                 }
             }
         }
+        block_sums<R>(acc, out, sh, tot, !RUNS || r1 - DA_RUN <= a, !RUNS || r1 == b);
+        if (!RUNS || r1 == b) break;
+#pragma unroll
+        for (int i = 0; i < R; ++i) acc[i] = 0.f;
     }
-    block_sums<R>(acc, out, sh);
 }
 
 // frequencies 1 + ORD1_GROUP group .. of an order-1 term
-template <bool COS>
+template <bool COS, bool RUNS>
 __device__ __forceinline__ void adjoint_order1(const DevPlan &P, const DirectTerm &T, const float2 *__restrict__ y,
-                                               long long a, long long b, float *out, float *sh) {
+                                               long long a, long long b, float *out, float *sh, double *tot) {
     float acc[32];
 #pragma unroll
     for (int i = 0; i < 32; ++i) acc[i] = 0.f;
     const float *x = P.x + (long long)T.col * P.M;
     const float2 *zc = P.z + (long long)T.col * P.M;
-    for (long long j = a + threadIdx.x; j < b; j += DA_THREADS) {
-        const float2 u = __ldg(y + j), z = __ldg(zc + j);
-        float2 w = unit_power(__ldg(x + j), 1 + ORD1_GROUP * T.group);
+    long long j = a + threadIdx.x;
+    for (long long r1 = RUNS ? min(b, a + DA_RUN) : b;; r1 = min(b, r1 + DA_RUN)) {
+        for (; j < r1; j += DA_THREADS) {
+            const float2 u = __ldg(y + j), z = __ldg(zc + j);
+            float2 w = unit_power(__ldg(x + j), 1 + ORD1_GROUP * T.group);
 #pragma unroll
-        for (int k = 0; k < ORD1_GROUP; ++k) {
-            float *v = acc + 4 * k;
-            v[0] = fmaf(u.x, w.x, v[0]);
-            v[2] = fmaf(u.y, w.x, v[2]);
-            if (!COS) {
-                v[1] = fmaf(u.y, w.y, v[1]);
-                v[3] = fmaf(u.x, w.y, v[3]);
+            for (int k = 0; k < ORD1_GROUP; ++k) {
+                float *v = acc + 4 * k;
+                v[0] = fmaf(u.x, w.x, v[0]);
+                v[2] = fmaf(u.y, w.x, v[2]);
+                if (!COS) {
+                    v[1] = fmaf(u.y, w.y, v[1]);
+                    v[3] = fmaf(u.x, w.y, v[3]);
+                }
+                w = cmul(w, z);
             }
-            w = cmul(w, z);
         }
+        block_sums<32>(acc, out, sh, tot, !RUNS || r1 - DA_RUN <= a, !RUNS || r1 == b);
+        if (!RUNS || r1 == b) break;
+#pragma unroll
+        for (int i = 0; i < 32; ++i) acc[i] = 0.f;
     }
-    block_sums<32>(acc, out, sh);
 }
 
 // Work item (active term or -1 for the empty set, row group, node chunk, chunks; its
 // term): partial sums into part[item]; the last block of a term to finish adds them
 // over the chunks in order and writes the coefficients.  BIG: plans that have
-// a term with more than 96 sums per item.
-template <bool COS, bool BIG>
+// a term with more than 96 sums per item.  RUNS: items of more than DA_RUN nodes.
+template <bool COS, bool BIG, bool RUNS>
 __global__ void __launch_bounds__(DA_THREADS, BIG ? DIRECT_RESIDENT_BIG : DIRECT_RESIDENT)
 direct_adjoint(DevPlan P, const DirectItem *__restrict__ items, const float2 *__restrict__ y, float2 *__restrict__ fhat,
                float *part, int *count) {
     __shared__ float sh[DA_MAX_ACC * (DA_THREADS / 32)];
-    __shared__ double shd[32];
+    __shared__ double shd[32], tot[RUNS ? DA_MAX_ACC : 1];
     __shared__ int s_last;
     if (P.skip && *P.skip) return;
     const DirectItem itm = items[blockIdx.x];
@@ -543,37 +572,37 @@ direct_adjoint(DevPlan P, const DirectItem *__restrict__ items, const float2 *__
         blocks *= adjoint_groups<COS>(T.order, T.K);
         cnt = count + 1 + itm.act;
         if (T.order == 1) {
-            adjoint_order1<COS>(P, T, y, a, b, out, sh);
+            adjoint_order1<COS, RUNS>(P, T, y, a, b, out, sh, tot);
         } else if constexpr (COS) {
             if (T.order == 3) switch (T.K) {
-                case 1: adjoint_rows<1, true, 3>(P, T, y, a, b, out, sh); break;
-                case 2: adjoint_rows<2, true, 3>(P, T, y, a, b, out, sh); break;
-                case 3: adjoint_rows<3, true, 3>(P, T, y, a, b, out, sh); break;
-                default: adjoint_rows<4, true, 3>(P, T, y, a, b, out, sh); break;
+                case 1: adjoint_rows<1, true, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 2: adjoint_rows<2, true, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 3: adjoint_rows<3, true, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                default: adjoint_rows<4, true, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
             } else if (!BIG || T.K <= 5) switch (T.K) {
-                case 1: adjoint_rows<1, true, 2>(P, T, y, a, b, out, sh); break;
-                case 2: adjoint_rows<2, true, 2>(P, T, y, a, b, out, sh); break;
-                case 3: adjoint_rows<3, true, 2>(P, T, y, a, b, out, sh); break;
-                case 4: adjoint_rows<4, true, 2>(P, T, y, a, b, out, sh); break;
-                default: adjoint_rows<5, true, 2>(P, T, y, a, b, out, sh); break;
+                case 1: adjoint_rows<1, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 2: adjoint_rows<2, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 3: adjoint_rows<3, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 4: adjoint_rows<4, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                default: adjoint_rows<5, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
             } else if constexpr (BIG) switch (T.K) {
-                case 6: adjoint_rows<6, true, 2>(P, T, y, a, b, out, sh); break;
-                case 7: adjoint_rows<7, true, 2>(P, T, y, a, b, out, sh); break;
-                case 8: adjoint_rows<8, true, 2>(P, T, y, a, b, out, sh); break;
-                default: adjoint_rows<9, true, 2>(P, T, y, a, b, out, sh); break;
+                case 6: adjoint_rows<6, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 7: adjoint_rows<7, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 8: adjoint_rows<8, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                default: adjoint_rows<9, true, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
             }
         } else {
             if (T.order == 3) switch (T.K) {
-                case 1: adjoint_rows<1, false, 3>(P, T, y, a, b, out, sh); break;
-                case 2: adjoint_rows<2, false, 3>(P, T, y, a, b, out, sh); break;
-                default: adjoint_rows<3, false, 3>(P, T, y, a, b, out, sh); break;
+                case 1: adjoint_rows<1, false, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 2: adjoint_rows<2, false, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                default: adjoint_rows<3, false, 3, RUNS>(P, T, y, a, b, out, sh, tot); break;
             } else if (!BIG || T.K <= 3) switch (T.K) {
-                case 1: adjoint_rows<1, false, 2>(P, T, y, a, b, out, sh); break;
-                case 2: adjoint_rows<2, false, 2>(P, T, y, a, b, out, sh); break;
-                default: adjoint_rows<3, false, 2>(P, T, y, a, b, out, sh); break;
+                case 1: adjoint_rows<1, false, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                case 2: adjoint_rows<2, false, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
+                default: adjoint_rows<3, false, 2, RUNS>(P, T, y, a, b, out, sh, tot); break;
             } else if constexpr (BIG) {
-                if (T.K == 4) adjoint_rows<4, false, 2>(P, T, y, a, b, out, sh);
-                else adjoint_rows<5, false, 2>(P, T, y, a, b, out, sh);
+                if (T.K == 4) adjoint_rows<4, false, 2, RUNS>(P, T, y, a, b, out, sh, tot);
+                else adjoint_rows<5, false, 2, RUNS>(P, T, y, a, b, out, sh, tot);
             }
         }
     }
@@ -807,8 +836,13 @@ int launch_direct_adjoint(Plan &p, const float2 *y, float2 *fhat) {
     }
     if (p.n_items == 0) return ANOVA_OK;
     stage_begin(p, ST_SPREAD);
-    auto k = p.basis == ANOVA_BASIS_COS ? (p.direct_big ? direct_adjoint<true, true> : direct_adjoint<true, false>)
-                                        : (p.direct_big ? direct_adjoint<false, true> : direct_adjoint<false, false>);
+    auto of = [&](auto runs) {
+        constexpr bool R = decltype(runs)::value;
+        return p.basis == ANOVA_BASIS_COS ? (p.direct_big ? direct_adjoint<true, true, R> : direct_adjoint<true, false, R>)
+                                          : (p.direct_big ? direct_adjoint<false, true, R> : direct_adjoint<false, false, R>);
+    };
+    const int C = p.h_ditems[0].chunks;   // the same for every item
+    auto k = (p.M + C - 1) / C > DA_RUN ? of(std::true_type()) : of(std::false_type());
     k<<<p.n_items, DA_THREADS, 0, p.stream>>>(v, p.direct_items, y, fhat, p.direct_part, p.direct_count);
     stage_end(p, ST_SPREAD);
     return cuda_status(cudaGetLastError());

@@ -187,6 +187,12 @@ __device__ __forceinline__ void term_rows(const DirectTerm &T, const float4 *st,
     }
 }
 
+// Units that a warp adds in one FP32 chain (up to 9 rows each) before their sum goes to
+// its total, kept in shared memory (in registers it spilled): the error of a chain grows
+// with the root of its length, and one over the 58 units of a warp at d = 30, N = 16/8
+// left 2.8e-7 at M = 3e4 where the NFFT has 2.1e-7.
+constexpr int DT_CHAIN = 8;
+
 // A CTA takes 32 NPL nodes and every gridDim.y-th set of work units (active term,
 // frequency group of order 1), its warps one unit each in turn; the warps' sums are
 // added in order, and so are the CTAs' of a node block by the last one to finish
@@ -216,9 +222,19 @@ direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f,
     }
     __syncthreads();
     float4 *st = stage + warp * DIRECT_MAX_COEF;
+    const int first = blockIdx.y * NW + warp, step = NW * gridDim.y;
     float2 acc[NPL];
+    float2 *sum = red + warp * NB + lane;   // this lane's sums of the chains before
 #pragma unroll
-    for (int u = 0; u < NPL; ++u) acc[u] = make_float2(0.f, 0.f);
+    for (int u = 0; u < NPL; ++u) sum[32 * u] = acc[u] = make_float2(0.f, 0.f);
+    auto end_chain = [&]() {
+#pragma unroll
+        for (int u = 0; u < NPL; ++u) {
+            sum[32 * u] = make_float2(sum[32 * u].x + acc[u].x, sum[32 * u].y + acc[u].y);
+            acc[u] = make_float2(0.f, 0.f);
+        }
+    };
+    int chain_end = first + DT_CHAIN * step;
     // A unit's coefficients are loaded while the unit before it is summed, and its
     // record before that: a lane holds up to three pairs (c_k, c_-k) of a term of
     // order >= 2 (cosine: three coefficients), an order-1 group all its coefficients.
@@ -243,12 +259,15 @@ direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f,
             }
         }
     };
-    const int first = blockIdx.y * NW + warp, step = NW * gridDim.y;
     DirectTerm next, after;
     if (first < n_units) next = units[first];
     if (first + step < n_units) after = units[first + step];
     if (first < n_units) prefetch(next);
     for (int s = first; s < n_units; s += step) {
+        if (s == chain_end) {
+            end_chain();
+            chain_end += DT_CHAIN * step;
+        }
         const DirectTerm T = next;
         if (T.order == 1) {
             next = after;
@@ -324,8 +343,7 @@ direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f,
                 }
         }
     }
-#pragma unroll
-    for (int u = 0; u < NPL; ++u) red[warp * NB + lane + 32 * u] = acc[u];
+    end_chain();
     __syncthreads();
     const int S = gridDim.y;
     auto write = [&](int u, float2 v) {

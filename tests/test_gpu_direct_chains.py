@@ -51,3 +51,34 @@ def test_adjoint_over_many_nodes(gft, basis, bws, M):
     off = np.concatenate([[0], np.cumsum([(b - 1) ** len(u) for u, b in zip(terms, bw)])])
     got = np.concatenate([g[off[u]:off[u + 1]] for u in pick])
     assert rel_l2(got, ref) <= 8 * U
+
+
+@pytest.mark.parametrize("basis,bws", [(0, (16, 4, 2)), (0, (16, 8)), (1, (9, 3, 2)), (1, (20, 8))])
+@pytest.mark.parametrize("M", [60, 2500, 30001])
+def test_forward_over_many_terms(gft, basis, bws, M):
+    """A warp's chain is at most 8 units of 9 rows of two additions (144: 4.9 u), its
+    total at most one addition per 8 of 566 units (3.4 u), the products 2 u: 6.3 u as
+    independent errors, bound 8 u."""
+    P, terms, bw, x = _plan(gft, basis, 30, bws, M)
+    fhat = inputs.complex_normal(3, 2, P.n_coeffs)
+    f = host(P.trafo(cplx_dev(fhat)))
+    pick = np.linspace(0, M - 1, min(M, 500)).astype(int)
+    ref = (ndct if basis else ndft).trafo(x[:, pick], terms, bw, fhat)
+    assert rel_l2(f[pick], ref) <= 8 * U
+
+
+def test_forward_over_many_terms_and_nodes(gft):
+    """Enough nodes that a block's eight warps share all 4526 terms: rows of about 700 in
+    one chain would leave 15 u."""
+    import torch
+    d, M, bws = 30, 4000000, (16, 4, 2)
+    terms = [u for s in range(4) for u in itertools.combinations(range(d), s)]
+    bw = [bws[len(u) - 1] if u else 0 for u in terms]
+    x = torch.rand(d, M, generator=torch.Generator("cuda").manual_seed(5), device="cuda") - 0.5
+    P = gft.Plan(x, terms, bw)
+    assert gft.anova_debug_plan_form(P.handle) == gft.FORM_DIRECT
+    fhat = inputs.complex_normal(3, 2, P.n_coeffs)
+    f = P.trafo(cplx_dev(fhat))
+    pick = torch.linspace(0, M - 1, 500, dtype=torch.float64, device="cuda").long()
+    ref = ndft.trafo(f32_nodes(x[:, pick].cpu().numpy()), terms, bw, fhat)
+    assert rel_l2(host(f[pick]), ref) <= 8 * U

@@ -105,12 +105,14 @@ __device__ __forceinline__ void mma3_tf32_0(float (&d)[4], const unsigned (&ah)[
 
 // ---- FP16 tensor-core products of scaled operands ----
 //
-// x = h + l with h the leading 11 bits of x (exact in FP16) and l the remainder
-// rounded to FP16: for |x| in [2^-4, 2^15] the two hold 21 bits of x, and below
-// that the error is at most 2^-25 in absolute size.  Operands bounded by 1 are used as they are;
-// others are scaled by a power of two to a maximum near 2^14, so what is lost
-// is below 2^-22 of the value or 2^-39 of the largest one.  Products are h h +
-// l h + h l as in the TF32 form, at twice its rate (m16n8k16).
+// x = h + l with h the nearest FP16 value and l the remainder rounded to FP16: for |x|
+// in [2^-3, 2^15] the two hold 22 bits of x, and below that the error is at most 2^-25
+// in absolute size.  Operands bounded by 1 are used as they are; others are scaled by a
+// power of two to a maximum near 2^14, so what is lost is below 2^-22 of the value or
+// 2^-39 of the largest one.  Products are h h + l h + h l as in the TF32 form, at twice
+// its rate (m16n8k16).  h is rounded, not cut off: remainders of one sign left out a
+// product l l of the result's own sign, 1.2e-7 of the adjoint (d = 10, M = 5e5 adjoint
+// 3.11 -> 3.14 ms, forward 2.94 -> 2.95; rounding by the TF32 form's packed split: 3.56).
 // Fragments (PTX ISA), lane = 4 g + t: A (16 x 16) a0 = A[g][2t, 2t+1], a1 =
 // A[g + 8][2t, 2t+1], a2 = A[g][2t + 8, 2t + 9], a3 = A[g + 8][2t + 8, 2t + 9]; B
 // (16 x 8) b0 = B[2t, 2t+1][g], b1 = B[2t + 8, 2t + 9][g]; the k8 form has a0, a1
@@ -120,12 +122,12 @@ __device__ __forceinline__ unsigned pack_f16(float lo, float hi) {
     asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
-// (x0, x1) in high parts (the leading 11 bits) and remainders
+// (x0, x1) in high parts and remainders
 __device__ __forceinline__ void split_f16(float x0, float x1, unsigned &h, unsigned &l) {
-    const float h0 = __uint_as_float(__float_as_uint(x0) & 0xffffe000u);
-    const float h1 = __uint_as_float(__float_as_uint(x1) & 0xffffe000u);
-    h = pack_f16(h0, h1);
-    l = pack_f16(x0 - h0, x1 - h1);
+    const __half2 hh = __floats2half2_rn(x0, x1);
+    const float2 hf = __half22float2(hh);
+    h = *(const unsigned *)&hh;
+    l = pack_f16(x0 - hf.x, x1 - hf.y);
 }
 __device__ __forceinline__ void mma_f16_k16(float (&d)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
     asm("mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, "

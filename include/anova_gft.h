@@ -160,7 +160,9 @@ int anova_term_grid(anova_plan_t plan, int u, int *n, int *m_col, int *m_row);
  * point, so the result is bitwise reproducible for a plan.  FP32 plans need
  * the oversampled grid values (about sum_k |fhat_k| at most) below 2^114
  * (2e34) in magnitude: the tensor-core kernels split each operand x into two
- * TF32 parts through 8193 x, which must stay finite.
+ * TF32 parts through 8193 x, which must stay finite.  A coefficient that is
+ * not finite leaves no f_j finite, a node coordinate that is not finite leaves
+ * f at that node not finite.
  */
 int grouped_trafo(anova_plan_t plan, const void *fhat_dev, void *f_dev);
 

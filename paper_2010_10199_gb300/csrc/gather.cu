@@ -362,9 +362,14 @@ static void launch_mr(cudaStream_t st, const DevPlan &v, const BatchArgs &B, con
     }
 }
 
+static size_t gather_smem(long long max_grid_bytes, int dmax) {
+    return (size_t)max_grid_bytes * 2 + (size_t)dmax * G2_TILE * 4 + 64;   // + barriers, counters
+}
+bool gather_fits(long long max_grid_bytes, int dmax) { return gather_smem(max_grid_bytes, dmax) <= (size_t)MAX_SMEM; }
+
 int gather_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, const float2 *fhat, float2 *f,
                   int n_tiles, int mr, int pitch, long long max_grid_bytes, int dmax, int sm_count, int prec) {
-    const size_t smem = (size_t)max_grid_bytes * 2 + (size_t)dmax * G2_TILE * 4 + 64;   // + barriers, counters
+    const size_t smem = gather_smem(max_grid_bytes, dmax);
     if (smem > (size_t)MAX_SMEM) return ANOVA_ERR_UNSUPPORTED;
     if (n_tiles <= 0) return ANOVA_OK;
     const int per_sm = smem * 2 <= (size_t)MAX_SMEM ? 2 : 1;

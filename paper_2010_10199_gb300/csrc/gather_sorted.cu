@@ -51,7 +51,8 @@ __global__ void k_fixed_point_finish(DevPlan single, BatchArgs B, const float2 *
         c0.x += c.x;
         c0.y += c.y;
     }
-    const double sc = ldexp(1.0, -*P.fexp);
+    // a coefficient that is not finite reaches every node (the accumulators hold no such value)
+    const double sc = P.fexp[2] ? __longlong_as_double(0x7ff8000000000000LL) : ldexp(1.0, -*P.fexp);
     float2 *__restrict__ f = f_base + P.vec_node_off;
     longlong2 *__restrict__ acc = (longlong2 *)P.facc;
     const long long M = P.M, step = (long long)gridDim.x * blockDim.x;

@@ -156,7 +156,7 @@ struct DevPlan {
     const int *tile_cell;     // cell of every tile (null: srec holds records)
     const int *tile_count;    // tiles per scheduled term
     unsigned long long *facc; // sorted forward: fixed-point accumulators [M][2] (or null), zero between calls
-    int *fexp;                // their exponent, and a block counter (zero between launches)
+    int *fexp;                // their exponent, a block counter (zero between launches), 1 if a coefficient is not finite
     long long n_coeffs;
     long long vec_node_off;   // offset of this problem's nodes in batched node vectors
     long long vec_coef_off;   // offset of this problem's coefficients in batched coefficient vectors
@@ -176,9 +176,9 @@ struct BatchArgs {
     const int *blk0;          // first block of each problem
 };
 
-// words of DevPlan::err: the error code of bounded waits; the largest |Re|, |Im| of
-// the adjoint's input (float bits, zero between calls)
-enum { ERR_CODE = 0, ERR_YMAX = 2 };
+// words of DevPlan::err: the error code of bounded waits; 1 if a node coordinate is not
+// finite; the largest |Re|, |Im| of the adjoint's input (float bits, zero between calls)
+enum { ERR_CODE = 0, ERR_NODE = 1, ERR_YMAX = 2 };
 
 constexpr int N_STAGES = 7;
 // How a plan keeps its nodes, and so which kernels read them.
@@ -309,8 +309,9 @@ double deconv_factor(int k, int n, int m, double b);
 void window_polys(Window &w, int m, double b);
 int fft_size(int N, double sigma);
 int row_stride(int n);
-// out = in * scale wrapped into [-1/2, 1/2) (scale 1/2 for cosine plans: x in [0, 1] -> x / 2)
-__global__ void wrap_nodes_f32(const float *in, float *out, long long total, float scale);
+// out = in * scale wrapped into [-1/2, 1/2) (scale 1/2 for cosine plans: x in [0, 1] -> x / 2);
+// *bad = 1 for a coordinate that is not finite (bad: may be null)
+__global__ void wrap_nodes_f32(const float *in, float *out, long long total, float scale, int *bad);
 
 // stage timing: call stage_begin before and stage_end after a kernel launch
 void stage_begin(Plan &p, int stage);
@@ -321,6 +322,7 @@ enum { ST_PRE = 0, ST_GATHER = 1, ST_SPREAD = 2, ST_REDUCE = 3, ST_POST = 4, ST_
 // kernels launched by the entry points (trafo.cu / adjoint.cu)
 int launch_trafo_f32(Plan &p, const float2 *fhat, float2 *f);
 int launch_gather_f32(Plan &p, const float2 *fhat, float2 *f);
+bool gather_fits(long long max_grid_bytes, int dmax);   // its shared memory
 // Sorted forward (gather_sorted.cu), every term over its cell-sorted records:
 // f = empty-set coefficient + all terms.
 int launch_gather_sorted_f32(Plan &p, const float2 *fhat, float2 *f);

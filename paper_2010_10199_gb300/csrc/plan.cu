@@ -130,12 +130,13 @@ int row_stride(int n) {
     return s;
 }
 
-__global__ void wrap_nodes_f32(const float *in, float *out, long long total, float scale) {
+__global__ void wrap_nodes_f32(const float *in, float *out, long long total, float scale, int *bad) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         float v = in[i] * scale;
         v = v - floorf(v + 0.5f);   // into [-1/2, 1/2)
         if (v >= 0.5f) v -= 1.0f;
+        if (bad && v != v) *bad = 1;
         out[i] = v;
     }
 }
@@ -776,14 +777,22 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
                                                           cosine ? 0.5 : 1.0);
         else
             wrap_nodes_f32<<<blocks, 256, 0, p.stream>>>((const float *)x_dev, (float *)p.x, total,
-                                                          cosine ? 0.5f : 1.0f);
+                                                          cosine ? 0.5f : 1.0f, p.err + ERR_NODE);
         chk(cudaGetLastError());
     }
     if (e == cudaSuccess && p.precision == ANOVA_PREC_F64) chk(cuda_err_of(build_window_tables_f64(p)));
     if (e == cudaSuccess && p.direct) chk(cuda_err_of(build_unit_table(p)));
     if (e == cudaSuccess) chk(cuda_err_of(sort_nodes_by_cell(p)));
     if (e == cudaSuccess) chk(cuda_err_of(set_active_terms(p, nullptr)));
+    int bad_node = 0;
+    if (p.facc) chk(cudaMemcpyAsync(&bad_node, p.err + ERR_NODE, sizeof(int), cudaMemcpyDeviceToHost, p.stream));
     chk(cudaStreamSynchronize(p.stream));
+    // the fixed-point accumulators hold no NaN: a plan with a node that is not finite sums
+    // point-major, where that node alone is NaN
+    if (bad_node && gather_fits(p.max_grid_bytes, p.d)) {
+        p.facc = nullptr;
+        p.fexp = nullptr;
+    }
     // wins vector is copied; keep host term table
     if (e != cudaSuccess) {
         cudaGetLastError();

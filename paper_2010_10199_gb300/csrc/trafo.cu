@@ -121,9 +121,11 @@ __device__ __forceinline__ void trafo_pre_body(const DevPlan &single, const Batc
         int e = 100;
         // a cosine coefficient stands for 2^s exponential ones of 2^{-s/2} its size
         // (s <= 3): their absolute sum is at most 2^{3/2} = 2.83 times larger
-        if (sum > 0) e = 61 - (int)ceil(log2(sum)) - (P.basis == ANOVA_BASIS_COS ? 2 : 0);
+        const bool finite = sum <= 1.7976931348623157e308;
+        if (sum > 0 && finite) e = 61 - (int)ceil(log2(sum)) - (P.basis == ANOVA_BASIS_COS ? 2 : 0);
         P.fexp[0] = max(-100, min(100, e));
         P.fexp[1] = 0;
+        P.fexp[2] = !finite;   // fixed point holds no infinity: the finish writes NaN
     }
 }
 

@@ -92,7 +92,12 @@ enum anova_status {
     ANOVA_ERR_NOT_FINITE = -7    /* a solver scalar became NaN or Inf */
 };
 
-/* Options of anova_plan_create; zero-initialise and set what you need. */
+/* Options of anova_plan_create; zero-initialise and set what you need.
+ * FP32 plans whose terms all have small bandwidths (N up to 10 for order 2, 6 for
+ * order 3, 256 for order 1; cosine N up to 10, 5, 129) may sum the transforms directly,
+ * without grids, where a cost model finds that faster.  sigma, window_m_col,
+ * window_m_row, n_ctas, node_sort and cell_kernel name parts of the NFFT: setting any
+ * of them keeps the plan on it. */
 typedef struct {
     int precision;      /* enum anova_precision */
     double eps;         /* target relative l2 error of F and F^H (0: default for the precision) */
@@ -146,7 +151,8 @@ int64_t anova_num_coeffs(anova_plan_t plan);
 /* Offset and length of block u in the coefficient vector. */
 int anova_term_offset(anova_plan_t plan, int u, int64_t *off, int64_t *len);
 
-/* Oversampled grid size n_u and window half-widths (col, row) chosen for term u. */
+/* Oversampled grid size n_u and window half-widths (col, row) chosen for term u (a plan
+ * that sums directly uses neither). */
 int anova_term_grid(anova_plan_t plan, int u, int *n, int *m_col, int *m_row);
 
 /*

@@ -605,11 +605,13 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     int kmax = (int)std::min<long long>(std::min<long long>(SPREAD_MAX_K, k_cap),
                                         std::max<long long>(1, (M + 2047) / 2048));
     if (o.n_ctas > 0) kmax = std::min(o.n_ctas, SPREAD_MAX_K);
-    // small bandwidths in every term: the sums themselves, where they are faster
-    // (default options only: the others ask for a path of the NFFT)
+    // small bandwidths in every term: the sums themselves, where they are faster.  An
+    // oversampling factor, a window, chunks, a node order or a cell kernel in the options
+    // ask for the NFFT; a target error does not (the sums meet any).
+    const bool asks_nfft = (opts && (opts->sigma > 0 || opts->window_m_row > 0 || opts->window_m_col > 0)) ||
+                           o.node_sort != 0 || o.cell_kernel != 0 || o.n_ctas > 0;
     long long d_groups = p.n_empty > 0 ? 1 : 0, d_units = 0;
-    if (allow_direct && p.precision == ANOVA_PREC_F32 && o.node_sort == 0 && o.cell_kernel == 0 &&
-        o.n_ctas <= 0 && M > 0 && p.n_terms > 0) {
+    if (allow_direct && !asks_nfft && p.precision == ANOVA_PREC_F32 && M > 0 && p.n_terms > 0) {
         double t_direct = DIRECT_FIXED_NS, t_nfft = NFFT_FIXED_NS;
         p.direct = true;
         for (int s = 0; s < p.n_terms && p.direct; ++s) {

@@ -399,8 +399,9 @@ int anova_profile_read(anova_plan_t plan, double *ms, int64_t *launches, const c
  * error is the largest relative l2 distance to the reference of F fhat, of
  * F^H y and of each coefficient block of F^H y on its own, and its time is
  * the mean of `reps` timed pairs after one warm-up pair on `stream`.
- * Candidates: sigma in {1.75, 2, 2.5} x row half-width in {3, 4}; then, around
- * the fastest one within eps_target, node chunks per term (n_ctas) in
+ * Candidates: the default options (sigma 0, window_m_row 0), where such a plan sums
+ * directly; sigma in {1.75, 2, 2.5} x row half-width in {3, 4}; then, around
+ * the fastest of these within eps_target, node chunks per term (n_ctas) in
  * {4, 16, 64}, the original node order (node_sort = -1) and the CUDA-core
  * cell kernels (cell_kernel = 1).
  *   opts       : in: base options (precision must be ANOVA_PREC_F32);

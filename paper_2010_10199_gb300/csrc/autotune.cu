@@ -4,7 +4,8 @@
 // list, by timing transform pairs of
 // candidate plans on the device and estimating each candidate's error against
 // a wider-window, more oversampled reference plan (the NFFT error falls with
-// both, Sec. 3 after eq. (somafm)).  The fastest candidate whose estimated
+// both, Sec. 3 after eq. (somafm)).  Where a plan with default options sums
+// directly it is a candidate too.  The fastest candidate whose estimated
 // error meets the target wins.
 #include <algorithm>
 #include <cmath>
@@ -197,10 +198,16 @@ int anova_plan_autotune(anova_plan_options *opts, int d, int64_t M, const void *
         bool ok;
     };
     std::vector<Cand> done;
-    auto trial = [&](const anova_plan_options &o) -> int {
+    // the plan that a caller gets for these options; only_direct: a candidate only if it sums directly
+    auto trial = [&](const anova_plan_options &o, bool only_direct) -> int {
         Cand c{o, INFINITY, INFINITY, false};
         anova_plan_t p = nullptr;
-        int r = plan_create(&p, d, M, x_dev, n_terms, term_dims, bandwidth, &o, stream, false);
+        int r = anova_plan_create(&p, d, M, x_dev, n_terms, term_dims, bandwidth, &o, stream);
+        if (only_direct && (r || !p->p.direct)) {
+            cudaGetLastError();
+            anova_plan_destroy(p);
+            return r == ANOVA_ERR_UNSUPPORTED || r == ANOVA_ERR_NOMEM ? ANOVA_OK : r;
+        }
         if (r == ANOVA_ERR_UNSUPPORTED || r == ANOVA_ERR_NOMEM) {
             cudaGetLastError();
             done.push_back(c);   // not buildable: recorded, never chosen
@@ -230,46 +237,51 @@ int anova_plan_autotune(anova_plan_options *opts, int d, int64_t M, const void *
         done.push_back(c);
         return r;
     };
-    auto best = [&]() -> int {
+    auto best = [&](int from) -> int {
         int b = -1;
-        for (int i = 0; i < (int)done.size(); ++i)
+        for (int i = from; i < (int)done.size(); ++i)
             if (done[i].ok && (b < 0 || done[i].ms < done[b].ms)) b = i;
         return b;
     };
-    // stage 1: oversampling and row window, default chunks and node order
+    // stage 1: default options, oversampling and row window, default chunks and node order
+    anova_plan_options def = *opts;
+    def.sigma = 0.0;
+    def.window_m_row = 0;
+    def.n_ctas = 0;
+    def.node_sort = 0;
+    def.cell_kernel = 0;
+    rc = trial(def, true);
+    const int nfft0 = (int)done.size();   // the first NFFT candidate
     for (double sg : {1.75, 2.0, 2.5})
         for (int mr : {3, 4}) {
-            anova_plan_options o = *opts;
+            if (rc) break;
+            anova_plan_options o = def;
             o.sigma = sg;
             o.window_m_row = mr;
-            o.n_ctas = 0;
-            o.node_sort = 0;
-            o.cell_kernel = 0;
-            rc = trial(o);
-            if (rc) break;
+            rc = trial(o, false);
         }
-    // stage 2: node chunks per term and node order around the best so far
-    int b = rc ? -1 : best();
+    // stage 2: node chunks per term and node order around the best of the NFFT so far
+    int b = rc ? -1 : best(nfft0);
     if (b >= 0) {
         const anova_plan_options base = done[b].o;
         for (int k : {4, 16, 64}) {
             anova_plan_options o = base;
             o.n_ctas = k;
-            rc = trial(o);
+            rc = trial(o, false);
             if (rc) break;
         }
         if (!rc) {
             anova_plan_options o = base;
             o.node_sort = -1;
-            rc = trial(o);
+            rc = trial(o, false);
         }
         if (!rc) {
             anova_plan_options o = base;
             o.cell_kernel = 1;
-            rc = trial(o);
+            rc = trial(o, false);
         }
-        b = best();
     }
+    if (!rc) b = best(0);
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     for (int i = 0; i < (int)done.size(); ++i) {

@@ -476,8 +476,8 @@ int grouped_trafo_noalloc(int d, int64_t M, const float *x_dev, int n_terms, con
  * of memory; the allocations after it succeed again.  k = 0 cancels a pending
  * failure.  A failing plan creation returns ANOVA_ERR_NOMEM after freeing
  * everything it had allocated, or -- where the failed allocation was an
- * optional one (the cell-sorted node copy, the fixed-point accumulators) --
- * builds the plan without it.  Process-wide; not for concurrent use.
+ * optional one (the cell-sorted node copy, the fixed-point accumulators, what
+ * only direct sums need) -- builds the plan without it.  Process-wide; not for concurrent use.
  * Errors: ANOVA_ERR_INVALID for k < 0.
  */
 int anova_debug_fail_allocation(int k);

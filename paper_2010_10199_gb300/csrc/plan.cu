@@ -280,16 +280,17 @@ struct Arena {
     };
     std::vector<Part> parts;
     size_t bytes = 0;
-    bool failed = false;
+    bool failed = false, lost = false;   // an injected failure: of any part, of an optional one
     template <typename T>
-    void want(T **ptr, size_t n) {   // n = 0: *ptr stays null
+    void want(T **ptr, size_t n, bool optional = false) {   // n = 0: *ptr stays null
         if (n == 0) return;
-        failed = alloc_fault() || failed;
+        bool &f = optional ? lost : failed;
+        f = alloc_fault() || f;
         parts.push_back({(void **)ptr, bytes});
         bytes = (bytes + n + 255) & ~(size_t)255;
     }
     cudaError_t commit(void **base) {
-        cudaError_t e = failed ? cudaErrorMemoryAllocation : cudaMalloc(base, bytes);
+        cudaError_t e = failed || lost ? cudaErrorMemoryAllocation : cudaMalloc(base, bytes);
         if (e != cudaSuccess) {
             *base = nullptr;
             return e;
@@ -342,8 +343,10 @@ const char *anova_version(void) { return "anova-gft 0.1 (sm_103a)"; }
 
 }  // extern "C"
 
+// direct_nomem: set when a plan to be summed directly found no memory for what only it needs
 static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct) {
+                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct,
+                  bool *direct_nomem) {
     if (!out) return ANOVA_ERR_INVALID;
     *out = nullptr;
     cudaGetLastError();   // do not report an earlier, unrelated error
@@ -652,17 +655,17 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     mem.want(&p.act_rec, sizeof(ActRec) * nt1);
     mem.want(&p.act_rec3, sizeof(ActRec) * nt1);
     mem.want(&p.items, sizeof(int4) * n_items);
-    mem.want(&p.direct_units, p.direct ? sizeof(DirectTerm) * d_units : 0);
-    mem.want(&p.direct_items, sizeof(DirectItem) * n_ditems);
+    mem.want(&p.direct_units, p.direct ? sizeof(DirectTerm) * d_units : 0, true);
+    mem.want(&p.direct_items, sizeof(DirectItem) * n_ditems, true);
     mem.want(&p.err, sizeof(int) * 4);
     mem.want(&p.counter, 2 * sizeof(int));
-    mem.want(&p.direct_fcount, sizeof(int) * f_blocks);
-    mem.want(&p.direct_count, p.direct ? sizeof(int) * (nt1 + 1) : 0);
+    mem.want(&p.direct_fcount, sizeof(int) * f_blocks, true);
+    mem.want(&p.direct_count, p.direct ? sizeof(int) * (nt1 + 1) : 0, true);
     mem.want(&p.x, xbytes);
     if (p.direct) {
-        mem.want(&p.z, sizeof(float2) * (size_t)d * M);
-        mem.want(&p.direct_part, sizeof(float) * DA_MAX_ACC * n_ditems);
-        mem.want(&p.direct_fpart, p.direct_split > 1 ? sizeof(float2) * (size_t)p.direct_split * M : 0);
+        mem.want(&p.z, sizeof(float2) * (size_t)d * M, true);
+        mem.want(&p.direct_part, sizeof(float) * DA_MAX_ACC * n_ditems, true);
+        mem.want(&p.direct_fpart, p.direct_split > 1 ? sizeof(float2) * (size_t)p.direct_split * M : 0, true);
     } else {
         mem.want(&p.grids, (size_t)std::max<long long>(1, p.grid_elems) * esize);
         mem.want(&p.partials, p.n_terms > 0 ? (size_t)kmax * (size_t)p.grid_elems * esize : 0);
@@ -677,12 +680,14 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     if (p.direct) {
         p.h_units = plan_new<DirectTerm>(d_units);
         p.h_ditems = plan_new<DirectItem>(n_ditems);
-        if (!p.h_units || !p.h_ditems) return ANOVA_ERR_NOMEM;
+        mem.lost = mem.lost || !p.h_units || !p.h_ditems;
     }
     if (!p.h_act || !p.h_items) return ANOVA_ERR_NOMEM;
     e = mem.commit(&p.arena);
     if (e != cudaSuccess) {
         cudaGetLastError();
+        // exp(2 pi i x) takes twice the nodes' memory: the NFFT may fit where the sums do not
+        *direct_nomem = p.direct && !mem.failed && e == cudaErrorMemoryAllocation;
         return cuda_status(e);
     }
     // cell-sorted node copies, if they fit in half the free device memory: node
@@ -808,7 +813,11 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
 int agft::plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
                       const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct) {
     try {
-        return create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, allow_direct);
+        bool direct_nomem = false;
+        int rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, allow_direct, &direct_nomem);
+        if (direct_nomem)
+            rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, false, &direct_nomem);
+        return rc;
     } catch (const std::bad_alloc &) {
         return ANOVA_ERR_NOMEM;
     } catch (...) {

@@ -693,13 +693,10 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     // cell-sorted node copies, if they fit in half the free device memory: node
     // tiles (tiles.cuh) for the tensor-core kernels, else records of 16 bytes per
     // node (32 for order 3; FP64 plans sort order <= 2 only), whose sort_slot
-    // counts units of M records of 16 bytes
-    if (o.node_sort >= 0 && M > 0 && p.n_terms > 0 && !p.direct) {
-        bool tiles = !f64 && o.cell_kernel == 0;
-        for (int s = 0; s < p.n_terms && tiles; ++s) {   // a tile's places are 32-bit
-            const Term &T = p.h_terms[s];
-            tiles = tile_capacity(M, T.order == 1 ? T.n : (long long)T.n * T.n * (T.order == 3 ? T.n : 1)) * TILE < (1LL << 31);
-        }
+    // counts units of M records of 16 bytes.  Padding makes tiles the larger form
+    // below 48 nodes per cell, up to twelve times at one node per cell: records may
+    // fit where tiles do not.
+    auto keep_sorted = [&](bool tiles) {
         long long n_rec = 0, n_tiles = 0;   // float4 records, tiles
         std::vector<int> slot(p.n_terms, -1);
         for (int s = 0; s < p.n_terms; ++s) {
@@ -725,38 +722,46 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
         }
         size_t free_b = 0, total_b = 0;
         const size_t need = (size_t)n_rec * sizeof(float4) + (size_t)n_tiles * sizeof(int);
-        if (n_rec > 0 && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess && need <= free_b / 2) {
-            auto sorted_parts = [&](Arena &A) {
-                A.want(&p.srec, (size_t)n_rec * sizeof(float4));
-                A.want(&p.tile_cell, (size_t)n_tiles * sizeof(int));
-                A.want(&p.tile_count, tiles ? sizeof(int) * p.n_terms : 0);
-            };
-            Arena opt;
-            sorted_parts(opt);
-            bool ok = !opt.failed, acc = p.precision == ANOVA_PREC_F32;
-            if (ok && acc) {
-                opt.want(&p.facc, sizeof(unsigned long long) * 2 * (size_t)M);
-                opt.want(&p.fexp, sizeof(int) * 4);
-                if (opt.failed || opt.commit(&p.arena_opt) != cudaSuccess) acc = false;
-            }
-            if (ok && !acc) {   // without accumulators the forward is the point-major gather
-                cudaGetLastError();
-                p.facc = nullptr;
-                p.fexp = nullptr;
-                Arena only;
-                sorted_parts(only);
-                ok = !only.failed && only.commit(&p.arena_opt) == cudaSuccess;
-            }
-            if (ok) {
-                for (int s = 0; s < p.n_terms; ++s) p.h_terms[s].sort_slot = slot[s];
-                p.n_sorted = tiles ? p.n_terms : (int)(n_rec / M);
-                p.cell_tc = tiles;
-            } else {
-                cudaGetLastError();
-                p.srec = nullptr;
-                p.tile_cell = p.tile_count = nullptr;
-            }
+        if (n_rec == 0 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need > free_b / 2) return false;
+        auto sorted_parts = [&](Arena &A) {
+            A.want(&p.srec, (size_t)n_rec * sizeof(float4));
+            A.want(&p.tile_cell, (size_t)n_tiles * sizeof(int));
+            A.want(&p.tile_count, tiles ? sizeof(int) * p.n_terms : 0);
+        };
+        Arena opt;
+        sorted_parts(opt);
+        bool ok = !opt.failed, acc = p.precision == ANOVA_PREC_F32;
+        if (ok && acc) {
+            opt.want(&p.facc, sizeof(unsigned long long) * 2 * (size_t)M);
+            opt.want(&p.fexp, sizeof(int) * 4);
+            if (opt.failed || opt.commit(&p.arena_opt) != cudaSuccess) acc = false;
         }
+        if (ok && !acc) {   // without accumulators the forward is the point-major gather
+            cudaGetLastError();
+            p.facc = nullptr;
+            p.fexp = nullptr;
+            Arena only;
+            sorted_parts(only);
+            ok = !only.failed && only.commit(&p.arena_opt) == cudaSuccess;
+        }
+        if (!ok) {
+            cudaGetLastError();
+            p.srec = nullptr;
+            p.tile_cell = p.tile_count = nullptr;
+            return false;
+        }
+        for (int s = 0; s < p.n_terms; ++s) p.h_terms[s].sort_slot = slot[s];
+        p.n_sorted = tiles ? p.n_terms : (int)(n_rec / M);
+        p.cell_tc = tiles;
+        return true;
+    };
+    if (o.node_sort >= 0 && M > 0 && p.n_terms > 0 && !p.direct) {
+        bool tiles = !f64 && o.cell_kernel == 0;
+        for (int s = 0; s < p.n_terms && tiles; ++s) {   // a tile's places are 32-bit
+            const Term &T = p.h_terms[s];
+            tiles = tile_capacity(M, T.order == 1 ? T.n : (long long)T.n * T.n * (T.order == 3 ? T.n : 1)) * TILE < (1LL << 31);
+        }
+        if (!tiles || !keep_sorted(true)) keep_sorted(false);
     }
     {   // the tables in one copy
         std::vector<unsigned char> host(table_bytes);

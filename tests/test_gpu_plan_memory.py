@@ -1,5 +1,5 @@
 """Plans where memory for a form of the nodes is lacking take one that needs less: the NFFT
-in place of direct sums."""
+in place of direct sums, records in place of tiles."""
 import numpy as np
 import pytest
 
@@ -64,3 +64,10 @@ def test_direct_sums_without_memory_become_the_nfft(gft):
     # sums, two host lists
     assert forms.count(gft.FORM_TILES) == 9
     assert forms.count(None) >= 20 and forms[-1] == gft.FORM_DIRECT
+
+
+def test_tiles_without_memory_become_records(gft):
+    forms = _forms_under_failures(gft, n_ctas=4)
+    # the tiles, their cells and their counts; without accumulators the tiles stay
+    assert forms.count(gft.FORM_RECORDS) == 3 and gft.FORM_OWN_ORDER not in forms
+    assert forms.count(None) >= 20 and forms[-1] == gft.FORM_TILES

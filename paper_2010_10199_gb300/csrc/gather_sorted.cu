@@ -128,7 +128,7 @@ gather_sorted_f32(DevPlan single, BatchArgs B, const int4 *__restrict__ items, i
             }
         }
         __syncthreads();
-        const float4 *rec = P.srec + (long long)T.sort_slot * M;
+        const float4 *rec = P.frec + (long long)T.sort_slot * M;
         const int stride = T.stride;
         const bool two = T.order == 2;
         if (T.order == 3) {
@@ -285,7 +285,7 @@ int launch_gather_sorted_f32(Plan &p, const float2 *fhat, float2 *f) {
     for (int s = 0; s < p.n_terms; ++s)
         if (p.h_terms[s].mr > 0) mr = p.h_terms[s].mr;
     return gather_sorted_launch(p.stream, v, B, 1, fhat, f, p.items, p.n_items3, p.n_items, p.counter,
-                                p.max_grid_bytes, p.M, p.sm_count, mr, p.cell_tc);
+                                p.max_grid_bytes, p.M, p.sm_count, mr, p.cell_tc && !p.frec);
 }
 
 }  // namespace agft

@@ -153,6 +153,7 @@ struct DevPlan {
     float2 *partials;         // adjoint partial grids [spread_chunks][grid_elems]
     int spread_chunks;        // node chunks of the adjoint (one partial grid each)
     const float4 *srec;       // nodes sorted by grid cell: [slot][M] records, or node tiles if tile_cell is set
+    const float4 *frec;       // records of the forward on the CUDA cores (srec, or a copy beside tiles; null: tiles only)
     const int *tile_cell;     // cell of every tile (null: srec holds records)
     const int *tile_count;    // tiles per scheduled term
     unsigned long long *facc; // sorted forward: fixed-point accumulators [M][2] (or null), zero between calls
@@ -247,6 +248,8 @@ struct Plan {
     int *counter;           // work-queue counters (2), zero between calls
     float4 *srec;           // cell-sorted node records (null: none), n_sorted slots of M
     bool cell_tc;           // srec holds node tiles: cell products on the tensor cores
+    float4 *frec;           // records beside tiles, for the forward (n_frec slots of M; null: none)
+    int n_frec;
     int *tile_cell;         // tiles: their cells, and the tiles per scheduled term
     int *tile_count;
     int n_sorted;
@@ -363,10 +366,10 @@ int direct_items(const Plan &p, DirectItem *out);
 int build_unit_table(Plan &p);
 int launch_direct_trafo(Plan &p, const float2 *fhat, float2 *f);
 int launch_direct_adjoint(Plan &p, const float2 *y, float2 *fhat);
-// anova_plan_create; allow_direct: small bandwidths may be summed directly (a batch's
-// kernels and the tuner's candidates need the NFFT)
+// anova_plan_create; own_kernels: the plan may be summed directly or gather over records
+// beside its tiles (false for a batch's plans and the tuner's reference, which are not)
 int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct);
+                const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool own_kernels);
 // FP64 path (f64.cu): window tables, forward and adjoint transforms.
 int build_window_tables_f64(Plan &p);
 int launch_trafo_f64(Plan &p, const double2 *fhat, double2 *f);

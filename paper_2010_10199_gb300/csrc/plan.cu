@@ -241,6 +241,7 @@ DevPlan dev_view(const Plan &p) {
     v.partials = (float2 *)p.partials;
     v.spread_chunks = p.spread_K;
     v.srec = p.srec;
+    v.frec = p.cell_tc ? p.frec : p.srec;
     v.tile_cell = p.tile_cell;
     v.tile_count = p.tile_count;
     v.facc = p.facc;
@@ -345,7 +346,7 @@ const char *anova_version(void) { return "anova-gft 0.1 (sm_103a)"; }
 
 // direct_nomem: set when a plan to be summed directly found no memory for what only it needs
 static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct,
+                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool own_kernels,
                   bool *direct_nomem) {
     if (!out) return ANOVA_ERR_INVALID;
     *out = nullptr;
@@ -614,7 +615,7 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     const bool asks_nfft = (opts && (opts->sigma > 0 || opts->window_m_row > 0 || opts->window_m_col > 0)) ||
                            o.node_sort != 0 || o.cell_kernel != 0 || o.n_ctas > 0;
     long long d_groups = p.n_empty > 0 ? 1 : 0, d_units = 0;
-    if (allow_direct && !asks_nfft && p.precision == ANOVA_PREC_F32 && M > 0 && p.n_terms > 0) {
+    if (own_kernels && !asks_nfft && p.precision == ANOVA_PREC_F32 && M > 0 && p.n_terms > 0) {
         double t_direct = DIRECT_FIXED_NS, t_nfft = NFFT_FIXED_NS;
         p.direct = true;
         for (int s = 0; s < p.n_terms && p.direct; ++s) {
@@ -696,8 +697,8 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     // counts units of M records of 16 bytes.  Padding makes tiles the larger form
     // below 48 nodes per cell, up to twelve times at one node per cell: records may
     // fit where tiles do not.
-    auto keep_sorted = [&](bool tiles) {
-        long long n_rec = 0, n_tiles = 0;   // float4 records, tiles
+    auto keep_sorted = [&](bool tiles, bool beside) {   // beside: records too
+        long long n_rec = 0, n_tiles = 0, n_side = 0;   // float4 records, tiles
         std::vector<int> slot(p.n_terms, -1);
         for (int s = 0; s < p.n_terms; ++s) {
             Term &T = p.h_terms[s];
@@ -707,7 +708,8 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
                 const long long cap = tile_capacity(M, cells);
                 T.rec_off = n_rec;
                 T.tile_off = n_tiles;
-                slot[s] = s;
+                slot[s] = beside ? (int)n_side : s;
+                n_side += beside ? (T.order <= 2 ? 1 : 2) : 0;
                 n_rec += cap * tile_f4(T.order);
                 n_tiles += cap;
             } else {
@@ -721,12 +723,13 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
             n_tiles += TILE_SLACK;
         }
         size_t free_b = 0, total_b = 0;
-        const size_t need = (size_t)n_rec * sizeof(float4) + (size_t)n_tiles * sizeof(int);
+        const size_t need = (size_t)(n_rec + n_side * M) * sizeof(float4) + (size_t)n_tiles * sizeof(int);
         if (n_rec == 0 || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess || need > free_b / 2) return false;
         auto sorted_parts = [&](Arena &A) {
             A.want(&p.srec, (size_t)n_rec * sizeof(float4));
             A.want(&p.tile_cell, (size_t)n_tiles * sizeof(int));
             A.want(&p.tile_count, tiles ? sizeof(int) * p.n_terms : 0);
+            A.want(&p.frec, (size_t)n_side * M * sizeof(float4));
         };
         Arena opt;
         sorted_parts(opt);
@@ -746,22 +749,39 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
         }
         if (!ok) {
             cudaGetLastError();
-            p.srec = nullptr;
+            p.srec = p.frec = nullptr;
             p.tile_cell = p.tile_count = nullptr;
             return false;
         }
         for (int s = 0; s < p.n_terms; ++s) p.h_terms[s].sort_slot = slot[s];
         p.n_sorted = tiles ? p.n_terms : (int)(n_rec / M);
+        p.n_frec = (int)n_side;
         p.cell_tc = tiles;
         return true;
     };
     if (o.node_sort >= 0 && M > 0 && p.n_terms > 0 && !p.direct) {
         bool tiles = !f64 && o.cell_kernel == 0;
+        // Third-order terms of few nodes per cell: a tile holds one cell's nodes, and every
+        // cell transforms its planes for them, where the CUDA cores' gather takes 32 nodes of
+        // any cells.  Such plans keep records beside the tiles for the forward; the adjoint
+        // is faster over tiles from half a node per cell on.  Forward over tiles / records
+        // in us, d = 10, N = 100/24/10 (n = 20), at 0.25, 1, 2.5, 6, 10 nodes per cell:
+        // 933 / 225, 861 / 304, 1052 / 429, 945 / 800, 970 / 1242; d = 6, 64/24/10: 584 / 129,
+        // 427 / 166, 245 / 128, 222 / 189, 226 / 274; n = 12, d = 8 crosses at 9 per cell.
+        // An explicit chunk count keeps one form for both directions.
+        double nodes3 = 0.0, cells3 = 0.0;
+        for (int s = 0; s < p.n_terms; ++s) {
+            const Term &T = p.h_terms[s];
+            if (T.order != 3) continue;
+            nodes3 += (double)M;
+            cells3 += (double)T.n * T.n * T.n;
+        }
+        const bool beside = own_kernels && o.n_ctas <= 0 && p.precision == ANOVA_PREC_F32 && nodes3 < 5.0 * cells3;
         for (int s = 0; s < p.n_terms && tiles; ++s) {   // a tile's places are 32-bit
             const Term &T = p.h_terms[s];
             tiles = tile_capacity(M, T.order == 1 ? T.n : (long long)T.n * T.n * (T.order == 3 ? T.n : 1)) * TILE < (1LL << 31);
         }
-        if (!tiles || !keep_sorted(true)) keep_sorted(false);
+        if (!tiles || !(keep_sorted(true, beside) || (beside && keep_sorted(true, false)))) keep_sorted(false, false);
     }
     {   // the tables in one copy
         std::vector<unsigned char> host(table_bytes);
@@ -816,10 +836,10 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
 }
 
 int agft::plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                      const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool allow_direct) {
+                      const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool own_kernels) {
     try {
         bool direct_nomem = false;
-        int rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, allow_direct, &direct_nomem);
+        int rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, own_kernels, &direct_nomem);
         if (direct_nomem)
             rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, false, &direct_nomem);
         return rc;

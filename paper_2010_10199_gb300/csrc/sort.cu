@@ -480,18 +480,25 @@ static int sort_tiles(Plan &p) {
     return cuda_status(e);
 }
 
-int sort_nodes_by_cell(Plan &p) {
-    if (!p.srec || p.n_sorted == 0 || p.M == 0) return ANOVA_OK;
-    if (p.cell_tc) return sort_tiles(p);
+// records of every term with sort_slot >= 0, n_slots slots of M
+static int sort_records(Plan &p, float4 *srec, int n_slots) {
     int max_bins = 1;
     for (int s = 0; s < p.n_terms; ++s) {
         const Term &T = p.h_terms[s];
         if (T.sort_slot >= 0)
             max_bins = std::max(max_bins, T.order == 3 ? T.n * T.n * T.n : (T.order == 2 ? T.n * T.n : T.n));
     }
-    int *counts = nullptr;
-    cudaError_t e = plan_malloc(&counts, sizeof(int) * (size_t)p.n_sorted * max_bins);
-    if (e != cudaSuccess) return cuda_status(e);
+    int *counts = nullptr, *own = nullptr;
+    const size_t need = sizeof(int) * (size_t)n_slots * max_bins;
+    cudaError_t e = cudaSuccess;
+    // beside tiles in the partial grids, which hold nothing yet, where they fit
+    if (p.frec && need <= (size_t)p.spread_kmax * (size_t)p.grid_elems * 8) {
+        counts = (int *)p.partials;
+    } else {
+        e = plan_malloc(&own, need);
+        if (e != cudaSuccess) return cuda_status(e);
+        counts = own;
+    }
     const size_t hist_bytes = sizeof(int) * (size_t)max_bins;
     const bool f64 = p.precision == ANOVA_PREC_F64;
     if (hist_bytes > 48 * 1024)
@@ -499,7 +506,7 @@ int sort_nodes_by_cell(Plan &p) {
                                  cudaFuncAttributeMaxDynamicSharedMemorySize, (int)hist_bytes);
     const int bx = (int)std::max<long long>(1, std::min<long long>(64, (p.M + 4095) / 4096));
     const dim3 grid(bx, p.n_terms);
-    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)p.n_sorted * max_bins, p.stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(counts, 0, need, p.stream);
     if (e == cudaSuccess) {
         if (f64)
             k_cell_count64<<<grid, 256, hist_bytes, p.stream>>>(p.terms, p.wb64, p.M, counts, max_bins);
@@ -507,15 +514,23 @@ int sort_nodes_by_cell(Plan &p) {
             k_cell_count<<<grid, 256, hist_bytes, p.stream>>>(p.terms, (const float *)p.x, p.M, counts, max_bins);
         k_cell_scan<<<p.n_terms, 1024, 0, p.stream>>>(p.terms, counts, max_bins);
         if (f64)
-            k_cell_scatter64<<<grid, 256, 0, p.stream>>>(p.terms, p.wb64, p.M, counts, max_bins, p.srec);
+            k_cell_scatter64<<<grid, 256, 0, p.stream>>>(p.terms, p.wb64, p.M, counts, max_bins, srec);
         else
-            k_cell_scatter<<<grid, 256, 0, p.stream>>>(p.terms, (const float *)p.x, p.M, counts, max_bins,
-                                                       p.srec);
+            k_cell_scatter<<<grid, 256, 0, p.stream>>>(p.terms, (const float *)p.x, p.M, counts, max_bins, srec);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);
-    cudaFree(counts);
+    if (own) {
+        if (e == cudaSuccess) e = cudaStreamSynchronize(p.stream);
+        cudaFree(own);
+    }
     return cuda_status(e);
+}
+
+int sort_nodes_by_cell(Plan &p) {
+    if (!p.srec || p.n_sorted == 0 || p.M == 0) return ANOVA_OK;
+    if (!p.cell_tc) return sort_records(p, p.srec, p.n_sorted);
+    const int rc = sort_tiles(p);
+    return rc || !p.frec ? rc : sort_records(p, p.frec, p.n_frec);
 }
 
 }  // namespace agft

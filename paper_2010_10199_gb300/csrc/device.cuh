@@ -113,18 +113,8 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {
 // (16 x 8) d0 = D[g][2t], d1 = D[g][2t + 1], d2 = D[g + 8][2t],
 // d3 = D[g + 8][2t + 1].  A product a b of FP32 values is taken as
 // ah bh + ah bl + al bh with x = xh + xl split below.
-// x = hi + lo for finite x: hi keeps the sign, the exponent and the leading
-// 10 mantissa bits of x rounded half away from zero (adding half a unit of
-// the 10th bit to the bit pattern carries into the exponent where it should),
-// lo = x - hi is exact in FP32; the tensor core reads the leading 10 mantissa
-// bits of lo (error below 2^-21 |x|)
-__device__ __forceinline__ void split_tf32(float x, unsigned &hi, unsigned &lo) {
-    hi = (__float_as_uint(x) + 0x1000u) & 0xffffe000u;
-    lo = __float_as_uint(x - __uint_as_float(hi));
-}
 
-// The same split for two values at once in three packed operations (instead
-// of two integer and one FP32 operation per value): c = fl(x + 2^13 x) =
+// x = hi + lo for two finite values at once, in three packed operations: c = fl(x + 2^13 x) =
 // fl(8193 x), hi = c - 2^13 x (exact: one fma), lo = x - hi (exact: the
 // rounding error of c).  ulp(c) >= 2^13 ulp(x), so hi is a multiple of
 // 2^13 ulp(x) no larger than 2 |x| in magnitude: at most 11 significant
@@ -162,45 +152,8 @@ __device__ __forceinline__ float horner8(const float c[NCOEF], float v) {
     return s;
 }
 
-// The same polynomial at v and at -v from its even and odd parts,
-// p(+-v) = E(v^2) +- v O(v^2): 9 operations instead of two Horner chains of 7.
-// Tap 2m - 1 - j of the (even) window at v is tap j at -v.
-__device__ __forceinline__ void horner8_pm(const float c[NCOEF], float v, float &p, float &m) {
-    static_assert(NCOEF == 8, "even/odd split of a degree-7 polynomial");
-    const float v2 = v * v;
-    const float e = fmaf(fmaf(fmaf(c[6], v2, c[4]), v2, c[2]), v2, c[0]);
-    const float o = fmaf(fmaf(fmaf(c[7], v2, c[5]), v2, c[3]), v2, c[1]);
-    p = fmaf(v, o, e);
-    m = fmaf(-v, o, e);
-}
-
-// Two degree-7 polynomials at once: coefficient pairs cp[i] = (a_i, b_i),
-// arguments (va, vb); the same operations as horner8 on each half.
-__device__ __forceinline__ void horner8_x2(const f32x2 cp[NCOEF], float va, float vb, float &pa, float &pb) {
-    const f32x2 v = pk2(va, vb);
-    f32x2 s = cp[NCOEF - 1];
-#pragma unroll
-    for (int i = NCOEF - 2; i >= 0; --i) s = fma2(s, v, cp[i]);
-    upk2(s, pa, pb);
-}
-
 // Direct evaluation of the normalised Kaiser--Bessel window at distance d
-// (grid units); used where no per-tap polynomial is kept in registers.
-__device__ __forceinline__ float kb_direct(float d, int m, float b, float inv_psi0) {
-    float s2 = fmaf(-d, d, (float)(m * m));
-    if (s2 <= 0.0f) return s2 == 0.0f ? b * (1.0f / 3.14159265358979f) * inv_psi0 : 0.0f;
-    float s = sqrtf(s2);
-    float bs = b * s;
-    float v;
-    if (bs < 1e-2f) {
-        v = b * (1.0f + bs * bs * (1.0f / 6.0f));
-    } else {
-        float e = expf(bs);
-        v = 0.5f * (e - 1.0f / e) / s;
-    }
-    return v * (1.0f / 3.14159265358979f) * inv_psi0;
-}
-
+// (grid units), for the FP64 plans' tables.
 __device__ __forceinline__ double kb_direct_d(double d, int m, double b, double inv_psi0) {
     double s2 = fma(-d, d, (double)(m * m));
     if (s2 <= 0.0) return s2 == 0.0 ? b / 3.141592653589793238 * inv_psi0 : 0.0;

@@ -13,8 +13,8 @@
 // Frequencies of the innermost axis are handled in pairs +-k, k < K = N / 2, and
 // -K alone; cosine axes have the functions sqrt(2) cos(2 pi k x), k = 1 .. N / 2 - 1,
 // at the plan's halved nodes.  z_t = exp(2 pi i x_t) is kept per node and coordinate,
-// and its powers come from multiplications: up to 5 of them, or 8 from a power
-// evaluated exactly (order 1).
+// and its powers come from multiplications: at most 4 in a row (cosine axes 8), on
+// order-1 axes 7 from a power that is evaluated from the node itself.
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -67,8 +67,8 @@ static int groups_of(const Term &T) {
     return T.basis == ANOVA_BASIS_COS ? adjoint_groups<true>(T.order, axis_count(T))
                                       : adjoint_groups<false>(T.order, axis_count(T));
 }
-// terms with more than 96 partial sums per adjoint item: a kernel of their own, with
-// more registers and fewer blocks per SM
+// second-order terms with more than 64 partial sums per adjoint item: a kernel of their
+// own, with more registers and fewer blocks per SM
 static bool is_big(const Term &T) {
     const int K = axis_count(T);
     return T.order > 1 && (T.basis == ANOVA_BASIS_COS ? K > 5 : K > 3);
@@ -561,7 +561,7 @@ __device__ __forceinline__ void adjoint_order1(const DevPlan &P, const DirectTer
 // Work item (active term or -1 for the empty set, row group, node chunk, chunks; its
 // term): partial sums into part[item]; the last block of a term to finish adds them
 // over the chunks in order and writes the coefficients.  BIG: plans that have
-// a term with more than 96 sums per item.  RUNS: items of more than DA_RUN nodes.
+// a second-order term with more than 64 sums per item.  RUNS: items of more than DA_RUN nodes.
 template <bool COS, bool BIG, bool RUNS>
 __global__ void __launch_bounds__(DA_THREADS, BIG ? DIRECT_RESIDENT_BIG : DIRECT_RESIDENT)
 direct_adjoint(DevPlan P, const DirectItem *__restrict__ items, const float2 *__restrict__ y, float2 *__restrict__ fhat,

@@ -92,15 +92,15 @@ __device__ __forceinline__ void horner_pair(const float4 *c, float v0, float v1,
 
 template <int MR>
 __global__ void __launch_bounds__(GS_THREADS, 3)
-gather_sorted_f32(DevPlan single, BatchArgs B, const int4 *__restrict__ items, int item_begin, int item_end,
-                  int *counter, long long max_grid_bytes) {
+gather_sorted_f32(DevPlan single, BatchArgs B, const int4 *__restrict__ items, int item_end, int *counter,
+                  long long max_grid_bytes) {
     extern __shared__ __align__(16) unsigned char smem[];
     float2 *S = (float2 *)smem;
     float4 *coef = (float4 *)(smem + max_grid_bytes);   // [8 column taps + 8 row taps][2]
     int &s_item = *(int *)(coef + 32);
     const int tid = threadIdx.x;
     for (;;) {
-        if (tid == 0) s_item = item_begin + atomicAdd(counter, 1);
+        if (tid == 0) s_item = atomicAdd(counter, 1);
         __syncthreads();
         const int item = s_item;
         __syncthreads();
@@ -264,9 +264,9 @@ int gather_sorted_launch(cudaStream_t st, const DevPlan &v, const BatchArgs &B, 
         const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(3, (size_t)(MAX_SMEM + 1024) / (smem + 1024)));
         const int ctas = std::max(1, std::min(n_items, per_sm * sm_count));
         if (mr <= 3)
-            gather_sorted_f32<3><<<ctas, GS_THREADS, smem, st>>>(v, B, items, 0, n_items, counter, max_grid_bytes);
+            gather_sorted_f32<3><<<ctas, GS_THREADS, smem, st>>>(v, B, items, n_items, counter, max_grid_bytes);
         else
-            gather_sorted_f32<4><<<ctas, GS_THREADS, smem, st>>>(v, B, items, 0, n_items, counter, max_grid_bytes);
+            gather_sorted_f32<4><<<ctas, GS_THREADS, smem, st>>>(v, B, items, n_items, counter, max_grid_bytes);
     }
     // two rounds of four nodes per thread for the largest problem, at least one
     // round filling the chip; a batch's smaller problems leave their blocks idle

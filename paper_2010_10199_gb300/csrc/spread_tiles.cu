@@ -98,7 +98,7 @@ constexpr size_t ST_A_BYTES = NCOEF * ST_AROW * sizeof(float2);
 constexpr size_t ST_B_BYTES = (NCOEF - 1) * ST_BROW * sizeof(float);
 constexpr size_t ST_ONE_BYTES = ST_BROW * sizeof(float);
 constexpr size_t ST_WARP_BYTES = (ST_A_BYTES + ST_B_BYTES + 127) / 128 * 128;
-static_assert(ST_A_BYTES % 128 == 0 && ST_ONE_BYTES == ST_BROW * sizeof(float), "row 0 of B lies a row's pitch before row 1");
+static_assert(ST_A_BYTES % 128 == 0, "B starts on a bank's first word");
 
 template <int MR, bool ORD2>
 __device__ __forceinline__ void spread_run12(const float4 *__restrict__ rec, const int *__restrict__ cells, int nt,

@@ -146,11 +146,6 @@ __device__ __forceinline__ void mma_f16_k8_0(float (&d)[4], unsigned a0, unsigne
         : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
         : "r"(a0), "r"(a1), "r"(b0), "f"(0.f));
 }
-__device__ __forceinline__ void mma_f16_k8(float (&d)[4], unsigned a0, unsigned a1, unsigned b0) {
-    asm("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0, %1, %2, %3}, {%4, %5}, {%6}, {%0, %1, %2, %3};"
-        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-        : "r"(a0), "r"(a1), "r"(b0));
-}
 
 // power of two that takes values of magnitude at most m (bits of a non-negative
 // float) to at most 2^top; 1 for zero, infinite and NaN m

@@ -105,15 +105,22 @@ typedef struct {
     int window_m_row;   /* window half-width along the other axes (0: auto: 4 for eps below
                            5e-5, which holds every term's block within 1e-5 in FP32; else 3) */
     double sigma;       /* minimal oversampling factor n_u / N_u (0: 2.0) */
-    int n_ctas;         /* adjoint: most node chunks (partial grids) per term, <= 64 (0: auto) */
-    int node_sort;      /* adjoint: 0 = keep a copy of the nodes sorted by grid cell for every
-                           term of order <= 2 when it fits in half the free device memory
-                           (16 bytes per node and term); -1 = never */
-    int cell_kernel;    /* terms of order <= 2 with sorted nodes: 0 = the per-cell products on
-                           the tensor cores (operands split into two TF32 parts, three
-                           products, FP32 sums): the adjoint spread of FP32, FP16 and BF16
-                           plans, and the forward gather of FP32 plans without third-order
-                           terms; 1 = on the CUDA cores (FP32) */
+    int n_ctas;         /* most node chunks (the adjoint's partial grids) per term, <= 64 (0: auto) */
+    int node_sort;      /* 0 = keep a copy of the nodes sorted by grid cell for every term where
+                           it fits in half the free device memory, for the adjoint and, in FP32
+                           plans, the forward: with cell_kernel 0 tiles of 16 nodes of one cell
+                           (12 bytes per place, 16 for order 3, a cell's last tile padded), or
+                           records where those do not fit; with cell_kernel 1 and in FP64 plans
+                           records of 16 bytes per node and term (32 for order 3; FP64: orders
+                           1 and 2 only).  Third-order terms with fewer than five nodes per cell
+                           keep an FP32 plan's records beside its tiles, unless n_ctas is set.
+                           -1 = never */
+    int cell_kernel;    /* plans with sorted nodes: 0 = the per-cell products on the tensor cores
+                           (operands in two TF32 parts, order 3 two scaled FP16 parts, three
+                           products, FP32 sums): the adjoint spread of FP32, FP16 and BF16 plans
+                           and the forward gather of FP32 plans, but for those that keep records
+                           beside their tiles, whose gather runs on the CUDA cores; 1 = both on
+                           the CUDA cores (FP32) */
     int basis;          /* enum anova_basis (0: the exponential system) */
 } anova_plan_options;
 

@@ -146,7 +146,7 @@ int anova_plan_autotune(anova_plan_options *opts, int d, int64_t M, const void *
     ro.window_m_row = 4;
     ro.eps = 1e-8;
     anova_plan_t ref = nullptr;
-    int rc = plan_create(&ref, d, M, x_dev, n_terms, term_dims, bandwidth, &ro, stream, false);
+    int rc = plan_create(&ref, d, M, x_dev, n_terms, term_dims, bandwidth, &ro, stream, {false, -1});
     if (rc) return rc;
     const long long n = anova_num_coeffs(ref);
     TuneBuffers T;

@@ -45,6 +45,7 @@ struct Batch {
     bool any_empty = false;
     bool sorted_fwd = false;  // every problem has sorted nodes of one form, and accumulators
     bool cell_tc = false;     // every problem has node tiles
+    bool fwd_tc = false;      // and the forward reads them (not records beside them)
     long long max_M = 0;
     double2 *scratch = nullptr;
     // batched LSQR workspace
@@ -94,7 +95,7 @@ static int batch_trafo(Batch &b, cudaStream_t st, const float2 *fhat, float2 *f)
     if (e != cudaSuccess) return cuda_status(e);
     if (b.sorted_fwd)
         return gather_sorted_launch(st, b.views[0], b.args, b.P, fhat, f, b.args.items, b.n_items3, b.n_items,
-                                    b.counter, b.max_grid_bytes, b.max_M, b.sm_count, b.mr, b.cell_tc);
+                                    b.counter, b.max_grid_bytes, b.max_M, b.sm_count, b.mr, b.fwd_tc);
     return gather_launch(st, b.views[0], b.args, fhat, f, b.n_tiles, b.mr, b.pitch, b.max_grid_bytes, b.dmax,
                          b.sm_count, ANOVA_PREC_F32);
 }
@@ -258,13 +259,19 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
     bool accumulators = true;
     int pitch = -1;
     bool mixed_pitch = false;
+    // One launch gathers for all problems, so records beside the tiles are kept by all or by
+    // none, by the nodes per third-order cell of the whole batch.
+    Cells3 c3;
+    for (int p = 0; p < n_problems; ++p) add_cells3(c3, M[p], n_terms[p], term_dims[p], bandwidth[p], o);
+    const int records = few_nodes3(c3);
+    bool side = true;
     for (int p = 0; p < n_problems; ++p) {
         if (M[p] < 1) {
             free_batch(b);
             return ANOVA_ERR_INVALID;
         }
         anova_plan_t h = nullptr;
-        int rc = plan_create(&h, d[p], M[p], x_dev[p], n_terms[p], term_dims[p], bandwidth[p], &o, stream, false);
+        int rc = plan_create(&h, d[p], M[p], x_dev[p], n_terms[p], term_dims[p], bandwidth[p], &o, stream, {false, records});
         if (rc) {
             free_batch(b);
             return rc;
@@ -302,6 +309,7 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
         b->max_grid_elems = std::max(b->max_grid_elems, pl.grid_elems);
         b->any_empty = b->any_empty || pl.n_empty > 0;
         forms.push_back(node_form(pl));
+        side = side && pl.frec;
         accumulators = accumulators && pl.facc && pl.n_act3 == 0;
         b->max_M = std::max(b->max_M, pl.M);
         b->sm_count = pl.sm_count;
@@ -309,6 +317,7 @@ int anova_batch_create(anova_batch_t *out, int n_problems, const int *d, const i
     const int form = batch_form(forms.data(), n_problems);
     b->sorted_fwd = form != FORM_NONE && accumulators;
     b->cell_tc = form == FORM_TILES;
+    b->fwd_tc = b->cell_tc && !side;
     b->pitch = mixed_pitch || pitch < 0 ? 0 : pitch;
     // spread items: every problem's active terms split into K_p node chunks of about
     // the same size for all problems (one chunk per term each, the largest problem's

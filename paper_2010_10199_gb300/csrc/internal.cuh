@@ -366,10 +366,24 @@ int direct_items(const Plan &p, DirectItem *out);
 int build_unit_table(Plan &p);
 int launch_direct_trafo(Plan &p, const float2 *fhat, float2 *f);
 int launch_direct_adjoint(Plan &p, const float2 *y, float2 *fhat);
-// anova_plan_create; own_kernels: the plan may be summed directly or gather over records
-// beside its tiles (false for a batch's plans and the tuner's reference, which are not)
+// anova_plan_create.  direct: the plan may be summed directly (a batch's plans and the
+// tuner's reference are not); records: beside its tiles, for the forward, 1 yes, 0 no,
+// -1 by few_nodes3 of its own terms (a batch's plans: of the batch's).
+struct PlanUse {
+    bool direct;
+    int records;
+};
 int plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool own_kernels);
+                const int32_t *bandwidth, const anova_plan_options *opts, void *stream, PlanUse use);
+// Nodes and grid cells of the third-order terms of a valid or invalid term list (terms
+// that a plan refuses are left out), and whether the forward of such a node density is
+// faster over records (plan.cu).
+struct Cells3 {
+    double nodes = 0.0, cells = 0.0;
+};
+void add_cells3(Cells3 &c, int64_t M, int n_terms, const int32_t *term_dims, const int32_t *bandwidth,
+                const anova_plan_options &o);
+bool few_nodes3(const Cells3 &c);
 // FP64 path (f64.cu): window tables, forward and adjoint transforms.
 int build_window_tables_f64(Plan &p);
 int launch_trafo_f64(Plan &p, const double2 *fhat, double2 *f);

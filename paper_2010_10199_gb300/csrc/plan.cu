@@ -130,6 +130,30 @@ int row_stride(int n) {
     return s;
 }
 
+void add_cells3(Cells3 &c, int64_t M, int n_terms, const int32_t *term_dims, const int32_t *bandwidth,
+                const anova_plan_options &o) {
+    const double sigma = o.sigma > 0 ? o.sigma : 2.0;
+    if (!term_dims || !bandwidth || sigma > 8) return;
+    for (int i = 0; i < n_terms; ++i) {
+        const long long N = bandwidth[i] * (o.basis == ANOVA_BASIS_COS ? 2LL : 1LL);
+        if (term_dims[3 * i + 2] < 0 || N < 2 || N > 4096) continue;
+        const double n = fft_size((int)N, sigma);
+        c.nodes += (double)M;
+        c.cells += n * n * n;
+    }
+}
+
+// Third-order terms of few nodes per cell: a tile holds one cell's nodes, and every
+// cell transforms its planes for them, where the CUDA cores' gather takes 32 nodes of
+// any cells.  Such plans keep records beside the tiles for the forward; the adjoint
+// is faster over tiles from half a node per cell on.  Forward over tiles / records
+// in us at 0.5, 2, 4, 6, 8 nodes per cell: d = 10, N = 100/24/10 (n = 20) 684 / 201,
+// 1017 / 418, 926 / 588, 944 / 814, 951 / 1038; d = 6, 32/12/8 (n = 16) 239 / 73, 237 / 111,
+// 158 / 136, 137 / 159, 129 / 184; the lines cross at 5 (n = 12, 16) and 7 (n = 8, 20).
+// A batch of four, d = 6, 64/24/10, at 1/8, 1/4, 5/4 nodes per cell: 504 / 139, 917 / 177,
+// 600 / 225.  An explicit chunk count keeps one form for both directions.
+bool few_nodes3(const Cells3 &c) { return c.nodes < 5.0 * c.cells; }
+
 __global__ void wrap_nodes_f32(const float *in, float *out, long long total, float scale, int *bad) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
@@ -346,7 +370,7 @@ const char *anova_version(void) { return "anova-gft 0.1 (sm_103a)"; }
 
 // direct_nomem: set when a plan to be summed directly found no memory for what only it needs
 static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool own_kernels,
+                  const int32_t *bandwidth, const anova_plan_options *opts, void *stream, PlanUse use,
                   bool *direct_nomem) {
     if (!out) return ANOVA_ERR_INVALID;
     *out = nullptr;
@@ -615,7 +639,7 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     const bool asks_nfft = (opts && (opts->sigma > 0 || opts->window_m_row > 0 || opts->window_m_col > 0)) ||
                            o.node_sort != 0 || o.cell_kernel != 0 || o.n_ctas > 0;
     long long d_groups = p.n_empty > 0 ? 1 : 0, d_units = 0;
-    if (own_kernels && !asks_nfft && p.precision == ANOVA_PREC_F32 && M > 0 && p.n_terms > 0) {
+    if (use.direct && !asks_nfft && p.precision == ANOVA_PREC_F32 && M > 0 && p.n_terms > 0) {
         double t_direct = DIRECT_FIXED_NS, t_nfft = NFFT_FIXED_NS;
         p.direct = true;
         for (int s = 0; s < p.n_terms && p.direct; ++s) {
@@ -761,22 +785,13 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     };
     if (o.node_sort >= 0 && M > 0 && p.n_terms > 0 && !p.direct) {
         bool tiles = !f64 && o.cell_kernel == 0;
-        // Third-order terms of few nodes per cell: a tile holds one cell's nodes, and every
-        // cell transforms its planes for them, where the CUDA cores' gather takes 32 nodes of
-        // any cells.  Such plans keep records beside the tiles for the forward; the adjoint
-        // is faster over tiles from half a node per cell on.  Forward over tiles / records
-        // in us, d = 10, N = 100/24/10 (n = 20), at 0.25, 1, 2.5, 6, 10 nodes per cell:
-        // 933 / 225, 861 / 304, 1052 / 429, 945 / 800, 970 / 1242; d = 6, 64/24/10: 584 / 129,
-        // 427 / 166, 245 / 128, 222 / 189, 226 / 274; n = 12, d = 8 crosses at 9 per cell.
-        // An explicit chunk count keeps one form for both directions.
-        double nodes3 = 0.0, cells3 = 0.0;
-        for (int s = 0; s < p.n_terms; ++s) {
-            const Term &T = p.h_terms[s];
-            if (T.order != 3) continue;
-            nodes3 += (double)M;
-            cells3 += (double)T.n * T.n * T.n;
+        bool beside = use.records > 0;
+        if (use.records < 0) {
+            Cells3 c;
+            add_cells3(c, M, n_terms, term_dims, bandwidth, o);
+            beside = few_nodes3(c);
         }
-        const bool beside = own_kernels && o.n_ctas <= 0 && p.precision == ANOVA_PREC_F32 && nodes3 < 5.0 * cells3;
+        beside = beside && o.n_ctas <= 0 && p.precision == ANOVA_PREC_F32;
         for (int s = 0; s < p.n_terms && tiles; ++s) {   // a tile's places are 32-bit
             const Term &T = p.h_terms[s];
             tiles = tile_capacity(M, T.order == 1 ? T.n : (long long)T.n * T.n * (T.order == 3 ? T.n : 1)) * TILE < (1LL << 31);
@@ -836,12 +851,14 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
 }
 
 int agft::plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms, const int32_t *term_dims,
-                      const int32_t *bandwidth, const anova_plan_options *opts, void *stream, bool own_kernels) {
+                      const int32_t *bandwidth, const anova_plan_options *opts, void *stream, PlanUse use) {
     try {
         bool direct_nomem = false;
-        int rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, own_kernels, &direct_nomem);
-        if (direct_nomem)
-            rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, false, &direct_nomem);
+        int rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, use, &direct_nomem);
+        if (direct_nomem) {
+            use.direct = false;
+            rc = create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, use, &direct_nomem);
+        }
         return rc;
     } catch (const std::bad_alloc &) {
         return ANOVA_ERR_NOMEM;
@@ -855,7 +872,7 @@ extern "C" {
 int anova_plan_create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_terms,
                       const int32_t *term_dims, const int32_t *bandwidth, const anova_plan_options *opts,
                       void *stream) {
-    return plan_create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, true);
+    return plan_create(out, d, M, x_dev, n_terms, term_dims, bandwidth, opts, stream, {true, -1});
 }
 
 int anova_debug_fail_allocation(int k) {

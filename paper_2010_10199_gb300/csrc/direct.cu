@@ -663,17 +663,29 @@ direct_adjoint(DevPlan P, const DirectItem *__restrict__ items, const float2 *__
         }
         const float *src = first + (long long)group * C * DA_MAX_ACC + at;
         float v[4] = {0.f, 0.f, 0.f, 0.f};
-        for (int c = 0; c < C; ++c) {
-            const float *s = src + (long long)c * DA_MAX_ACC;
-            if (COS && T.order > 1) {
-                v[0] += __ldcg(s);
-                v[2] += __ldcg(s + 1);
-            } else {
-                const float4 w = __ldcg((const float4 *)s);
-                v[0] += w.x;
-                v[1] += w.y;
-                v[2] += w.z;
-                v[3] += w.w;
+        auto add = [&](float (&r)[4], int c0, int c1) {
+            for (int c = c0; c < c1; ++c) {
+                const float *s = src + (long long)c * DA_MAX_ACC;
+                if (COS && T.order > 1) {
+                    r[0] += __ldcg(s);
+                    r[2] += __ldcg(s + 1);
+                } else {
+                    const float4 w = __ldcg((const float4 *)s);
+                    r[0] += w.x;
+                    r[1] += w.y;
+                    r[2] += w.z;
+                    r[3] += w.w;
+                }
+            }
+        };
+        if (C <= DIRECT_MAX_CHUNKS) {
+            add(v, 0, C);
+        } else {   // in runs, which keeps the FP32 chains as short as those of fewer chunks
+            for (int c = 0; c < C; c += DIRECT_MAX_CHUNKS) {
+                float r[4] = {0.f, 0.f, 0.f, 0.f};
+                add(r, c, min(C, c + DIRECT_MAX_CHUNKS));
+#pragma unroll
+                for (int i = 0; i < 4; ++i) v[i] += r[i];
             }
         }
         float2 g;
@@ -687,12 +699,20 @@ direct_adjoint(DevPlan P, const DirectItem *__restrict__ items, const float2 *__
 
 // --------------------------------------------------------------- host ----
 
-// Whether the kernels take a term, and both ways' times per transform (the mean of the
-// two directions) in nanoseconds.  The constants are least-squares fits to both ways
-// measured at 66 shapes: d = 5 .. 20, |u| <= 1, 2, 3, both systems, 500 to 300 000
-// nodes; the faster way is taken at each of them but one, where they differ by 2 %.
-// Direct: order 1 per frequency, the others per multiply-add.  NFFT: per tile of 16
-// nodes (half a tile more per cell for the ragged last one) and per cell.
+// Whether the kernels take a term.
+bool direct_term(const Term &T) {
+    const int K = axis_count(T);
+    if (T.order == 1) return K <= 128;
+    if (T.basis == ANOVA_BASIS_COS) return T.order == 2 ? K <= 9 : K <= 4;
+    return T.order == 2 ? K <= 5 : K <= 3;
+}
+
+// Whether a plan of such terms is faster summed directly: both ways' times per transform
+// (the mean of the two directions) in nanoseconds.  The constants of a term are
+// least-squares fits to both ways measured at 66 shapes: d = 5 .. 20, |u| <= 1, 2, 3, both
+// systems, 500 to 300 000 nodes; the faster way is taken at each of them but one, where
+// they differ by 2 %.  Direct: order 1 per frequency, the others per multiply-add.  NFFT:
+// per tile of 16 nodes (half a tile more per cell for the ragged last one) and per cell.
 //   d  |u|    N            M        direct us         NFFT us    (forward / adjoint)
 //   9   3  26/6/4      10 000       23 / 15           93 / 107
 //   6   2   16/8       300 000      62 / 62           78 / 101
@@ -700,26 +720,50 @@ direct_adjoint(DevPlan P, const DirectItem *__restrict__ items, const float2 *__
 //   8   2   32/10      300 000     136 / 143         117 / 142
 //  20   1     64       100 000      60 / 43           44 / 40
 //  12   2  82/10 cos   100 000     136 / 195         102 / 122
-bool direct_term(const Term &T) {
-    const int K = axis_count(T);
-    if (T.order == 1) return K <= 128;
-    if (T.basis == ANOVA_BASIS_COS) return T.order == 2 ? K <= 9 : K <= 4;
-    return T.order == 2 ? K <= 5 : K <= 3;
-}
-double direct_term_ns(const Term &T, long long M) {
-    const int K = axis_count(T);
-    if (T.order == 1) return 7.5e-4 * K * (double)M;
-    const bool c = T.basis == ANOVA_BASIS_COS;
-    const int n = c ? axis_coefs<true>(K) : axis_coefs<false>(K);
-    const double ops = (T.order == 2 ? n : n * n) * (c ? 2.0 * K + 2.0 : 4.0 * K + 8.0);
-    return (1.84e-3 + 4.4e-5 * ops) * (double)M;
-}
-double nfft_term_ns(const Term &T, long long M) {
-    double cells = T.n;
-    for (int j = 1; j < T.order; ++j) cells *= T.n;
-    cells = std::min(cells, (double)M);
-    const double tiles = M / 16.0 + 0.5 * cells;
-    return T.order == 3 ? 0.46 * tiles + 1.54 * cells : 0.131 * tiles + 0.041 * cells;
+// Beyond these, from 20 shapes at 100 000 to 10 million nodes (d = 1 .. 30):
+// * every node costs both ways the same whatever the terms (blocks of few units, the
+//   accumulators' pass): what plans of one or two coordinates take at a million nodes;
+// * beyond 40 MB of powers and values, a third of L2, the adjoint's items wait for their
+//   reads, those of the larger second-order terms, with two blocks to an SM, longer than
+//   the others, with four;
+// * the tiles' accumulators, 16 bytes a node, outgrow L2 and are added to from memory by
+//   all terms but a few;
+// * up to three third-order terms, of at most 64 items each, leave SMs idle.
+//   1   1     16     1 000 000      49 / 39           66 / 56
+//   4   2   16/8     1 000 000     121 / 96          128 / 124
+//   4   2   16/8     3 000 000     415 / 494         317 / 307
+//   6   2   16/8     1 000 000     202 / 338         199 / 220
+//   6   2   16/4     3 000 000     490 / 492         520 / 564
+//   6   2   16/8    10 000 000    2128 / 3334       4732 / 1846
+// The slower way is taken at three of these 97 measurements, by 9, 10 and 16 %.
+bool direct_faster(const Term *terms, int n_terms, int d, long long M) {
+    double t_direct = DIRECT_FIXED_NS + 0.023 * M, t_nfft = NFFT_FIXED_NS + 0.020 * M, read = 0.0;
+    int n3 = 0;
+    bool big = false;
+    for (int s = 0; s < n_terms; ++s) {
+        const Term &T = terms[s];
+        const int K = axis_count(T);
+        if (T.order == 1) {
+            t_direct += 7.5e-4 * K * (double)M;
+        } else {
+            const bool c = T.basis == ANOVA_BASIS_COS;
+            const int n = c ? axis_coefs<true>(K) : axis_coefs<false>(K);
+            const double ops = (T.order == 2 ? n : n * n) * (c ? 2.0 * K + 2.0 : 4.0 * K + 8.0);
+            t_direct += (1.84e-3 + 4.4e-5 * ops) * (double)M;
+        }
+        read += (double)groups_of(T) * (T.order == 1 ? 20 : 8 + 8 * T.order);
+        big = big || is_big(T);
+        n3 += T.order == 3;
+        double cells = T.n;
+        for (int j = 1; j < T.order; ++j) cells *= T.n;
+        cells = std::min(cells, (double)M);
+        const double tiles = M / 16.0 + 0.5 * cells;
+        t_nfft += T.order == 3 ? 0.46 * tiles + 1.54 * cells : 0.131 * tiles + 0.041 * cells;
+    }
+    if (8.0 * (d + 1) * M > 40e6) t_direct += 0.5 * read * (big ? 3.0e-4 : 1.05e-4) * M;   // one of two directions
+    if (16.0 * M > 80e6) t_nfft += 0.007 * std::max(0, n_terms - 3) * (double)M;
+    if (n3 > 0) t_nfft += 0.46 * M / 16.0 * std::max(0.0, 3.4 - n3);
+    return t_direct < t_nfft;
 }
 
 int direct_groups(const Term &T) { return groups_of(T); }
@@ -753,7 +797,7 @@ int direct_items(const Plan &p, DirectItem *out) {
     const long long R = (long long)p.sm_count * (p.direct_big ? DIRECT_RESIDENT_BIG : DIRECT_RESIDENT);
     int C = 1;
     double best = 0.0;
-    for (int c = 1; c <= direct_max_chunks(p.M); ++c) {
+    for (int c = 1; c <= direct_max_chunks(p.M, p.direct_kt == 0); ++c) {
         if (c > 1 && groups * c > DIRECT_MAX_BLOCKS) break;
         const double t = (double)((groups * c + R - 1) / R) * ((double)p.M / c + 2000.0);
         if (c == 1 || t < 0.98 * best) {

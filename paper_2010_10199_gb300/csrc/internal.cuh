@@ -352,12 +352,18 @@ constexpr int DIRECT_RESIDENT = 4, DIRECT_RESIDENT_BIG = 2;       // its blocks 
 constexpr int DIRECT_MAX_SPLITS = 16;         // forward: sets of terms per node block
 constexpr double DIRECT_FIXED_NS = 8400.0, NFFT_FIXED_NS = 33000.0;   // launches and latencies of a transform
 bool direct_term(const Term &T);
-double direct_term_ns(const Term &T, long long M);
-double nfft_term_ns(const Term &T, long long M);
+bool direct_faster(const Term *terms, int n_terms, int d, long long M);
 size_t direct_smem(int d, int kt, int npl, bool cosine);
 int direct_npl(int d, int kt, long long M, bool cosine);
 int direct_splits(long long n_units, long long M, int npl, int sm_count);
-inline long long direct_max_chunks(long long M) { return std::min<long long>(DIRECT_MAX_CHUNKS, std::max<long long>(1, M / 256)); }
+// Node chunks of an adjoint item, at most: of 256 nodes up to 64 chunks.  Plans of order-1
+// terms alone, whose items cost the same, then take chunks of 16384 nodes, one FP32 chain
+// per thread: one coordinate's plan had 128 blocks at any size (d = 1, N = 16, M = 1e7
+// 755 -> 183 us, 2e6 72 -> 53).
+inline long long direct_max_chunks(long long M, bool order1) {
+    const long long c = std::min<long long>(DIRECT_MAX_CHUNKS, std::max<long long>(1, M / 256));
+    return order1 ? std::max(c, (M + 16383) / 16384) : c;
+}
 int direct_unit_list(const Plan &p, DirectTerm *out);
 bool direct_big(const Term &T);
 int direct_axis(const Term &T);

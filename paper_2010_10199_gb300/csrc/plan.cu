@@ -640,19 +640,17 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
                            o.node_sort != 0 || o.cell_kernel != 0 || o.n_ctas > 0;
     long long d_groups = p.n_empty > 0 ? 1 : 0, d_units = 0;
     if (use.direct && !asks_nfft && p.precision == ANOVA_PREC_F32 && M > 0 && p.n_terms > 0) {
-        double t_direct = DIRECT_FIXED_NS, t_nfft = NFFT_FIXED_NS;
         p.direct = true;
         for (int s = 0; s < p.n_terms && p.direct; ++s) {
             const Term &T = p.h_terms[s];
             p.direct = direct_term(T);
-            t_direct += direct_term_ns(T, M);
-            t_nfft += nfft_term_ns(T, M);
             d_groups += direct_groups(T);
             d_units += T.order == 1 ? direct_groups(T) : 1;
             p.direct_big = p.direct_big || direct_big(T);
             if (T.order > 1) p.direct_kt = std::max(p.direct_kt, direct_axis(T));
         }
-        p.direct = p.direct && t_direct < t_nfft && direct_smem(d, p.direct_kt, 1, cosine) <= DIRECT_MAX_SMEM;
+        p.direct = p.direct && direct_faster(p.h_terms, p.n_terms, d, M) &&
+                   direct_smem(d, p.direct_kt, 1, cosine) <= DIRECT_MAX_SMEM;
     }
     if (p.direct) {
         p.direct_npl = direct_npl(d, p.direct_kt, M, cosine);
@@ -660,7 +658,7 @@ static int create(anova_plan_t *out, int d, int64_t M, const void *x_dev, int n_
     }
     const size_t f_blocks = p.direct ? (size_t)((M + 32 * p.direct_npl - 1) / (32 * p.direct_npl)) : 0;
     if (p.direct) kmax = 1;
-    const size_t n_ditems = p.direct ? (size_t)std::max(d_groups, std::min<long long>(DIRECT_MAX_BLOCKS, d_groups * direct_max_chunks(M)))
+    const size_t n_ditems = p.direct ? (size_t)std::max(d_groups, std::min<long long>(DIRECT_MAX_BLOCKS, d_groups * direct_max_chunks(M, p.direct_kt == 0)))
                                      : 0;
     const size_t n_items = p.direct ? 1 : nt1 * kmax;
     p.spread_kmax = kmax;

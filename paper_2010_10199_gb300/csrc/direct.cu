@@ -190,14 +190,16 @@ __device__ __forceinline__ void term_rows(const DirectTerm &T, const float4 *st,
 // Units that a warp adds in one FP32 chain (up to 9 rows each) before their sum goes to
 // its total, kept in shared memory (in registers it spilled): the error of a chain grows
 // with the root of its length, and one over the 58 units of a warp at d = 30, N = 16/8
-// left 2.8e-7 at M = 3e4 where the NFFT has 2.1e-7.
+// left 2.8e-7 at M = 3e4 where the NFFT has 2.1e-7.  Plans whose warps have no more units
+// than that run kernels without totals (CHAINS false): d = 3, N = 16/8/4, M = 2e5 24.5 ->
+// 23.6 us, d = 1, N = 16, M = 1e7 599 -> 533.
 constexpr int DT_CHAIN = 8;
 
 // A CTA takes 32 NPL nodes and every gridDim.y-th set of work units (active term,
 // frequency group of order 1), its warps one unit each in turn; the warps' sums are
 // added in order, and so are the CTAs' of a node block by the last one to finish
 // (bitwise reproducible).
-template <int NPL, bool COS>
+template <int NPL, bool COS, bool CHAINS>
 __global__ void __launch_bounds__(DT_THREADS, NPL == 4 ? 2 : 3)
 direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f, int KT,
              const DirectTerm *__restrict__ units, int n_units, float2 *fpart, int *count) {
@@ -226,15 +228,16 @@ direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f,
     float2 acc[NPL];
     float2 *sum = red + warp * NB + lane;   // this lane's sums of the chains before
 #pragma unroll
-    for (int u = 0; u < NPL; ++u) sum[32 * u] = acc[u] = make_float2(0.f, 0.f);
+    for (int u = 0; u < NPL; ++u) acc[u] = make_float2(0.f, 0.f);
+    int chain_end = first + DT_CHAIN * step;
     auto end_chain = [&]() {
+        const bool later = CHAINS && chain_end != first + DT_CHAIN * step;   // not the first chain
 #pragma unroll
         for (int u = 0; u < NPL; ++u) {
-            sum[32 * u] = make_float2(sum[32 * u].x + acc[u].x, sum[32 * u].y + acc[u].y);
+            sum[32 * u] = later ? make_float2(sum[32 * u].x + acc[u].x, sum[32 * u].y + acc[u].y) : acc[u];
             acc[u] = make_float2(0.f, 0.f);
         }
     };
-    int chain_end = first + DT_CHAIN * step;
     // A unit's coefficients are loaded while the unit before it is summed, and its
     // record before that: a lane holds up to three pairs (c_k, c_-k) of a term of
     // order >= 2 (cosine: three coefficients), an order-1 group all its coefficients.
@@ -264,7 +267,7 @@ direct_trafo(DevPlan P, const float2 *__restrict__ fhat, float2 *__restrict__ f,
     if (first + step < n_units) after = units[first + step];
     if (first < n_units) prefetch(next);
     for (int s = first; s < n_units; s += step) {
-        if (s == chain_end) {
+        if (CHAINS && s == chain_end) {
             end_chain();
             chain_end += DT_CHAIN * step;
         }
@@ -867,11 +870,14 @@ template <int NPL, bool COS>
 static void launch_trafo(Plan &p, const DevPlan &v, const float2 *fhat, float2 *f) {
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
-        cudaFuncSetAttribute(direct_trafo<NPL, COS>, cudaFuncAttributeMaxDynamicSharedMemorySize, DIRECT_MAX_SMEM);
+        cudaFuncSetAttribute(direct_trafo<NPL, COS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, DIRECT_MAX_SMEM);
+        cudaFuncSetAttribute(direct_trafo<NPL, COS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, DIRECT_MAX_SMEM);
     });
     const int NB = 32 * NPL;
     const dim3 grid((unsigned)((p.M + NB - 1) / NB), p.direct_split);
-    direct_trafo<NPL, COS><<<grid, DT_THREADS, direct_smem(p.d, p.direct_kt, NPL, COS), p.stream>>>(
+    const bool chains = p.n_direct_units > DT_CHAIN * (DT_THREADS / 32) * p.direct_split;
+    auto k = chains ? direct_trafo<NPL, COS, true> : direct_trafo<NPL, COS, false>;
+    k<<<grid, DT_THREADS, direct_smem(p.d, p.direct_kt, NPL, COS), p.stream>>>(
         v, fhat, f, p.direct_kt, p.direct_units, p.n_direct_units, p.direct_fpart, p.direct_fcount);
 }
 

@@ -430,20 +430,21 @@ static int sort_tiles(Plan &p) {
             place_bins = std::max(place_bins, T.order == 2 ? T.n * T.n : T.n);
     }
     // slices of at least 16384 nodes (a block also moves a histogram)
-    const int S = (int)std::max<long long>(1, std::min<long long>(SORT_MAX_SLICES, p.M / 16384));
+    int S = (int)std::max<long long>(1, std::min<long long>(SORT_MAX_SLICES, p.M / 16384));
     const size_t n_bins = (size_t)p.n_terms * max_bins;
     // (first tile, nodes) per cell, then the slices' histograms: in the partial
     // grids, which hold nothing yet, where they fit
     int2 *info = nullptr, *own = nullptr;
-    const size_t need = sizeof(int2) * n_bins + sizeof(int) * n_bins * S;
+    const size_t room = (size_t)p.spread_kmax * (size_t)p.grid_elems * (p.precision == ANOVA_PREC_F32 ? 8 : 4);
     cudaError_t e = cudaSuccess;
-    if (need <= (size_t)p.spread_kmax * (size_t)p.grid_elems * (p.precision == ANOVA_PREC_F32 ? 8 : 4)) {
-        info = (int2 *)p.partials;
-    } else {
-        e = plan_malloc(&own, need);
-        if (e != cudaSuccess) return cuda_status(e);
-        info = own;
+    auto need = [&]() { return sizeof(int2) * n_bins + sizeof(int) * n_bins * S; };
+    if (need() > room && (e = plan_malloc(&own, need())) != cudaSuccess && S > 1) {
+        cudaGetLastError();   // one slice takes up to six times less
+        S = 1;
+        e = need() > room ? plan_malloc(&own, need()) : cudaSuccess;
     }
+    if (e != cudaSuccess) return cuda_status(e);
+    info = own ? own : (int2 *)p.partials;
     const size_t bytes = sizeof(int) * (size_t)max_bins;
     static std::atomic<unsigned long long> attr_seen{0};
     once_per_device(attr_seen, [] {
@@ -455,7 +456,7 @@ static int sort_tiles(Plan &p) {
     const size_t cells = 2 * sizeof(int) * (size_t)place_bins;
     const int cap = (int)std::min<long long>({(long long)PLACE_MAX, (long long)((TILES_MAX_SMEM - cells) / 2), (p.M + S - 1) / S});
     const size_t place_bytes = cells + sizeof(unsigned short) * (size_t)cap;
-    if (e == cudaSuccess) {
+    {
         const dim3 grid(S, p.n_terms);
         const float *x = (const float *)p.x;
         int *hist = (int *)(info + n_bins);

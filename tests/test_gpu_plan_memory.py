@@ -71,3 +71,35 @@ def test_tiles_without_memory_become_records(gft):
     # the tiles, their cells and their counts; without accumulators the tiles stay
     assert forms.count(gft.FORM_RECORDS) == 3 and gft.FORM_OWN_ORDER not in forms
     assert forms.count(None) >= 20 and forms[-1] == gft.FORM_TILES
+
+
+def test_sorting_without_memory_takes_one_slice(gft):
+    """Many order-1 terms beside a third-order one: the sort's histograms (40000 nodes: two
+    slices of 8000 cells per term) do not fit in the partial grids, and one slice's have to do
+    where theirs cannot be allocated."""
+    import torch
+    M, terms = 40000, [(t,) for t in range(40)] + [(0, 1, 2)]
+    bw = [16] * 40 + [10]
+    x = inputs.uniform_points(5, 40, M)
+    xd, xo = to_dev(x, torch.float32), f32_nodes(x)
+    fhat, y = inputs.complex_normal(5, 2, 40 * 15 + 9 ** 3), inputs.complex_normal(5, 4, M)
+    f_ref, g_ref = ndft.trafo(xo, terms, bw, fhat), ndft.adjoint(xo, terms, bw, y)
+    built = []
+    try:
+        for k in range(1, 48):
+            gft.anova_debug_fail_allocation(k)
+            try:
+                P = gft.Plan(xd, terms, bw, n_ctas=1)
+            except gft.AnovaError as e:
+                assert e.status == -3, f"k={k}"
+                built.append(False)
+                continue
+            finally:
+                gft.anova_debug_fail_allocation(0)
+            built.append(True)
+            assert rel_l2(host(P.trafo(cplx_dev(fhat))), f_ref) <= TOL and rel_l2(host(P.adjoint(cplx_dev(y))), g_ref) <= TOL
+            P.close()
+    finally:
+        gft.anova_debug_fail_allocation(0)
+    # every allocation after those that a plan cannot do without has something in its place
+    assert built.count(False) >= 15 and all(built[built.index(True):])

@@ -530,8 +530,16 @@ static int sort_records(Plan &p, float4 *srec, int n_slots) {
 int sort_nodes_by_cell(Plan &p) {
     if (!p.srec || p.n_sorted == 0 || p.M == 0) return ANOVA_OK;
     if (!p.cell_tc) return sort_records(p, p.srec, p.n_sorted);
-    const int rc = sort_tiles(p);
-    return rc || !p.frec ? rc : sort_records(p, p.frec, p.n_frec);
+    int rc = sort_tiles(p);
+    if (rc || !p.frec) return rc;
+    rc = sort_records(p, p.frec, p.n_frec);
+    if (rc == ANOVA_ERR_NOMEM) {   // the forward runs over the tiles then
+        cudaGetLastError();
+        p.frec = nullptr;
+        p.n_frec = 0;
+        rc = ANOVA_OK;
+    }
+    return rc;
 }
 
 }  // namespace agft

@@ -73,23 +73,24 @@ def test_tiles_without_memory_become_records(gft):
     assert forms.count(None) >= 20 and forms[-1] == gft.FORM_TILES
 
 
-def test_sorting_without_memory_takes_one_slice(gft):
-    """Many order-1 terms beside a third-order one: the sort's histograms (40000 nodes: two
-    slices of 8000 cells per term) do not fit in the partial grids, and one slice's have to do
-    where theirs cannot be allocated."""
+@pytest.mark.parametrize("M,kw", [(40000, dict(n_ctas=1)), (39000, {})], ids=["tiles", "records_beside"])
+def test_sorting_without_memory(gft, M, kw):
+    """Many order-1 terms beside a third-order one: the sorts' histograms (8000 cells per term,
+    two slices into tiles) do not fit in the partial grids.  Where they cannot be allocated one
+    slice's have to do, and the forward runs over the tiles instead of records beside them."""
     import torch
-    M, terms = 40000, [(t,) for t in range(40)] + [(0, 1, 2)]
-    bw = [16] * 40 + [10]
-    x = inputs.uniform_points(5, 40, M)
+    terms = [(t,) for t in range(100)] + [(0, 1, 2)]
+    bw = [16] * 100 + [10]
+    x = inputs.uniform_points(5, 100, M)
     xd, xo = to_dev(x, torch.float32), f32_nodes(x)
-    fhat, y = inputs.complex_normal(5, 2, 40 * 15 + 9 ** 3), inputs.complex_normal(5, 4, M)
+    fhat, y = inputs.complex_normal(5, 2, 100 * 15 + 9 ** 3), inputs.complex_normal(5, 4, M)
     f_ref, g_ref = ndft.trafo(xo, terms, bw, fhat), ndft.adjoint(xo, terms, bw, y)
     built = []
     try:
         for k in range(1, 48):
             gft.anova_debug_fail_allocation(k)
             try:
-                P = gft.Plan(xd, terms, bw, n_ctas=1)
+                P = gft.Plan(xd, terms, bw, **kw)
             except gft.AnovaError as e:
                 assert e.status == -3, f"k={k}"
                 built.append(False)

@@ -132,8 +132,10 @@ __device__ __forceinline__ void gather_run12(const float4 *__restrict__ rec, con
         }
         float h[4];
         window_to_basis(g0, g1, __ldg(pbc + t * NCOEF + g), __ldg(pbc + (t + 4) * NCOEF + g), r0, r1, h);
-        split_tf32_x2(pk2(h[0] * sc, h[1] * sc), bh[0], bl[0], bh[1], bl[1]);
-        split_tf32_x2(pk2(h[2] * sc, h[3] * sc), bh[2], bl[2], bh[3], bl[3]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h[k] = uncut(h[k] * sc, ord2 ? 3.f : 2.f);
+        split_tf32_x2(pk2(h[0], h[1]), bh[0], bl[0], bh[1], bl[1]);
+        split_tf32_x2(pk2(h[2], h[3]), bh[2], bl[2], bh[3], bl[3]);
     };
     struct Tile {
         float4 q;   // (vr_g, vr_g+8, vc_g, vc_g+8)
@@ -236,8 +238,10 @@ __device__ __forceinline__ void gather_run3(const float4 *__restrict__ rec, cons
         float h[4];
         window_to_basis(g0, g1, __ldg(&wc->pb[t][g]), __ldg(&wc->pb[t + 4][g]), r0, r1, h);
         uint4 r;
-        split_f16(h[0] * gscale, h[1] * gscale, r.x, r.y);
-        split_f16(h[2] * gscale, h[3] * gscale, r.z, r.w);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) h[k] = uncut(h[k] * gscale, 3.f);
+        split_f16(h[0], h[1], r.x, r.y);
+        split_f16(h[2], h[3], r.z, r.w);
         return r;
     };
     int cur = -1;   // cell whose planes are held

@@ -103,6 +103,17 @@ __device__ __forceinline__ void mma3_tf32_0(float (&d)[4], const unsigned (&ah)[
     mma_tf32(d, ah, bh0, bh1);
 }
 
+// The tensor core cuts its sums off at 24 bits where FP32 rounds them.  A stage of the
+// split products leaves its value short by 2^-24 of it on average: half a unit of the last
+// place, 0.72 x 2^-24 of a value with an evenly spread mantissa, and what smaller addends
+// lose where they are aligned to it.  The gather's stages (two window products, the basis
+// sum; order 1 has one window product) so left f short by 3 and 1.9 x 2^-24 (measured
+// against FP64 plans on the same window, N = 4 .. 64), the larger part of its error beside
+// the CUDA cores'.  The window values take it back in between, once per cell: error of f
+// against 64-bit sums at order 2, N = 32 2.47e-7 -> 1.65e-7 (CUDA cores 1.48), orders 1 to 3,
+// N = 36/32/4 2.63 -> 1.95 (1.79); d = 20, M = 1e6 1.660 -> 1.662 ms, 0.7 % at three nodes per cell.
+__device__ __forceinline__ float uncut(float h, float stages) { return fmaf(h, stages * 0x1p-24f, h); }
+
 // ---- FP16 tensor-core products of scaled operands ----
 //
 // x = h + l with h the nearest FP16 value and l the remainder rounded to FP16: for |x|
